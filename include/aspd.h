@@ -247,8 +247,8 @@ int aspd_plan_create(const aspd_shape_t* shape, const aspd_request_t* req, const
  * device block is parked with an event recorded on every stream the plan was used on, and a later
  * aspd_plan_create reuses a parked block of fitting size after making its own stream wait for
  * those events (so a decode loop that makes a plan per step neither allocates nor synchronises in
- * steady state).  Up to 8 blocks and 2 GiB in total are kept per process; what does not fit is
- * freed at once (cudaFree, which waits for the device).
+ * steady state).  Up to 8 blocks and 2 GiB in total are kept per process; the ones parked longest
+ * ago are freed to make room (cudaFree, which waits for the device).
  */
 int aspd_plan_destroy(aspd_plan_t* plan);
 /*
