@@ -94,7 +94,7 @@ typedef struct {
 typedef struct {
   int32_t n_q_heads, n_kv_heads;
   int32_t head_dim;  /* 64 or 128 */
-  int32_t page_size; /* tokens per page: 16 (8, 32 also accepted by the generic kernel) */
+  int32_t page_size; /* tokens per page: 8, 16 or 32 */
   int32_t dtype;     /* ASPD_DTYPE_* : element type of q, out, k_new, v_new and the pools */
   float rope_theta;
   float sm_scale;    /* Eq. 1's 1/sqrt(d_k), as a parameter */

@@ -1213,11 +1213,13 @@ static int launch_tc(const aspd_plan* p, const void* q, const void* k_new, const
 }
 
 int launch_attn_mma(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool, void* out, cudaStream_t s) {
+  if (p->dec) return launch_attn_dec(p, q, nullptr, nullptr, k_pool, v_pool, out, s);
   return launch_tc(p, q, nullptr, nullptr, k_pool, v_pool, out, s);
 }
 
 int launch_attn_mma_step(const aspd_plan* p, const void* q, const void* k_new, const void* v_new, void* k_pool, void* v_pool,
                          void* out, cudaStream_t s) {
+  if (p->dec) return launch_attn_dec(p, q, k_new, v_new, k_pool, v_pool, out, s);
   return launch_tc(p, q, k_new, v_new, k_pool, v_pool, out, s);
 }
 

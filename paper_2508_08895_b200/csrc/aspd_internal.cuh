@@ -112,6 +112,8 @@ struct aspd_plan {
   int shared_mask = 0;             // parallel step under the ablation's visible mask
   int wide = 0;                    // dealt plan of the tensor-core kernel: row blocks of up to kMaxRowsWide rows
   int m64 = 0;                     // stream-K plan of the tensor-core kernel whose MMAs take M = 64 (row blocks are at most 64 rows)
+  int dec = 0;                     // tensor-core plan of a shape that aspd_attn_dec.cu serves (head_dim 64, pages of 8 or 32)
+  int max_rows = 0;                // largest number of query rows of an item
   int stagger_start = 0;           // few tiles per CTA: order the requests of a CTA's first tiles (see the producers)
   int single_launch = 0;           // stream-K plan of the tensor-core kernel whose last-arriving CTAs merge the records themselves
   int64_t n_pool_pages = 0;
@@ -172,6 +174,9 @@ int launch_attn_generic(const aspd_plan* p, const void* q, const void* k_pool, c
 // kernel itself when the plan has one item per (token, KV head) (ignored otherwise)
 int launch_attn_mma(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool, void* out,
                     cudaStream_t s);
+// the same for plans with p->dec; k_new / v_new non-null: the step's new rows are written first
+int launch_attn_dec(const aspd_plan* p, const void* q, const void* k_new, const void* v_new, const void* k_pool, const void* v_pool,
+                    void* out, cudaStream_t s);
 inline bool attn_mma_direct(const aspd_plan* p) { return p->kernel == ASPD_KERNEL_MMA && p->dealt; }   // one item per (token, KV head)
 inline bool attn_mma_writes_output(const aspd_plan* p) { return attn_mma_direct(p) || (p->kernel == ASPD_KERNEL_MMA && p->single_launch); }
 int launch_combine(const aspd_plan* p, void* out, cudaStream_t s);

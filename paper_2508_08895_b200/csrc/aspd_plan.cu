@@ -363,7 +363,8 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   if (tune.mma_m != 0 && tune.mma_m != 64 && tune.mma_m != 96 && tune.mma_m != 128) return ASPD_ERR_INVALID_ARG;
   if (tune.combine != ASPD_COMBINE_AUTO && tune.combine != ASPD_COMBINE_KERNEL && tune.combine != ASPD_COMBINE_FUSED) return ASPD_ERR_INVALID_ARG;
   const bool shared_mask = tune.mask == ASPD_MASK_SHARED && mode == ASPD_MODE_BRANCH;
-  const bool mma_ok = shape->dtype == ASPD_DTYPE_BF16 && d == 128 && ps == 16;
+  const bool mma_ok = shape->dtype == ASPD_DTYPE_BF16;
+  const bool wide_ok = mma_ok && d == 128 && ps == 16;                 // aspd_attn_tc.cu; the other bf16 shapes: aspd_attn_dec.cu
   int kernel = tune.kernel;
   if (kernel == ASPD_KERNEL_AUTO) kernel = mma_ok ? ASPD_KERNEL_MMA : ASPD_KERNEL_GENERIC;
   if (kernel == ASPD_KERNEL_MMA && !mma_ok) return ASPD_ERR_UNSUPPORTED;
@@ -374,6 +375,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   p->shape = *shape; p->mode = mode; p->n_req = n_req; p->n_new = n_new; p->kernel = kernel;
   p->stable_cache = tune.stable_cache ? 1 : 0;
   p->shared_mask = (tune.mask == ASPD_MASK_SHARED && mode == ASPD_MODE_BRANCH) ? 1 : 0;
+  p->dec = kernel == ASPD_KERNEL_MMA && !wide_ok;
   p->host_only = tune.host_only; p->n_pool_pages = n_pool_pages; p->device_base = nullptr; p->device_bytes = 0;
   memset(&p->dev, 0, sizeof(p->dev));
   p->tune = tune;
@@ -525,11 +527,13 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     }
   };
   build_streams(max_tok);
+  const int tile_pages = 128 / ps;
   auto ctas_for = [&](long pages) {
     const int want = tune.n_ctas > 0 ? tune.n_ctas : p->sm_count;
     // do not cut finer than one 128-key tile per CTA (measured on a 2.5 k-token step: 80 CTAs with a
     // full tile each take 10.6 us per layer, 148 CTAs with half a tile 11.9: fewer records to combine)
-    return (int)std::max(1L, std::min((long)want, (pages + 7) / 8));
+    const int least = kernel == ASPD_KERNEL_MMA ? tile_pages : 8;
+    return (int)std::max(1L, std::min((long)want, (pages + least - 1) / least));
   };
   // With many more streams than CTAs (a step with many query tokens per branch: masked prefill,
   // teacher forcing) nothing is cut: every stream is one item, and the streams are dealt to the
@@ -542,7 +546,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
                       (long)streams.size() >= 4L * ctas_for(total_pages) && (tune.n_ctas > 0 || ctas_for(total_pages) >= p->sm_count);
   p->wide = 0;
   if (deal_streams) {
-    p->wide = (kernel == ASPD_KERNEL_MMA && kMaxRowsWide / G > max_tok) ? 1 : 0;
+    p->wide = (kernel == ASPD_KERNEL_MMA && wide_ok && kMaxRowsWide / G > max_tok) ? 1 : 0;
     // A step in which some request has more query tokens than one 128-row tile holds takes row blocks
     // of two tiles (the two-tile variant of the kernel: both tiles are scored against every K/V tile
     // the CTA fetches, one softmax group per tile), unless the caller asked for single tiles.
@@ -555,6 +559,8 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     build_visit(tok_per_block);
     build_streams(tok_per_block);
   }
+  p->max_rows = 0;
+  for (const int2& rb : row_blocks) p->max_rows = std::max(p->max_rows, rb.y * G);
   const int n_ctas = ctas_for(total_pages);
   const int chunk_pages = tune.chunk_tokens > 0 ? tune.chunk_tokens / ps : (1 << 28);
   p->chunk_tokens = tune.chunk_tokens; p->n_ctas = n_ctas;
@@ -585,7 +591,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     // Every CTA gets the same cost, cost = pages + kItemCost per item it starts: an item boundary
     // (new query tile, ragged last tile, epilogue) costs about as much as streaming a dozen pages,
     // so CTAs that end up with several short items get fewer pages.
-    const double kItemCost = 12.0;
+    const double kItemCost = 192.0 / ps;
     // a page costs a little more the more query rows are scored against it (best measured balance:
     // 0.35 % per row), so streams of requests with many branches weigh more
     const double kRowCost = 0.0035;
@@ -611,10 +617,10 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
         if (room < 1.0 && acc > 0.0 && cta + 1 < n_ctas) { next_cta(); continue; }
         long take = std::min<long>(st.n_pages - at, chunk_pages);
         if (cta + 1 < n_ctas) take = std::min<long>(take, std::max<long>(1, (long)(room + 0.5)));
-        // a cut inside a stream goes on a tile boundary (8 pages) where the item is long enough: the item's
+        // a cut inside a stream goes on a tile boundary (128 keys) where the item is long enough: the item's
         // last tile is then a full one (measured on the serving mix: 0.4 % on the step)
-        if (take < st.n_pages - at && tune.chunk_tokens == 0 && ps == 16 && take >= 12)
-          take = std::min<long>((take + 4) / 8 * 8, st.n_pages - at);
+        if (take < st.n_pages - at && tune.chunk_tokens == 0 && take >= tile_pages + tile_pages / 2)
+          take = std::min<long>((take + tile_pages / 2) / tile_pages * tile_pages, st.n_pages - at);
         DeviceItem it;
         it.q_tok0 = st.tok0; it.n_q_tok = st.n_tok; it.kv_head = st.head; it.page0 = st.page0 + at;
         it.n_pages = (int)take; it.key0 = at * ps; it.part_slot = slot++; it.request = st.request;
@@ -656,14 +662,14 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   // 1: both MMAs with M = 64; 2: only P.V (the default: at most 64 of P.V's 128 rows are ever read, a quarter
   // less tensor work lifts the power-capped clock and the softmax layout, which M = 64 scores would slow
   // down, stays as it is); 0: both with M = 128
-  p->m64 = (kernel == ASPD_KERNEL_MMA && !deal_streams) ? (tune.mma_m == 64 ? 1 : tune.mma_m == 128 ? 0 : 2) : 0;
+  p->m64 = (kernel == ASPD_KERNEL_MMA && !deal_streams && !p->dec) ? (tune.mma_m == 64 ? 1 : tune.mma_m == 128 ? 0 : 2) : 0;
   p->stagger_start = (!deal_streams && total_pages <= 6L * 8 * n_ctas) ? 1 : 0;       // at most six 128-key tiles per CTA
   // Merging inside the attention kernel is an option, not the default.  Measured on every workload of
   // the benchmark, the CTA that stores a pair's last record is a CTA at the very end of its own work,
   // so its fence, count and merge (1.5 us + one memory round trip per 16 rows of the pairs it ended
   // up with; all rows of a stream cut into dozens of parts land on one CTA) lengthen the kernel by
   // more than the combine launch costs, whose blocks are resident and waiting when the pass ends.
-  p->single_launch = (kernel == ASPD_KERNEL_MMA && !deal_streams && tune.combine == ASPD_COMBINE_FUSED) ? 1 : 0;
+  p->single_launch = (kernel == ASPD_KERNEL_MMA && !deal_streams && !p->dec && tune.combine == ASPD_COMBINE_FUSED) ? 1 : 0;
   for (size_t i = 0; i < n_parts.size(); ++i) part_base[i + 1] = part_base[i] + n_parts[i];
   p->n_items = (int)p->items.size();
   p->n_partials = part_base[n_parts.size()];
@@ -812,7 +818,7 @@ int aspd_plan_update(aspd_plan_t* p, const aspd_request_t* req, const aspd_branc
   if (rc) return rc;
   const aspd::PlanLayout& L = p->layout;
   if (t->n_new != p->n_new || t->n_ctas != p->n_ctas || t->kernel != p->kernel || t->wide != p->wide || t->dealt != p->dealt ||
-      t->fuse_append != p->fuse_append || t->shared_mask != p->shared_mask || t->single_launch != p->single_launch || t->m64 != p->m64 || t->kernel != ASPD_KERNEL_MMA ||
+      t->fuse_append != p->fuse_append || t->shared_mask != p->shared_mask || t->single_launch != p->single_launch || t->m64 != p->m64 || (p->dec && t->max_rows != p->max_rows) || t->kernel != ASPD_KERNEL_MMA ||
       t->row_blocks.size() != L.n_row_blocks || t->part_base.size() != L.n_part_base ||
       (t->algorithmic_bytes >= (128LL << 20)) != (p->algorithmic_bytes >= (128LL << 20))) {   // the combine's launch attribute
     delete t;
