@@ -23,7 +23,7 @@ template <> __device__ inline __nv_bfloat16 from_f32<__nv_bfloat16>(float x) { r
 constexpr int kAppendThreads = 128;
 template <typename T>
 __global__ void __launch_bounds__(kAppendThreads)
-append_kernel(const T* __restrict__ k_new, const T* __restrict__ v_new, const int32_t* __restrict__ pos,
+append_kernel(const T* __restrict__ k_new, const T* __restrict__ v_new, const int32_t* __restrict__ pos, const float2* __restrict__ cs_table,
               const int32_t* __restrict__ tok_page, const int32_t* __restrict__ tok_row,
               const double* __restrict__ inv_freq, T* __restrict__ k_pool, T* __restrict__ v_pool,
               int n_new, int n_kv_heads, int head_dim, int page_size, PlanDevice pd) {
@@ -33,25 +33,31 @@ append_kernel(const T* __restrict__ k_new, const T* __restrict__ v_new, const in
   const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const long t = gid / (chunks * n_kv_heads);
   const int h = (int)(gid / chunks % n_kv_heads), c = (int)(gid % chunks);
-  double f[VEC];                                   // plan data: may be read before the dependency wait
-#pragma unroll
-  for (int j = 0; j < VEC; ++j) f[j] = inv_freq[c * VEC + j];
+  const int page = t < n_new ? tok_page[t] : 0, row = t < n_new ? tok_row[t] : 0;   // plan data: may be read before the dependency wait
   pdl_wait();
-  if (t >= n_new || !bounds_ok(pd, tok_page[t], tok_row[t], page_size)) return;
-  // angle reduced to [-pi, pi] in fp64, then fp32 sincos: the error stays near 1e-7 rad
-  // however large the position is
+  if (t >= n_new || !bounds_ok(pd, page, row, page_size)) return;
   float sn[VEC], cs[VEC];
-  const double p = (double)pos[t];
+  if (cs_table != nullptr) {                       // the plan's own positions: their sines and cosines are there already
+    const float4* w = reinterpret_cast<const float4*>(cs_table + t * half + c * VEC);
 #pragma unroll
-  for (int j = 0; j < VEC; ++j) {
-    double a = p * f[j];
-    a -= rint(a * 0.15915494309189535) * 6.283185307179586;
-    sincosf((float)a, &sn[j], &cs[j]);
+    for (int j = 0; j < VEC; j += 2) {
+      const float4 x = w[j / 2];
+      cs[j] = x.x; sn[j] = x.y; cs[j + 1] = x.z; sn[j + 1] = x.w;
+    }
+  } else {
+    // angle reduced to [-pi, pi] in fp64, then fp32 sincos: the error stays near 1e-7 rad
+    // however large the position is
+    const double p = (double)pos[t];
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) {
+      double a = p * inv_freq[c * VEC + j];
+      a -= rint(a * 0.15915494309189535) * 6.283185307179586;
+      sincosf((float)a, &sn[j], &cs[j]);
+    }
   }
   const uint32_t rb = head_dim * sizeof(T);
   const size_t tb = tile_bytes(page_size, head_dim, sizeof(T));
-  const size_t tile0 = (size_t)tok_page[t] * n_kv_heads * tb;
-  const int row = tok_row[t];
+  const size_t tile0 = (size_t)page * n_kv_heads * tb;
   const uint32_t o0 = tile_offset(row, c * 16, rb), o1 = tile_offset(row, half * sizeof(T) + c * 16, rb);
   {
     const size_t src = ((size_t)t * n_kv_heads + h) * head_dim;
@@ -377,11 +383,12 @@ int launch_append(const aspd_plan* p, const void* k_new, const void* v_new, cons
   const aspd_shape_t& sh = p->shape;
   const int chunks = sh.head_dim / 2 / (16 / esize_of(sh.dtype));
   const dim3 grid((unsigned)(((long)p->n_new * sh.n_kv_heads * chunks + kAppendThreads - 1) / kAppendThreads)), block(kAppendThreads);
+  const float2* cs = pos == p->dev.tok_pos ? p->dev.q_cs : nullptr;
   if (sh.dtype == ASPD_DTYPE_BF16)
     return status_of(launch_pdl(kPdlAppend, append_kernel<__nv_bfloat16>, grid, block, 0, s, (const __nv_bfloat16*)k_new,
-                                (const __nv_bfloat16*)v_new, pos, p->dev.tok_page, p->dev.tok_row, p->dev.inv_freq,
+                                (const __nv_bfloat16*)v_new, pos, cs, p->dev.tok_page, p->dev.tok_row, p->dev.inv_freq,
                                 (__nv_bfloat16*)k_pool, (__nv_bfloat16*)v_pool, p->n_new, sh.n_kv_heads, sh.head_dim, sh.page_size, p->dev));
-  return status_of(launch_pdl(kPdlAppend, append_kernel<float>, grid, block, 0, s, (const float*)k_new, (const float*)v_new, pos,
+  return status_of(launch_pdl(kPdlAppend, append_kernel<float>, grid, block, 0, s, (const float*)k_new, (const float*)v_new, pos, cs,
                               p->dev.tok_page, p->dev.tok_row, p->dev.inv_freq, (float*)k_pool, (float*)v_pool, p->n_new,
                               sh.n_kv_heads, sh.head_dim, sh.page_size, p->dev));
 }
