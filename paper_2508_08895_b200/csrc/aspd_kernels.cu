@@ -258,94 +258,193 @@ rerotate_ranges_kernel(const PoolList pools, const int32_t* __restrict__ page_ta
 }
 
 // ------------------------------------------------------------------- generic attention
-// One block per work item, one warp per query row at a time.  Lane j scores key j of each
-// group of 32 keys (a full dot product against the rotated, pre-scaled query held in shared
-// memory); the weighted V sum is taken with each lane owning D/32 output elements.
+// CUDA-core split-K pass for every dtype, head_dim and page size (fp32 steps, and KERNEL_GENERIC plans).
+// A CTA walks its items 32 keys at a time: the pages of the next 32 keys are on their way to shared memory
+// (cp.async, the cache's swizzled tile image as it lies) while these are scored.  A warp owns RPW query rows from
+// the score to the record -- lane j scores key j against all of them (the key's 16-byte chunk is read once, the
+// queries are broadcast), then each lane owns D / 32 output elements -- so that inside a chunk nothing
+// crosses warps.  Bound by latency on the steps it serves: 3 branches over 256 tokens (fp32, 4 heads of 64) are
+// 10 CTAs of 32 keys, 7.4 us a step (append, this, combine) in a graph; 5 CTAs of 64 keys 10.2; the kernel before, a
+// block of four warps to 128 keys, each warp walking one row's keys through memory at a time, 153.7.
+constexpr int kGenThreads = 256, kGenWarps = kGenThreads / 32, kGenKeys = 32;
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool there) {   // 16 zero bytes if not there
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(there ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 template <typename T, int D>
-__global__ void __launch_bounds__(128) attn_generic_kernel(PlanDevice pd, const T* __restrict__ q,
-                                                           const T* __restrict__ k_pool, const T* __restrict__ v_pool,
-                                                           int n_q_heads, int n_kv_heads, int page_size, float scale_log2) {
-  constexpr int EPL = D / 32;                 // output elements per lane
-  constexpr int EPC = 16 / (int)sizeof(T);    // elements per 16-byte chunk
-  __shared__ float q_s[4][D];
-  pdl_launch_dependents();
-  pdl_wait();
-  const DeviceItem it = pd.items[blockIdx.x];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int G = n_q_heads / n_kv_heads, n_rows = it.n_q_tok * G, n_keys = it.n_pages * page_size;
+struct GenSmem {
+  T k[2][kGenKeys * D], v[2][kGenKeys * D];      // two chunks of 32 keys, tile images
+  float q[kMaxRowsPerItem * D];                  // rotated, scaled queries
+  float p[kGenWarps][kMaxRowsPerItem / kGenWarps][kGenKeys];
+  int4 vis[kMaxRowsPerItem];                     // per token of the item
+};
+
+// The 16-byte piece of this lane's D / 32 elements of row `tok` of a tile image, as floats
+template <typename T, int D>
+__device__ __forceinline__ void lane_elems(const T* tile, int tok, int lane, float (&x)[D / 32]) {
+  const char* at = reinterpret_cast<const char*>(tile) + tile_offset(tok, lane * (D / 32) * (int)sizeof(T), D * sizeof(T));
+  T e[D / 32];
+  if constexpr (sizeof(e) == 16) *reinterpret_cast<uint4*>(e) = *reinterpret_cast<const uint4*>(at);
+  else if constexpr (sizeof(e) == 8) *reinterpret_cast<uint2*>(e) = *reinterpret_cast<const uint2*>(at);
+  else *reinterpret_cast<uint32_t*>(e) = *reinterpret_cast<const uint32_t*>(at);
+#pragma unroll
+  for (int i = 0; i < D / 32; ++i) x[i] = to_f32(e[i]);
+}
+
+template <typename T, int D, int RPW>
+__device__ __forceinline__ void generic_item(const PlanDevice& pd, const DeviceItem& it, GenSmem<T, D>& sm, const T* __restrict__ q,
+                                             const T* __restrict__ k_pool, const T* __restrict__ v_pool, int n_q_heads, int n_kv_heads,
+                                             int page_size, float scale_log2) {
+  constexpr int EPL = D / 32, EPC = 16 / (int)sizeof(T), RB = D * (int)sizeof(T);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int G = n_q_heads / n_kv_heads, n_rows = it.n_q_tok * G, ppc = kGenKeys / page_size;   // pages of a chunk (4, 2, 1)
+  const int n_chunks = (it.n_pages + ppc - 1) / ppc, page_shift = 31 - __clz(page_size);
   const size_t tb = tile_bytes(page_size, D, sizeof(T));
-  for (int r = warp; r < n_rows; r += 4) {
-    const int tl = r / G, g = r % G, tok = it.q_tok0 + tl, hq = it.kv_head * G + g;
-    // rotate the query at its own position (table built on the host in fp64), fold in the scale
-    const T* qrow = q + ((size_t)tok * n_q_heads + hq) * D;
-    for (int i = lane; i < D / 2; i += 32) {
-      const float2 cs = pd.q_cs[(size_t)tok * (D / 2) + i];
-      const float x0 = to_f32(qrow[i]), x1 = to_f32(qrow[i + D / 2]);
-      q_s[warp][i] = (x0 * cs.x - x1 * cs.y) * scale_log2;
-      q_s[warp][i + D / 2] = (x1 * cs.x + x0 * cs.y) * scale_log2;
+  // lane l < ppc: entry of page l of a chunk (no valid rows behind the item's pages)
+  auto entry_of = [&](int chunk) {
+    int2 e = make_int2(0, 0);
+    if (lane < ppc && chunk * ppc + lane < it.n_pages) {
+      e = pd.visit[it.page0 + chunk * ppc + lane];
+      if (!bounds_ok(pd, e.x, 0, page_size)) e = make_int2(0, 0);     // checking builds: flagged, keys left out
     }
-    __syncwarp();
-    // stream keys [0, pe) and [lo, hi) are visible; under the shared mask (w > 0) also keys of other
-    // branches whose offset in their branch (page index in the upper bits of the page entry) is below w
-    const int4 vis = pd.tok_vis[tok];
-    float m = -INFINITY, l = 0.f, acc[EPL];
+    return e;
+  };
+  auto request = [&](int2 entry, int st) {
+    const uint32_t kd = (uint32_t)__cvta_generic_to_shared(sm.k[st]), vd = (uint32_t)__cvta_generic_to_shared(sm.v[st]);
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
-    for (int base = 0; base < n_keys; base += 32) {
-      const int j = base + lane;
-      bool seen = false;
-      float s = -INFINITY;
-      if (j < n_keys) {
-        const int2 pg = pd.visit[it.page0 + j / page_size];
-        const int row = j % page_size, kg = it.key0 + j;
-        seen = row < (pg.y & 255) && (kg < vis.x || (kg >= vis.y && kg < vis.z) || (pg.y >> 13) * page_size + row < vis.w);
-        if (seen && !bounds_ok(pd, pg.x, row, page_size)) seen = false;      // checking builds: flagged, key left out
-        if (seen) {
-          const char* tile = reinterpret_cast<const char*>(k_pool) + ((size_t)pg.x * n_kv_heads + it.kv_head) * tb;
-          float dot = 0.f;
-#pragma unroll 4
-          for (int c = 0; c < D / EPC; ++c) {
-            const uint4 raw = *reinterpret_cast<const uint4*>(tile + tile_offset(row, c * 16, D * sizeof(T)));
-            const T* e8 = reinterpret_cast<const T*>(&raw);
+    for (int u = 0; u < kGenKeys * RB / 16 / kGenThreads; ++u) {
+      const uint32_t b = (tid + u * kGenThreads) * 16u;
+      const int pg = (int)(b / (uint32_t)tb);
+      const int id = __shfl_sync(0xffffffffu, entry.x, pg), there = __shfl_sync(0xffffffffu, entry.y, pg) & 255;
+      const size_t src = ((size_t)id * n_kv_heads + it.kv_head) * tb + (b - pg * (uint32_t)tb);
+      cp_async16(kd + b, reinterpret_cast<const char*>(k_pool) + src, there != 0);
+      cp_async16(vd + b, reinterpret_cast<const char*>(v_pool) + src, there != 0);
+    }
+    cp_async_commit();
+  };
+  int2 cur = entry_of(0), nxt = entry_of(1);
+  request(cur, 0);
+  // the queries, rotated at their own positions (table of the plan), scale folded in
+  for (int e = tid; e < it.n_q_tok; e += kGenThreads) sm.vis[e] = pd.tok_vis[it.q_tok0 + e];
+  for (int e = tid; e < n_rows * (D / 2); e += kGenThreads) {
+    const int r = e / (D / 2), i = e % (D / 2), tok = it.q_tok0 + r / G;
+    const T* qrow = q + ((size_t)tok * n_q_heads + it.kv_head * G + r % G) * D;
+    const float2 cs = pd.q_cs[(size_t)tok * (D / 2) + i];
+    const float x0 = to_f32(qrow[i]), x1 = to_f32(qrow[i + D / 2]);
+    sm.q[r * D + i] = (x0 * cs.x - x1 * cs.y) * scale_log2;
+    sm.q[r * D + i + D / 2] = (x1 * cs.x + x0 * cs.y) * scale_log2;
+  }
+  const int row0 = warp * RPW;                    // rows row0 ... row0 + RPW - 1, those below n_rows
+  float m[RPW], l[RPW], acc[RPW][EPL];
 #pragma unroll
-            for (int e = 0; e < EPC; ++e) dot = fmaf(q_s[warp][c * EPC + e], to_f32(e8[e]), dot);
+  for (int i = 0; i < RPW; ++i) {
+    m[i] = -INFINITY; l[i] = 0.f;
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) acc[i][e] = 0.f;
+  }
+  for (int ch = 0; ch < n_chunks; ++ch) {
+    const int st = ch & 1;
+    const int2 after = entry_of(ch + 2);
+    if (ch + 1 < n_chunks) { request(nxt, st ^ 1); cp_async_wait<1>(); }
+    else cp_async_wait<0>();
+    __syncthreads();
+    if (row0 < n_rows) {
+      float s[RPW][2];                            // even and odd chunks of the dot products apart
+#pragma unroll
+      for (int i = 0; i < RPW; ++i) s[i][0] = s[i][1] = 0.f;
+#pragma unroll (RPW < 8 ? 4 : 2)
+      for (int c = 0; c < RB / 16; ++c) {
+        const uint4 raw = *reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(sm.k[st]) + tile_offset(lane, c * 16, RB));
+        const T* e8 = reinterpret_cast<const T*>(&raw);
+        float kx[EPC];
+#pragma unroll
+        for (int e = 0; e < EPC; ++e) kx[e] = to_f32(e8[e]);
+#pragma unroll
+        for (int i = 0; i < RPW; ++i) {
+          const float4* qr = reinterpret_cast<const float4*>(sm.q + min(row0 + i, n_rows - 1) * D + c * EPC);
+#pragma unroll
+          for (int e = 0; e < EPC / 4; ++e) {
+            const float4 w = qr[e];
+            float& d = s[i][(EPC == 4 ? c : e) & 1];
+            d = fmaf(w.x, kx[4 * e], d); d = fmaf(w.y, kx[4 * e + 1], d); d = fmaf(w.z, kx[4 * e + 2], d); d = fmaf(w.w, kx[4 * e + 3], d);
           }
-          s = dot;
         }
       }
-      if (!__any_sync(0xffffffffu, seen)) continue;
-      float mx = s;
+      // stream keys [0, pe) and [lo, hi) are visible; under the shared mask (w > 0) also keys of other
+      // branches whose offset in their branch (page index in the upper bits of the page entry) is below w
+      const int ye = __shfl_sync(0xffffffffu, cur.y, lane >> page_shift), row = lane & (page_size - 1), kg = it.key0 + ch * kGenKeys + lane;
+      const bool valid = row < (ye & 255);
 #pragma unroll
-      for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const float m_new = fmaxf(m, mx);           // finite: at least one key of the group is seen
-      const float p = seen ? exp2f(s - m_new) : 0.f;
-      const float alpha = exp2f(m - m_new);       // m = -inf before the first seen key: alpha = 0
-      float ps = p;
+      for (int i = 0; i < RPW; ++i) {
+        const int4 vis = sm.vis[min(row0 + i, n_rows - 1) / G];
+        const bool seen = valid && (kg < vis.x || (kg >= vis.y && kg < vis.z) || (ye >> 13) * page_size + row < vis.w);
+        const float x = seen ? s[i][0] + s[i][1] : -INFINITY;
+        float mx = x;
 #pragma unroll
-      for (int o = 16; o; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
-      l = l * alpha + ps;
+        for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const float mn = fmaxf(m[i], mx), base = mn == -INFINITY ? 0.f : mn;      // no key seen so far: every weight is 0
+        const float pw = exp2f(x - base), alpha = exp2f(m[i] - base);
+        float ps = pw;
 #pragma unroll
-      for (int e = 0; e < EPL; ++e) acc[e] *= alpha;
-      const int cnt = min(32, n_keys - base);
-      for (int jj = 0; jj < cnt; ++jj) {
-        const float pj = __shfl_sync(0xffffffffu, p, jj);
-        if (pj == 0.f) continue;                  // masked (or negligible) key: its V row is not touched
-        const int key = base + jj;
-        const int2 pg = pd.visit[it.page0 + key / page_size];
-        const char* tile = reinterpret_cast<const char*>(v_pool) + ((size_t)pg.x * n_kv_heads + it.kv_head) * tb;
+        for (int o = 16; o; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
+        l[i] = l[i] * alpha + ps;
+        m[i] = mn;
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) {
-          const T v = *reinterpret_cast<const T*>(tile + tile_offset(key % page_size, (lane * EPL + e) * sizeof(T), D * sizeof(T)));
-          acc[e] = fmaf(pj, to_f32(v), acc[e]);
+        for (int e = 0; e < EPL; ++e) acc[i][e] *= alpha;
+        sm.p[warp][i][lane] = pw;
+      }
+      __syncwarp();
+#pragma unroll (RPW < 8 ? 2 : 1)
+      for (int j = 0; j < kGenKeys; j += 4) {
+        float v[4][EPL];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) lane_elems<T, D>(sm.v[st], j + k, lane, v[k]);
+#pragma unroll
+        for (int i = 0; i < RPW; ++i) {
+          const float4 w = *reinterpret_cast<const float4*>(&sm.p[warp][i][j]);
+#pragma unroll
+          for (int e = 0; e < EPL; ++e)
+            acc[i][e] = fmaf(w.w, v[3][e], fmaf(w.z, v[2][e], fmaf(w.y, v[1][e], fmaf(w.x, v[0][e], acc[i][e]))));
         }
       }
-      m = m_new;
     }
-    const size_t rec = (size_t)(pd.part_base[tok * n_kv_heads + it.kv_head] + it.part_slot) * G + g;
-    if (lane == 0) pd.ws_ml[rec] = make_float2(m, l);
+    __syncthreads();                              // the chunk's buffers (and, after the last one, the queries) are free
+    cur = nxt;
+    nxt = after;
+  }
 #pragma unroll
-    for (int e = 0; e < EPL; ++e) pd.ws_o[rec * D + lane * EPL + e] = acc[e];
-    __syncwarp();
+  for (int i = 0; i < RPW; ++i) {
+    const int r = row0 + i;
+    if (r >= n_rows) break;
+    const size_t rec = (size_t)(pd.part_base[(it.q_tok0 + r / G) * n_kv_heads + it.kv_head] + it.part_slot) * G + r % G;
+    if (lane == 0) pd.ws_ml[rec] = make_float2(m[i], l[i]);
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) pd.ws_o[rec * D + lane * EPL + e] = acc[i][e];
+  }
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kGenThreads, 2) attn_generic_kernel(PlanDevice pd, const T* __restrict__ q, const T* __restrict__ k_pool,
+                                                                      const T* __restrict__ v_pool, int n_q_heads, int n_kv_heads,
+                                                                      int page_size, float scale_log2) {
+  extern __shared__ __align__(1024) uint8_t gen_smem[];
+  GenSmem<T, D>& sm = *reinterpret_cast<GenSmem<T, D>*>(gen_smem);
+  pdl_launch_dependents();
+  const int4 head = pd.cta_head[blockIdx.x];
+  DeviceItem it = {};
+  if (head.x < head.y) it = pd.items[head.x];
+  pdl_wait();
+  for (int idx = head.x; idx < head.y; ++idx) {
+    if (idx > head.x) it = pd.items[idx];
+    const int rows = it.n_q_tok * (n_q_heads / n_kv_heads);
+#define ASPD_GEN_ITEM(RPW) generic_item<T, D, RPW>(pd, it, sm, q, k_pool, v_pool, n_q_heads, n_kv_heads, page_size, scale_log2)
+    if (rows <= 8) ASPD_GEN_ITEM(1);
+    else if (rows <= 16) ASPD_GEN_ITEM(2);
+    else if (rows <= 32) ASPD_GEN_ITEM(4);
+    else ASPD_GEN_ITEM(8);
+#undef ASPD_GEN_ITEM
   }
 }
 
@@ -393,19 +492,27 @@ int launch_append(const aspd_plan* p, const void* k_new, const void* v_new, cons
                               sh.n_kv_heads, sh.head_dim, sh.page_size, p->dev));
 }
 
-int launch_attn_generic(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool, cudaStream_t s) {
+template <typename T, int D>
+static int launch_generic(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool, cudaStream_t s) {
+  static bool configured[64] = {};                 // the attribute belongs to the (function, device) pair
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return ASPD_ERR_CUDA;
+  if (dev < 0 || dev >= 64 || !configured[dev]) {
+    if (cudaFuncSetAttribute(attn_generic_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GenSmem<T, D>)) != cudaSuccess)
+      return ASPD_ERR_CUDA;
+    if (dev >= 0 && dev < 64) configured[dev] = true;
+  }
   const aspd_shape_t& sh = p->shape;
+  return status_of(launch_pdl(kPdlAttn, attn_generic_kernel<T, D>, dim3(p->n_ctas), dim3(kGenThreads), sizeof(GenSmem<T, D>), s, p->dev,
+                              (const T*)q, (const T*)k_pool, (const T*)v_pool, sh.n_q_heads, sh.n_kv_heads, sh.page_size, sh.sm_scale * kLog2e));
+}
+
+int launch_attn_generic(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool, cudaStream_t s) {
   if (p->n_items == 0) return ASPD_OK;
-  const float sc = sh.sm_scale * kLog2e;
-  const dim3 grid(p->n_items), block(128);
-#define ASPD_GEN(T, D)                                                                                         \
-  return status_of(launch_pdl(kPdlAttn, attn_generic_kernel<T, D>, grid, block, 0, s, p->dev, (const T*)q, (const T*)k_pool, \
-                              (const T*)v_pool, sh.n_q_heads, sh.n_kv_heads, sh.page_size, sc))
-  if (sh.dtype == ASPD_DTYPE_BF16 && sh.head_dim == 128) ASPD_GEN(__nv_bfloat16, 128);
-  else if (sh.dtype == ASPD_DTYPE_BF16) ASPD_GEN(__nv_bfloat16, 64);
-  else if (sh.head_dim == 128) ASPD_GEN(float, 128);
-  else ASPD_GEN(float, 64);
-#undef ASPD_GEN
+  const aspd_shape_t& sh = p->shape;
+  if (sh.dtype == ASPD_DTYPE_BF16) return sh.head_dim == 128 ? launch_generic<__nv_bfloat16, 128>(p, q, k_pool, v_pool, s)
+                                                             : launch_generic<__nv_bfloat16, 64>(p, q, k_pool, v_pool, s);
+  return sh.head_dim == 128 ? launch_generic<float, 128>(p, q, k_pool, v_pool, s) : launch_generic<float, 64>(p, q, k_pool, v_pool, s);
 }
 
 int launch_qcs(const aspd_plan* p, cudaStream_t s) {

@@ -527,13 +527,14 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     }
   };
   build_streams(max_tok);
-  const int tile_pages = 128 / ps;
+  const bool cores = kernel == ASPD_KERNEL_GENERIC;
+  const int tile_pages = std::max(1, (cores ? 32 : 128) / ps);
   auto ctas_for = [&](long pages) {
-    const int want = tune.n_ctas > 0 ? tune.n_ctas : p->sm_count;
     // do not cut finer than one 128-key tile per CTA (measured on a 2.5 k-token step: 80 CTAs with a
-    // full tile each take 10.6 us per layer, 148 CTAs with half a tile 11.9: fewer records to combine)
-    const int least = kernel == ASPD_KERNEL_MMA ? tile_pages : 8;
-    return (int)std::max(1L, std::min((long)want, (pages + least - 1) / least));
+    // full tile each take 10.6 us per layer, 148 CTAs with half a tile 11.9: fewer records to combine);
+    // the CUDA-core kernel takes 32 keys at a time and two of its CTAs fit an SM
+    const int want = tune.n_ctas > 0 ? tune.n_ctas : p->sm_count * (cores ? 2 : 1);
+    return (int)std::max(1L, std::min((long)want, (pages + tile_pages - 1) / tile_pages));
   };
   // With many more streams than CTAs (a step with many query tokens per branch: masked prefill,
   // teacher forcing) nothing is cut: every stream is one item, and the streams are dealt to the
@@ -591,7 +592,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     // Every CTA gets the same cost, cost = pages + kItemCost per item it starts: an item boundary
     // (new query tile, ragged last tile, epilogue) costs about as much as streaming a dozen pages,
     // so CTAs that end up with several short items get fewer pages.
-    const double kItemCost = 192.0 / ps;
+    const double kItemCost = (cores ? 64.0 : 192.0) / ps;
     // a page costs a little more the more query rows are scored against it (best measured balance:
     // 0.35 % per row), so streams of requests with many branches weigh more
     const double kRowCost = 0.0035;
@@ -617,8 +618,8 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
         if (room < 1.0 && acc > 0.0 && cta + 1 < n_ctas) { next_cta(); continue; }
         long take = std::min<long>(st.n_pages - at, chunk_pages);
         if (cta + 1 < n_ctas) take = std::min<long>(take, std::max<long>(1, (long)(room + 0.5)));
-        // a cut inside a stream goes on a tile boundary (128 keys) where the item is long enough: the item's
-        // last tile is then a full one (measured on the serving mix: 0.4 % on the step)
+        // a cut inside a stream goes on a tile boundary (128 keys; CUDA cores: 32) where the item is long
+        // enough: the item's last tile is then a full one (measured on the serving mix: 0.4 % on the step)
         if (take < st.n_pages - at && tune.chunk_tokens == 0 && take >= tile_pages + tile_pages / 2)
           take = std::min<long>((take + tile_pages / 2) / tile_pages * tile_pages, st.n_pages - at);
         DeviceItem it;
