@@ -68,6 +68,7 @@ EXPORTS = ("aspd_strerror", "aspd_pool_bytes", "aspd_count_new_tokens", "aspd_po
            "aspd_branch_step", "aspd_serial_step", "aspd_step_host", "aspd_step_host_async", "aspd_attn_static", "aspd_static_status", "aspd_k_rerotate", "aspd_k_rerotate_ranges", "aspd_k_rerotate_ranges_layers", "aspd_debug_read_token", "aspd_debug_bounded_wait", "aspd_debug_profile", "aspd_debug_pool_limit")
 
 _lib = None
+_raw_stream = _get_device = None
 
 
 def library_path() -> str:
@@ -143,15 +144,30 @@ def _ptr(x) -> Optional[int]:
         return None
     if isinstance(x, np.ndarray):
         assert x.flags.c_contiguous
-        return x.ctypes.data
+        try:                                    # a third of the time that x.ctypes takes
+            return ctypes.addressof(ctypes.c_char.from_buffer(x))
+        except (TypeError, ValueError):         # read-only or empty
+            return x.ctypes.data
     return x.data_ptr()
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else None
+        return _current_stream()
     return getattr(stream, "cuda_stream", stream)
+
+
+def _current_stream() -> Optional[int]:
+    """Handle of torch's current stream.  (``torch.cuda.current_stream()`` makes a Stream object first: 4.4 us
+    a call, a quarter of a step's host time; the raw handle of the current device takes 0.1 us.)"""
+    global _raw_stream, _get_device
+    if _raw_stream is None:
+        import torch
+        if not torch.cuda.is_available():
+            return None
+        torch.cuda.init()
+        _raw_stream, _get_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+    return _raw_stream(_get_device())
 
 
 def make_shape(n_q_heads, n_kv_heads, head_dim, page_size, dtype, rope_theta, sm_scale) -> Shape:
