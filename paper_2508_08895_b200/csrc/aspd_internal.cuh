@@ -87,9 +87,20 @@ namespace aspd {
 // length-dependent ones have room for.
 struct PlanLayout {
   size_t o_items = 0, o_cta = 0, o_visit = 0, o_cdirty = 0, o_dirty = 0, o_tpage = 0, o_trow = 0, o_tpos = 0, o_tvis = 0,
-         o_rb = 0, o_pbase = 0, o_freq = 0, o_status = 0, o_arrive = 0, upload_bytes = 0, o_qcs = 0, o_wso = 0, o_wsml = 0, o_stq = 0,
+         o_rb = 0, o_pbase = 0, o_freq = 0, o_status = 0, o_arrive = 0, upload_bytes = 0, cleared_end = 0, o_qcs = 0, o_wso = 0, o_wsml = 0, o_stq = 0,
          o_stk = 0, o_stv = 0, o_sto = 0, o_stp = 0, device_bytes = 0;
   size_t cap_items = 0, cap_visit = 0, cap_dirty = 0, cap_partials = 0, n_row_blocks = 0, n_part_base = 0;
+};
+// A plan's device block, the page-locked host buffer its tables are assembled in, and the block's events.
+struct PlanBlock {
+  void* ptr = nullptr;
+  size_t bytes = 0;
+  void* host = nullptr;
+  size_t host_bytes = 0;
+  int device = -1;
+  cudaEvent_t upload_done = nullptr;   // recorded after the table copy: the host buffer may be rewritten once it has completed
+  std::vector<cudaEvent_t> events;     // the first n_wait: recorded on the streams the last plan was used on
+  int n_wait = 0;
 };
 }  // namespace aspd
 
@@ -120,10 +131,7 @@ struct aspd_plan {
   int64_t kv_tokens_read = 0;
   int64_t algorithmic_bytes = 0;
   size_t device_bytes = 0;
-  void* host_block = nullptr;      // page-locked host buffer the tables were assembled in (travels with the device block)
-  size_t host_block_bytes = 0;
-  cudaEvent_t upload_done = nullptr;   // recorded after the table copy: the host buffer may be rewritten once it has completed
-  size_t block_bytes = 0;          // size of the device block the plan holds (a reused block may be larger than needed)
+  aspd::PlanBlock block;           // the device block the plan holds (a reused one may be larger than needed)
   std::vector<cudaStream_t> streams;   // streams the plan's work was enqueued on
   void* device_base = nullptr;
   aspd::PlanDevice dev = {};

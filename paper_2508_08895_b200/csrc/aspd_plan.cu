@@ -29,108 +29,115 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // upload_done: recorded right after the plan's table copy; the host may write the buffer again only
 // once it has completed, so a block whose copy is still queued is passed over (a fresh one is
 // allocated instead and the pool settles at the depth the loop needs).
-struct ParkedBlock { void* ptr; size_t bytes; void* host; size_t host_bytes; int device; cudaEvent_t upload_done; std::vector<cudaEvent_t> events; };
+// The events live as long as the block: recording one again costs half of creating and destroying one.
 std::mutex g_blocks_mu;
-std::vector<ParkedBlock> g_blocks;
+std::vector<PlanBlock> g_blocks;
 constexpr size_t kParkedMax = 8;                       // blocks kept per process
 constexpr size_t kParkedMaxBytes = 2048ull << 20;     // all parked blocks together
 
-bool block_free(ParkedBlock& b) {
+bool block_free(PlanBlock& b) {
   for (cudaEvent_t e : b.events) cudaEventDestroy(e);
   if (b.upload_done) cudaEventDestroy(b.upload_done);
-  const bool ok = cudaFree(b.ptr) == cudaSuccess;    // waits for the device: the host buffer's last copy is done after it
+  const bool ok = b.ptr == nullptr || cudaFree(b.ptr) == cudaSuccess;    // waits for the device: the host buffer's last copy is done after it
   if (b.host) cudaFreeHost(b.host);
+  b = PlanBlock();
   return ok;
 }
 
-int block_acquire(size_t bytes, size_t host_need, cudaStream_t s, void** out, size_t* got, void** host, size_t* host_got) {
+// Sizes are rounded up (to a quarter of their power of two), so that the plans of steps that differ a little
+// share one size of block.
+size_t rounded_size(size_t bytes, size_t least) {
+  size_t p2 = least;
+  while (2 * p2 <= bytes) p2 *= 2;
+  return align_up(std::max(bytes, least), std::max(least, p2 / 4));
+}
+
+int block_acquire(size_t bytes, size_t host_need, cudaStream_t s, PlanBlock* out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return ASPD_ERR_CUDA;
+  bytes = rounded_size(bytes, 4u << 20); host_need = rounded_size(host_need, 64u << 10);
   {
     std::lock_guard<std::mutex> lock(g_blocks_mu);
     int best = -1, oldest = -1, fitting = 0;
     for (int i = 0; i < (int)g_blocks.size(); ++i) {
-      if (g_blocks[i].device != dev || g_blocks[i].bytes < bytes || g_blocks[i].bytes > 4 * bytes + (1u << 20)) continue;
+      if (g_blocks[i].device != dev || g_blocks[i].bytes < bytes || g_blocks[i].bytes > 4 * bytes) continue;
       ++fitting;
       if (oldest < 0) oldest = i;
-      if ((best < 0 || g_blocks[i].bytes < g_blocks[best].bytes) &&
-          (g_blocks[i].upload_done == nullptr || cudaEventQuery(g_blocks[i].upload_done) == cudaSuccess))
-        best = i;
+      if ((best < 0 || g_blocks[i].bytes < g_blocks[best].bytes) && cudaEventQuery(g_blocks[i].upload_done) == cudaSuccess) best = i;
     }
     // every fitting block still has its copy queued: with a couple of them parked the host is simply
     // ahead of the GPU and waits for the oldest one instead of allocating more
     if (best < 0 && fitting >= 2 && cudaEventSynchronize(g_blocks[oldest].upload_done) == cudaSuccess) best = oldest;
     if (best >= 0) {
-      ParkedBlock b = g_blocks[best];
+      PlanBlock b;
+      std::swap(b, g_blocks[best]);
       g_blocks.erase(g_blocks.begin() + best);
       int rc = ASPD_OK;
-      if (b.upload_done) cudaEventDestroy(b.upload_done);
-      for (cudaEvent_t e : b.events) {
-        if (cudaStreamWaitEvent(s, e, 0) != cudaSuccess) rc = ASPD_ERR_CUDA;
-        cudaEventDestroy(e);
-      }
+      for (int i = 0; i < b.n_wait; ++i)
+        if (cudaStreamWaitEvent(s, b.events[i], 0) != cudaSuccess) rc = ASPD_ERR_CUDA;
+      b.n_wait = 0;
       if (rc == ASPD_OK && b.host_bytes < host_need) {           // too small for the new tables (its last copy has completed)
         cudaFreeHost(b.host);
         b.host = nullptr; b.host_bytes = 0;
-        if (rc == ASPD_OK && cudaMallocHost(&b.host, host_need) != cudaSuccess) rc = ASPD_ERR_NOMEM;
-        if (rc == ASPD_OK) b.host_bytes = host_need;
+        if (cudaMallocHost(&b.host, host_need) != cudaSuccess) rc = ASPD_ERR_NOMEM;
+        else b.host_bytes = host_need;
       }
-      if (rc) { cudaFree(b.ptr); if (b.host) cudaFreeHost(b.host); return rc; }
-      *out = b.ptr; *got = b.bytes; *host = b.host; *host_got = b.host_bytes;
+      if (rc) { block_free(b); return rc; }
+      *out = b;
       return ASPD_OK;
     }
   }
-  if (cudaMalloc(out, bytes) != cudaSuccess) return ASPD_ERR_NOMEM;
-  if (cudaMallocHost(host, host_need) != cudaSuccess) { cudaFree(*out); return ASPD_ERR_NOMEM; }
-  *got = bytes; *host_got = host_need;
+  PlanBlock b;
+  b.device = dev; b.bytes = bytes; b.host_bytes = host_need;
+  if (cudaMalloc(&b.ptr, bytes) != cudaSuccess) { b.ptr = nullptr; return ASPD_ERR_NOMEM; }
+  if (cudaMallocHost(&b.host, host_need) != cudaSuccess) { b.host = nullptr; block_free(b); return ASPD_ERR_NOMEM; }
+  if (cudaEventCreateWithFlags(&b.upload_done, cudaEventDisableTiming) != cudaSuccess) { b.upload_done = nullptr; block_free(b); return ASPD_ERR_CUDA; }
+  *out = b;
   return ASPD_OK;
 }
 
-int block_release(void* ptr, size_t bytes, void* host, size_t host_bytes, cudaEvent_t upload_done,
-                  const std::vector<cudaStream_t>& streams) {
+int block_release(PlanBlock& b, const std::vector<cudaStream_t>& streams) {
   int dev = 0;
-  bool park = cudaGetDevice(&dev) == cudaSuccess;
-  cudaPointerAttributes attr;
-  if (park && (cudaPointerGetAttributes(&attr, ptr) != cudaSuccess || attr.device != dev)) park = false;   // freed from another device's context
-  std::vector<cudaEvent_t> events;
+  bool park = cudaGetDevice(&dev) == cudaSuccess && dev == b.device && b.bytes <= kParkedMaxBytes;   // not from another device's context
+  b.n_wait = 0;
   for (size_t i = 0; park && i < streams.size(); ++i) {
-    cudaEvent_t e;
-    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) { park = false; break; }
-    if (cudaEventRecord(e, streams[i]) != cudaSuccess) { cudaEventDestroy(e); park = false; break; }   // e.g. the stream is gone
-    events.push_back(e);
-  }
-  if (park && bytes <= kParkedMaxBytes) {
-    // The park keeps the blocks of the latest plans: the ones parked longest ago make room.  (A park
-    // that kept the earliest ones -- a batch whose size has changed since never fits them -- turned
-    // every later plan into cudaMalloc + cudaFree, i.e. a device synchronisation per step: a serving
-    // mix step of 28 layers took 2.46 ms instead of 1.48 once eight other sizes had been planned.)
-    std::vector<ParkedBlock> evicted;
-    {
-      std::lock_guard<std::mutex> lock(g_blocks_mu);
-      size_t parked = bytes;
-      for (const ParkedBlock& b : g_blocks) parked += b.bytes;
-      while (!g_blocks.empty() && (g_blocks.size() >= kParkedMax || parked > kParkedMaxBytes)) {
-        parked -= g_blocks.front().bytes;
-        evicted.push_back(g_blocks.front());
-        g_blocks.erase(g_blocks.begin());
-      }
-      g_blocks.push_back({ptr, bytes, host, host_bytes, dev, upload_done, events});
+    if (i == b.events.size()) {
+      cudaEvent_t e;
+      if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) { park = false; break; }
+      b.events.push_back(e);
     }
-    for (ParkedBlock& b : evicted) block_free(b);
-    return ASPD_OK;
+    if (cudaEventRecord(b.events[i], streams[i]) != cudaSuccess) park = false;   // e.g. the stream is gone
+    else b.n_wait = (int)i + 1;
   }
-  ParkedBlock b = {ptr, bytes, host, host_bytes, dev, upload_done, events};
-  return block_free(b) ? ASPD_OK : ASPD_ERR_CUDA;
+  if (!park) return block_free(b) ? ASPD_OK : ASPD_ERR_CUDA;
+  // The park keeps the blocks of the latest plans: the ones parked longest ago make room.  (A park
+  // that kept the earliest ones -- a batch whose size has changed since never fits them -- turned
+  // every later plan into cudaMalloc + cudaFree, i.e. a device synchronisation per step: a serving
+  // mix step of 28 layers took 2.46 ms instead of 1.48 once eight other sizes had been planned.)
+  std::vector<PlanBlock> evicted;
+  {
+    std::lock_guard<std::mutex> lock(g_blocks_mu);
+    size_t parked = b.bytes;
+    for (const PlanBlock& x : g_blocks) parked += x.bytes;
+    while (!g_blocks.empty() && (g_blocks.size() >= kParkedMax || parked > kParkedMaxBytes)) {
+      parked -= g_blocks.front().bytes;
+      evicted.push_back(g_blocks.front());
+      g_blocks.erase(g_blocks.begin());
+    }
+    g_blocks.push_back(b);
+  }
+  for (PlanBlock& x : evicted) block_free(x);
+  return ASPD_OK;
 }
 
 int block_cache_clear() {
-  std::vector<ParkedBlock> all;
+  std::vector<PlanBlock> all;
   {
     std::lock_guard<std::mutex> lock(g_blocks_mu);
     all.swap(g_blocks);
   }
   int rc = ASPD_OK;
-  for (ParkedBlock& b : all)
+  for (PlanBlock& b : all)
     if (!block_free(b)) rc = ASPD_ERR_CUDA;
   return rc;
 }
@@ -197,12 +204,10 @@ int check_layout(const aspd_shape_t* s, const aspd_request_t* req, const aspd_br
     }
     for (const Region& g : regs)
       if (g.hi > cap) return ASPD_ERR_BAD_DESCRIPTOR;
-    std::vector<Region> sorted;
-    for (const Region& g : regs)
-      if (g.hi > g.lo) sorted.push_back(g);
-    std::sort(sorted.begin(), sorted.end(), [](const Region& a, const Region& b) { return a.lo < b.lo; });
-    for (size_t i = 1; i < sorted.size(); ++i)
-      if (sorted[i].lo < sorted[i - 1].hi) return ASPD_ERR_BAD_DESCRIPTOR;
+    regs.erase(std::remove_if(regs.begin(), regs.end(), [](const Region& g) { return g.hi <= g.lo; }), regs.end());
+    std::sort(regs.begin(), regs.end(), [](const Region& a, const Region& b) { return a.lo < b.lo; });
+    for (size_t i = 1; i < regs.size(); ++i)
+      if (regs[i].lo < regs[i - 1].hi) return ASPD_ERR_BAD_DESCRIPTOR;
     for (int p = 0; p < q.n_pages; ++p) {
       int32_t id = page_ids[q.page_begin + p];
       if (id < 0 || id >= n_pool_pages) return ASPD_ERR_BAD_DESCRIPTOR;
@@ -426,14 +431,20 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     // first key's offset / page_size; such plans never fuse the append): a token at offset k
     // also sees the keys of other branches whose offset is below k.
     auto push_region = [&](const aspd_request_t& q, int slot0, int len, int new_key0, int new_tok0, bool branch_pages = false) {
-      for (int s0 = 0; s0 < len; s0 += ps) {
+      const size_t at = visit.size();
+      const int32_t* ids = page_ids + q.page_begin + slot0 / ps;
+      const int n_old = (shared_mask && branch_pages) ? 0 : std::min(len, new_key0) / ps;       // full pages without new rows
+      visit.resize(at + (len + ps - 1) / ps);
+      int2* out = visit.data() + at;
+      for (int i = 0; i < n_old; ++i) out[i] = make_int2(ids[i], ps);
+      for (int s0 = n_old * ps; s0 < len; s0 += ps) {
         const int nv = std::min(ps, len - s0), first_new = std::max(s0, new_key0);
         const int n_newrows = std::max(0, s0 + nv - first_new);
         int y = nv;
         if (n_newrows > 0) y |= (std::min(n_newrows, 31) << 8);   // 5 bits; a count is only needed where pages have 16 rows
         if (shared_mask) y |= branch_pages ? (s0 / ps) << 13 : 0;
         else if (n_newrows > 0 && tok_field_fits) y |= (new_tok0 + first_new - new_key0) << 13;
-        visit.push_back(make_int2(page_ids[q.page_begin + (slot0 + s0) / ps], y));
+        out[s0 / ps] = make_int2(ids[s0 / ps], y);
       }
     };
     auto push_shared = [&](const aspd_request_t& q) {            // prefix and regions of earlier stages: seen by every branch
@@ -468,10 +479,17 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
           }
           blocks.push_back({r, t_req, nq, v0, (int)visit.size() - v0});
         } else {
+          int n_shared = 0;                                    // pages that every block of the request lists
           for (int blk0 = 0; blk0 < nq; blk0 += block_tok) {
             const int blk1 = std::min(nq, blk0 + block_tok), bv0 = (int)visit.size();
-            push_shared(q);
-            const int pe = ((int)visit.size() - bv0) * ps;
+            if (blk0 == 0) {
+              push_shared(q);
+              n_shared = (int)visit.size() - bv0;
+            } else {                                           // as in the request's first block
+              visit.resize((size_t)bv0 + n_shared);
+              std::copy(visit.begin() + v0, visit.begin() + v0 + n_shared, visit.begin() + bv0);
+            }
+            const int pe = n_shared * ps;
             int off = 0;                                       // index, among the request's new tokens, of the branch's first
             for (int b = 0; b < q.n_branches; ++b) {
               const aspd_branch_t& x = br[q.branch_begin + b];
@@ -637,27 +655,32 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     }
     while (cta < n_ctas) cta_item0[++cta] = (int)p->items.size();
   }
-  // rows that are new this step, per CTA: what a fused step must write before the CTA reads
+  // Rows that are new this step, per CTA: what a fused step must write before the CTA reads.  The fused step
+  // writes them in batches at the start of the kernel; with many new rows per CTA (a branch-open step) the
+  // separate append kernel is the faster way, and such plans carry no list.  (The few pages that hold new rows
+  // are found once, not once per KV head and CTA.)
+  constexpr int kMostFused = 20;
   std::vector<int4> dirty;
   std::vector<int32_t> cta_dirty0(n_ctas + 1, 0);
-  for (int c = 0; c < n_ctas; ++c) {
-    cta_dirty0[c] = (int)dirty.size();
-    for (int i = cta_item0[c]; i < cta_item0[c + 1] && !shared_mask; ++i) {
-      const DeviceItem& it = p->items[i];
-      for (int pg = 0; pg < it.n_pages; ++pg) {
-        const int2 v = visit[it.page0 + pg];
-        const int cnt = (v.y >> 8) & 31, tok0 = v.y >> 13, row0 = (v.y & 255) - cnt;
-        for (int k = 0; k < cnt; ++k) dirty.push_back(make_int4(v.x, it.kv_head, tok0 + k, row0 + k));
+  p->fuse_append = (kernel == ASPD_KERNEL_MMA && !shared_mask && tok_field_fits && p->wide != 2) ? 1 : 0;
+  if (p->fuse_append) {
+    std::vector<int> fresh;                        // entries of `visit` with new rows, ascending
+    for (size_t i = 0; i < visit.size(); ++i)
+      if ((visit[i].y >> 8) & 31) fresh.push_back((int)i);
+    for (int c = 0; c < n_ctas && p->fuse_append; ++c) {
+      cta_dirty0[c] = (int)dirty.size();
+      for (int i = cta_item0[c]; i < cta_item0[c + 1]; ++i) {
+        const DeviceItem& it = p->items[i];
+        for (auto e = std::lower_bound(fresh.begin(), fresh.end(), it.page0); e != fresh.end() && *e < it.page0 + it.n_pages; ++e) {
+          const int2 v = visit[*e];
+          const int cnt = (v.y >> 8) & 31, tok0 = v.y >> 13, row0 = (v.y & 255) - cnt;
+          for (int k = 0; k < cnt; ++k) dirty.push_back(make_int4(v.x, it.kv_head, tok0 + k, row0 + k));
+        }
       }
+      if ((int)dirty.size() - cta_dirty0[c] > kMostFused) p->fuse_append = 0;
     }
-  }
-  cta_dirty0[n_ctas] = (int)dirty.size();
-  {
-    // the fused step writes a CTA's new rows in batches at the start of the kernel; with many new
-    // rows per CTA (a branch-open step) the separate append kernel is the faster way
-    int most = 0;
-    for (int c = 0; c < n_ctas; ++c) most = std::max(most, cta_dirty0[c + 1] - cta_dirty0[c]);
-    p->fuse_append = (most <= 20 && !shared_mask && tok_field_fits && p->wide != 2) ? 1 : 0;
+    cta_dirty0[n_ctas] = (int)dirty.size();
+    if (!p->fuse_append) { dirty.clear(); std::fill(cta_dirty0.begin(), cta_dirty0.end(), 0); }
   }
   // the merge of a token's records inside the attention kernel: stream-K plans of the tensor-core kernel
   // 1: both MMAs with M = 64; 2: only P.V (the default: at most 64 of P.V's 128 rows are ever read, a quarter
@@ -676,11 +699,9 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   p->n_partials = part_base[n_parts.size()];
   p->kv_tokens_read = kv_tokens;
   p->algorithmic_bytes = 2LL * Hkv * d * es * kv_tokens + 2LL * es * Hq * d * n_new + 2LL * Hkv * d * es * n_new;
-  p->visit = visit;
   p->n_row_blocks = (int)row_blocks.size();
-  p->cta_item0 = cta_item0; p->part_base = part_base; p->row_blocks = row_blocks; p->q_pos = pos;
-  p->tok_vis = tok_vis;
-  p->tok_page = tok_page; p->tok_row = tok_row; p->dirty = dirty; p->cta_dirty0 = cta_dirty0;
+  p->visit.swap(visit); p->cta_item0.swap(cta_item0); p->part_base.swap(part_base); p->row_blocks.swap(row_blocks); p->q_pos.swap(pos);
+  p->tok_vis.swap(tok_vis); p->tok_page.swap(tok_page); p->tok_row.swap(tok_row); p->dirty.swap(dirty); p->cta_dirty0.swap(cta_dirty0);
   if (tune.host_only) { *plan_out = p; return ASPD_OK; }
   rc = plan_to_device(p, (cudaStream_t)stream);
   if (rc) { delete p; return rc; }
@@ -703,7 +724,7 @@ static void plan_layout(const aspd_plan* p, double slack, aspd::PlanLayout* L) {
   const int d = sh.head_dim, Hq = sh.n_q_heads, Hkv = sh.n_kv_heads, G = Hq / Hkv, es = esize_of(sh.dtype), n_new = p->n_new;
   auto cap = [&](size_t n) { return std::max<size_t>(1, (size_t)((double)n * slack) + (slack > 1.0 ? 64 : 0)); };
   L->cap_items = cap(p->items.size()); L->cap_visit = cap(p->visit.size()); L->cap_dirty = cap(p->dirty.size());
-  L->cap_partials = cap((size_t)p->n_partials);
+  L->cap_partials = p->wide == 2 ? 1 : cap((size_t)p->n_partials);      // (the two-tile kernel never writes records)
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   L->o_items = take(sizeof(DeviceItem) * L->cap_items);
@@ -722,7 +743,8 @@ static void plan_layout(const aspd_plan* p, double slack, aspd::PlanLayout* L) {
   // the status word is zeroed when the plan is created and never uploaded again, so that a time-out
   // recorded by an earlier launch survives aspd_plan_update until aspd_plan_status reads it
   L->o_status = take(sizeof(int32_t) * 2);
-  L->o_arrive = take(sizeof(int32_t) * std::max(1, n_new) * Hkv);   // right behind the status word: cleared with it
+  L->o_arrive = take(p->single_launch ? sizeof(int32_t) * std::max(1, n_new) * Hkv : 0);   // right behind the status word: cleared with it
+  L->cleared_end = off;
   L->o_qcs = take(sizeof(float2) * std::max(1, n_new) * (d / 2));   // filled on the device from tok_pos and inv_freq
   L->o_wso = take(sizeof(float) * L->cap_partials * G * d);
   L->o_wsml = take(sizeof(float2) * L->cap_partials * G);
@@ -737,11 +759,10 @@ static void plan_layout(const aspd_plan* p, double slack, aspd::PlanLayout* L) {
 
 // Assembles the tables in the plan's page-locked buffer, sends them to the device block and fills
 // the cos/sin table there.  The caller has made sure that the buffer's previous copy has completed.
-static int plan_upload(aspd_plan* p, cudaStream_t s) {
+static int plan_upload(aspd_plan* p, cudaStream_t s, bool clear) {
   const aspd::PlanLayout& L = p->layout;
   const int n_new = p->n_new, d = p->shape.head_dim, n_ctas = p->n_ctas;
-  uint8_t* blob = static_cast<uint8_t*>(p->host_block);
-  memset(blob, 0, L.upload_bytes);
+  uint8_t* blob = static_cast<uint8_t*>(p->block.host);
   if (!p->items.empty()) memcpy(blob + L.o_items, p->items.data(), sizeof(DeviceItem) * p->items.size());
   fill_cta_head(p, reinterpret_cast<int4*>(blob + L.o_cta));
   if (!p->visit.empty()) memcpy(blob + L.o_visit, p->visit.data(), sizeof(int2) * p->visit.size());
@@ -757,14 +778,13 @@ static int plan_upload(aspd_plan* p, cudaStream_t s) {
   memcpy(blob + L.o_pbase, p->part_base.data(), sizeof(int32_t) * p->part_base.size());
   double* freq = reinterpret_cast<double*>(blob + L.o_freq);
   for (int i = 0; i < d / 2; ++i) freq[i] = pow((double)p->shape.rope_theta, -2.0 * i / d);
-  if (cudaMemcpyAsync(p->device_base, blob, L.upload_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) return ASPD_ERR_CUDA;
-  if (p->upload_done) { cudaEventDestroy(p->upload_done); p->upload_done = nullptr; }
-  if (cudaEventCreateWithFlags(&p->upload_done, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventRecord(p->upload_done, s) != cudaSuccess) {
-    if (p->upload_done) cudaEventDestroy(p->upload_done);
-    p->upload_done = nullptr;
-    cudaStreamSynchronize(s);                      // no event to tell when the buffer is free again: be done with it now
+  size_t bytes = L.upload_bytes;
+  if (clear) {                                     // the status word and the counters lie right behind the tables: one copy
+    memset(blob + L.o_status, 0, L.cleared_end - L.o_status);
+    bytes = L.cleared_end;
   }
+  if (cudaMemcpyAsync(p->device_base, blob, bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) return ASPD_ERR_CUDA;
+  if (cudaEventRecord(p->block.upload_done, s) != cudaSuccess) return ASPD_ERR_CUDA;
   if (std::find(p->streams.begin(), p->streams.end(), s) == p->streams.end()) p->streams.push_back(s);
   // cos/sin of every new token's position (query rotation, fused append): on the device, after the upload
   return n_new > 0 ? launch_qcs(p, s) : ASPD_OK;
@@ -774,11 +794,10 @@ static int plan_to_device(aspd_plan* p, cudaStream_t s) {
   plan_layout(p, p->tune.updatable ? 1.25 : 1.0, &p->layout);
   const aspd::PlanLayout& L = p->layout;
   p->device_bytes = L.device_bytes;
-  void* base = nullptr;
-  int rc = block_acquire(L.device_bytes, L.upload_bytes, s, &base, &p->block_bytes, &p->host_block, &p->host_block_bytes);
+  int rc = block_acquire(L.device_bytes, L.cleared_end, s, &p->block);
   if (rc) return rc;
-  uint8_t* b8 = (uint8_t*)base;
-  p->device_base = base;
+  uint8_t* b8 = (uint8_t*)p->block.ptr;
+  p->device_base = b8;
   p->dev.items = (const DeviceItem*)(b8 + L.o_items);
   p->dev.cta_head = (const int4*)(b8 + L.o_cta);
   p->dev.visit = (const int2*)(b8 + L.o_visit);
@@ -800,12 +819,8 @@ static int plan_to_device(aspd_plan* p, cudaStream_t s) {
   p->dev.st_q = b8 + L.o_stq; p->dev.st_k = b8 + L.o_stk; p->dev.st_v = b8 + L.o_stv; p->dev.st_out = b8 + L.o_sto;
   p->dev.st_pos = (int32_t*)(b8 + L.o_stp);
   p->dev.pool_limit = (int32_t)std::min<int64_t>(p->n_pool_pages, INT32_MAX);
-  rc = cudaMemsetAsync(p->dev.status, 0, (L.o_arrive - L.o_status) + sizeof(int32_t) * std::max(1, p->n_new) * p->shape.n_kv_heads, s) == cudaSuccess
-           ? plan_upload(p, s) : ASPD_ERR_CUDA;
-  if (rc) {
-    cudaFree(base); cudaFreeHost(p->host_block);
-    p->device_base = nullptr; p->host_block = nullptr;
-  }
+  rc = plan_upload(p, s, true);
+  if (rc) { block_free(p->block); p->device_base = nullptr; }
   return rc;
 }
 
@@ -826,25 +841,25 @@ int aspd_plan_update(aspd_plan_t* p, const aspd_request_t* req, const aspd_branc
     return ASPD_ERR_UNSUPPORTED;
   }
   if (t->items.size() > L.cap_items || t->visit.size() > L.cap_visit || t->dirty.size() > L.cap_dirty ||
-      (size_t)t->n_partials > L.cap_partials) {
+      (p->wide != 2 && (size_t)t->n_partials > L.cap_partials)) {
     delete t;
     return ASPD_ERR_TOO_LARGE;
   }
   // the page-locked buffer is written again: its previous copy must be through
-  if (p->upload_done && cudaEventSynchronize(p->upload_done) != cudaSuccess) { delete t; return ASPD_ERR_CUDA; }
+  if (cudaEventSynchronize(p->block.upload_done) != cudaSuccess) { delete t; return ASPD_ERR_CUDA; }
   p->n_req = t->n_req; p->n_items = t->n_items; p->n_partials = t->n_partials; p->n_row_blocks = t->n_row_blocks;
   p->kv_tokens_read = t->kv_tokens_read; p->algorithmic_bytes = t->algorithmic_bytes;
   p->items.swap(t->items); p->visit.swap(t->visit); p->tok_vis.swap(t->tok_vis); p->cta_item0.swap(t->cta_item0);
   p->part_base.swap(t->part_base); p->q_pos.swap(t->q_pos); p->row_blocks.swap(t->row_blocks);
   p->tok_page.swap(t->tok_page); p->tok_row.swap(t->tok_row); p->cta_dirty0.swap(t->cta_dirty0); p->dirty.swap(t->dirty);
   delete t;
-  return plan_upload(p, (cudaStream_t)stream);
+  return plan_upload(p, (cudaStream_t)stream, false);
 }
 
 int aspd_plan_destroy(aspd_plan_t* plan) {
   if (!plan) return ASPD_OK;
   int rc = ASPD_OK;
-  if (plan->device_base) rc = block_release(plan->device_base, plan->block_bytes, plan->host_block, plan->host_block_bytes, plan->upload_done, plan->streams);
+  if (plan->device_base) rc = block_release(plan->block, plan->streams);
   delete plan;
   return rc;
 }

@@ -32,3 +32,34 @@ def test_a_plan_size_used_after_many_others_is_parked_too(earlier):
 
 def _shape(wl):
     return B.make_shape(wl.Hq, wl.Hkv, wl.d, wl.page_size, wl.dtype, wl.theta, wl.sm_scale)
+
+
+@pytest.mark.parametrize("n_streams", [1, 3])
+def test_blocks_that_change_streams_keep_the_plans_apart(n_streams):
+    """Plans made and destroyed in turn on several streams, with different steps sharing one size of block: every
+    result is its own step's, also for the plans whose block was last used on another stream."""
+    import torch
+    from paper_2508_08895_b200 import engine as E
+    wls = [W.build_segment_workload("s", 60 + i, 28, 4, 128, "bf16", 1e6, [300 + 64 * i], [[20, 9 + i]], [[1, 1]]) for i in range(3)]
+    runs, want, args = [], [], []
+    for wl in wls:
+        run = E.WorkloadRun(wl)
+        for ph in wl.phases:
+            run.step(ph)
+        ph = wl.phases[-1]
+        runs.append(run); want.append(run.outputs[-1])
+        args.append([E.to_device(x, wl.dtype) for x in (ph.q, ph.k_new, ph.v_new)])
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(n_streams)]
+    outs = []
+    for i in range(40):
+        wl, run, st, (q, k, v) = wls[i % 3], runs[i % 3], streams[(i * 7 // 3) % n_streams], args[i % 3]
+        out = torch.full_like(q, float("nan"))
+        st.wait_stream(torch.cuda.current_stream())
+        plan = B.Plan(run.shape, wl.phases[-1].desc, wl.n_pool_pages, B.MODE_BRANCH, stream=st)
+        B.branch_attn(plan, q, run.cache.k, run.cache.v, out, stream=st)
+        plan.destroy()
+        outs.append(out)
+    torch.cuda.synchronize()
+    for i, out in enumerate(outs):
+        assert (E.to_host_f32(out) == want[i % 3]).all(), i
