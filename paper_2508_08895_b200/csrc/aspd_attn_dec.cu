@@ -182,7 +182,8 @@ __device__ __forceinline__ void append_rows(const Ctx& c, int tid, int n_threads
   constexpr int UK = D / 16, U = UK + D / 8;
   const uint32_t tb = (uint32_t)c.page_size * D * 2;
   for (int u = tid; u < n_rows * U; u += n_threads) {
-    const int4 d = c.pd.dirty[d0 + u / U];                        // (page, KV head, token, row)
+    int4 d = c.pd.dirty[d0 + u / U];                              // (page, KV head, token, row | ...)
+    d.w &= 255;
     const int sub = u % U;
     if (!bounds_ok(c.pd, d.x, d.w, c.page_size)) continue;
     const size_t src = ((size_t)d.z * c.n_kv_heads + d.y) * D, tile = ((size_t)d.x * c.n_kv_heads + d.y) * tb;
@@ -448,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
   volatile int* ab = &misc->abort_flag;
   constexpr uint32_t kTileBytes = kTile * D * 2;
   if (tid == 0) pdl_launch_dependents();
-  const int4 head = c.pd.cta_head[blockIdx.x];
+  const int4 head = c.pd.cta_head[2 * blockIdx.x], head2 = c.pd.cta_head[2 * blockIdx.x + 1];
   const int item_begin = head.x, item_end = head.y;
   const int ps = c.page_size, ps_shift = 31 - __clz(ps), ppt = kTile >> ps_shift;
   int2 first_pages = make_int2(0, 0);
@@ -467,11 +468,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = misc->tmem_base;
-  // plan data of the first item and of the fused append
+  // plan data of the first item
   DeviceItem first = {};
-  int dirty0 = 0, dirty_rows = 0;
   if (warp < 8 && item_begin < item_end) first = c.pd.items[item_begin];
-  if (warp >= W_S && c.k_new != nullptr) { dirty0 = c.pd.cta_dirty0[blockIdx.x]; dirty_rows = c.pd.cta_dirty0[blockIdx.x + 1] - dirty0; }
   // everything above touches only the plan's own tables; inputs written by earlier kernels of the stream are
   // used from here on.  With the plan's stable-cache promise the producers go ahead with pages that hold no
   // new rows; they wait themselves before the first page that does.
@@ -590,7 +589,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
     auto wait_all = [&](uint32_t bar, uint32_t parity) { return __all_sync(fm, mbar_wait(bar, parity, ab)) != 0; };
     constexpr uint32_t kRowGroup = 8 * D * 2;                     // bytes of 8 tokens in a tile
     if (c.k_new != nullptr) {                                     // beside the preparation of the first query tile
-      append_rows<D>(c, tid - W_S * 32, 64, dirty0, dirty_rows);
+      append_rows<D>(c, tid - W_S * 32, 64, head2.x, head2.y);
       warp_arrive(bars + 8 * A_DONE, lane);
     }
     int g = 0, item_no = 0;

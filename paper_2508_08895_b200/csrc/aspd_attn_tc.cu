@@ -53,9 +53,9 @@ constexpr uint32_t OFF_K = 0, OFF_V = 2 * kTileBytes, OFF_Q = 4 * kTileBytes, OF
 constexpr uint32_t OFF_MISC = OFF_P + 8192;
 
 enum Bar { K_FULL = 0, K_EMPTY = 2, V_FULL = 4, V_EMPTY = 6, S_FULL = 8, S_EMPTY = 10, P_FULL = 12, P_EMPTY = 13,
-           O_FULL = 14, O_EMPTY = 16, Q_FULL = 18, Q_EMPTY = 20, E_FULL = 22, A_DONE = 24, NUM_BARS = 25 };
+           O_FULL = 14, O_EMPTY = 16, Q_FULL = 18, Q_EMPTY = 20, E_FULL = 22, K_PATCH = 24, V_PATCH = 26, A_DONE = 28, NUM_BARS = 29 };
 
-constexpr int kItemCache = 10;      // items of a CTA kept in shared memory (more are read from global)
+constexpr int kItemCache = 9;       // items of a CTA kept in shared memory (more are read from global)
 constexpr int kMergeQueue = 21;     // (token, KV head) pairs whose last record this CTA stored, waiting to be merged
 constexpr int kMaxTokPerItem = 16;  // tokens of a row block whose ranges are cached (n_q_tok is at most 64 / G)
 
@@ -78,7 +78,11 @@ struct Misc {
   int mq[kMergeQueue][3];      // (token * n_kv_heads + KV head, first record, number of records)
 };
 static_assert(sizeof(Misc) <= 8192, "Misc must fit into the unused rows of the P tile");
-constexpr size_t kSmemBytes = 7 * kTileBytes + 1024;   // + slack to align the base to 1024
+// The step's new rows (512 bytes each: K, rotated, and V) wait in shared memory until their tiles have landed (plans
+// that patch their tiles): the first sixteen in the unused rows of the P tile's second span, the rest behind the tiles.
+constexpr uint32_t OFF_ROWS = OFF_P + kHalf + 8192, OFF_ROWS2 = 7 * kTileBytes;
+constexpr size_t kSmemBytes = 7 * kTileBytes + (kMostFusedRows - 16) * 512 + 1024;   // + slack to align the base to 1024
+__device__ __forceinline__ uint32_t row_stash(uint32_t base, int e) { return base + (e < 16 ? OFF_ROWS + e * 512 : OFF_ROWS2 + (e - 16) * 512); }
 
 // TMEM columns: S double buffer, O double buffer
 constexpr uint32_t COL_S = 0, COL_O = 256;
@@ -106,6 +110,7 @@ struct Ctx {
   const char* k_pool;
   const char* v_pool;
   int n_items, n_q_heads, n_kv_heads;
+  int G, inv_g;                // query heads of a KV head; 65536 / G rounded up (token_of)
   float scale_log2;
   int early_fetch;             // plan promise: pages without new rows are not written by in-flight work
   int m64;                     // MMAs with M = 64: row blocks of at most 64 rows are not padded to 128 (half the tensor work)
@@ -121,13 +126,16 @@ struct Ctx {
 // records in slot order (the combine kernel's arithmetic).  Called by `n_warps` warps that have
 // passed a barrier after the last push; the caller resets the queue behind another barrier.
 __device__ __forceinline__ void drain_merge_queue(const Ctx& c, const Misc* misc, int warp_rank, int n_warps, int lane) {
-  const int G = c.n_q_heads / c.n_kv_heads, n = min(misc->mq_n, kMergeQueue) * G;
+  const int G = c.G, n = min(misc->mq_n, kMergeQueue) * G;
   for (int u = warp_rank; u < n; u += n_warps) {
     const int idx = misc->mq[u / G][0], g = u % G, tok = idx / c.n_kv_heads, h = idx % c.n_kv_heads;
     const int p0 = misc->mq[u / G][1], np = misc->mq[u / G][2];
     combine_row<__nv_bfloat16, 128>(c.pd.ws_o, c.pd.ws_ml, p0, np, G, g, lane, c.merge_out + ((size_t)tok * c.n_q_heads + h * G + g) * 128);
   }
 }
+
+// r / G of a row index below 256 (G is at most 64): a division by a run-time number is some forty instructions
+__device__ __forceinline__ int token_of(const Ctx& c, int r) { return (r * c.inv_g) >> 16; }
 
 // Item idx of this CTA (rel = idx - item_begin): from the shared-memory cache when it is there.
 __device__ __forceinline__ DeviceItem get_item(const Ctx& c, const Misc* misc, int idx, int item_begin) {
@@ -147,14 +155,15 @@ __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it,
                                              uint32_t tmem, int item_no, int& g) {   // item_no = index among this CTA's items
   constexpr int R = NC, KS = 128 / NC, HC = NC / 2;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int tl = tid & 127, half = tid >> 7;     // TMEM lane of the thread; which half of the replica's columns
-  const int r = tl % R, j = tl / R;
+  const int tmem_lane = tid & 127, half = tid >> 7;     // of the thread; which half of the replica's columns
+  const int r = tmem_lane % R, j = tmem_lane / R;
   const int col0 = j * NC + half * HC;           // first tile column (key) of this thread
-  const int G = c.n_q_heads / c.n_kv_heads, M = it.n_q_tok * G;
+  const int G = c.G, M = it.n_q_tok * G;
   const int n_tiles = (it.n_pages + 7) >> 3;
   volatile int* ab = &misc->abort_flag;
   int4 vis = make_int4(0, 0, 0, 0);             // padding rows see nothing
-  if (r < M) vis = (item_no < kItemCache && r / G < kMaxTokPerItem) ? misc->vis[item_no][r / G] : c.pd.tok_vis[it.q_tok0 + r / G];
+  const int tl = token_of(c, r);
+  if (r < M) vis = (item_no < kItemCache && tl < kMaxTokPerItem) ? misc->vis[item_no][tl] : c.pd.tok_vis[it.q_tok0 + tl];
   const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
   const bool o_owner = half == 0 && (warp & 3) < R / 32;   // threads whose TMEM lane holds a row of O
   const int ob = item_no & 1;
@@ -345,12 +354,13 @@ __device__ __forceinline__ bool softmax_item_m64(const Ctx& c, const DeviceItem&
   const int j = rho_a / R;                                     // their replica (the same for both: R is a multiple of 16)
   const int ra = rho_a % R, rb = rho_b % R;                    // the query rows they stand for
   const int col0 = j * NCOL + half * NH;                       // first tile column (key) of this thread
-  const int G = c.n_q_heads / c.n_kv_heads, M = it.n_q_tok * G;
+  const int G = c.G, M = it.n_q_tok * G;
   const int n_tiles = (it.n_pages + 7) >> 3;
   volatile int* ab = &misc->abort_flag;
   int4 vis_a = make_int4(0, 0, 0, 0), vis_b = vis_a;           // padding rows see nothing
-  if (ra < M) vis_a = (item_no < kItemCache && ra / G < kMaxTokPerItem) ? misc->vis[item_no][ra / G] : c.pd.tok_vis[it.q_tok0 + ra / G];
-  if (rb < M) vis_b = (item_no < kItemCache && rb / G < kMaxTokPerItem) ? misc->vis[item_no][rb / G] : c.pd.tok_vis[it.q_tok0 + rb / G];
+  const int tla = token_of(c, ra), tlb = token_of(c, rb);
+  if (ra < M) vis_a = (item_no < kItemCache && tla < kMaxTokPerItem) ? misc->vis[item_no][tla] : c.pd.tok_vis[it.q_tok0 + tla];
+  if (rb < M) vis_b = (item_no < kItemCache && tlb < kMaxTokPerItem) ? misc->vis[item_no][tlb] : c.pd.tok_vis[it.q_tok0 + tlb];
   const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
   const bool o_owner = half == 0 && j == 0;                    // threads whose rows are rows of O
   const int ob = item_no & 1;
@@ -509,12 +519,13 @@ __device__ __forceinline__ bool softmax_item_wide(const Ctx& c, const DeviceItem
   const int tid = threadIdx.x, warp = tid >> 5;
   const int r = tid & 127, half = tid >> 7;
   const int col0 = half * 64;
-  const int G = c.n_q_heads / c.n_kv_heads, M = it.n_q_tok * G;
+  const int G = c.G, M = it.n_q_tok * G;
   const int n_tiles = (it.n_pages + 7) >> 3;
   volatile int* ab = &misc->abort_flag;
   float* fin_m_wide = reinterpret_cast<float*>(misc + 1);
   int4 vis = make_int4(0, 0, 0, 0);
-  if (r < M) vis = (item_no < kItemCache && r / G < kMaxTokPerItem) ? misc->vis[item_no][r / G] : c.pd.tok_vis[it.q_tok0 + r / G];
+  const int tl = token_of(c, r);
+  if (r < M) vis = (item_no < kItemCache && tl < kMaxTokPerItem) ? misc->vis[item_no][tl] : c.pd.tok_vis[it.q_tok0 + tl];
   const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
   const bool o_owner = half == 0;
   const int ob = item_no & 1;
@@ -627,26 +638,28 @@ __device__ __forceinline__ bool softmax_item_wide(const Ctx& c, const DeviceItem
 
 // Rotate the item's query rows (RoPE at the token's position, cos/sin table from the plan),
 // round to bf16 and store them, replicated KS = 128 / R times, as the 128-byte-swizzled K-major
-// A operand.  Called by the 128 epilogue threads (rank 0..127); all loads of a thread's rows
-// are issued before the first use.  Unit e = (row e / 8, 16-byte chunk e % 8 of each span); a
-// call covers units e0 + rank + 128 u, u < 4 (row blocks of 128 rows need two calls).
+// A operand.  Called by NT threads (rank 0 .. NT - 1); all loads of a thread's rows are issued
+// before the first use.  Unit e = (row e / 8, 16-byte chunk e % 8 of each span); a call covers
+// units e0 + rank + NT u, u < U (row blocks of 64 rows have 512 units, of 128 rows 1024).
+template <int U>
 struct QUnits {
-  uint32_t lo[4][4], hi[4][4];   // per unit: the rotated chunk of the first and of the second span, bf16 pairs
+  uint32_t lo[U][4], hi[U][4];   // per unit: the rotated chunk of the first and of the second span, bf16 pairs
 };
 // tile128: the rows always form a 128-row tile of their own (no replication), however few they are
-__device__ __forceinline__ void prep_q_compute(const Ctx& c, const DeviceItem& it, int rank, int e0, QUnits& qu, bool tile128 = false) {
-  const int G = c.n_q_heads / c.n_kv_heads;
+template <int NT = 128, int U = 4>
+__device__ __forceinline__ void prep_q_compute(const Ctx& c, const DeviceItem& it, int rank, int e0, QUnits<U>& qu, bool tile128 = false) {
+  const int G = c.G;
   const int M = it.n_q_tok * G, R = tile128 ? 128 : (M <= 32 ? 32 : (M <= 64 ? 64 : 128));
-  uint4 a[4], b[4];
-  float4 w[4][4];
+  uint4 a[U], b[U];
+  float4 w[U][4];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int e = e0 + rank + u * 128, r = e >> 3, ch = e & 7;
+  for (int u = 0; u < U; ++u) {
+    const int e = e0 + rank + u * NT, r = e >> 3, ch = e & 7;
     a[u] = make_uint4(0, 0, 0, 0); b[u] = make_uint4(0, 0, 0, 0);
 #pragma unroll
     for (int i = 0; i < 4; ++i) w[u][i] = make_float4(1.f, 0.f, 1.f, 0.f);
     if (e < R * 8 && r < M) {
-      const int tok = it.q_tok0 + r / G, hq = it.kv_head * G + r % G;
+      const int tl = token_of(c, r), tok = it.q_tok0 + tl, hq = it.kv_head * G + r - tl * G;
       const __nv_bfloat16* qrow = c.q + ((size_t)tok * c.n_q_heads + hq) * 128;
       a[u] = *reinterpret_cast<const uint4*>(qrow + ch * 8);
       b[u] = *reinterpret_cast<const uint4*>(qrow + 64 + ch * 8);
@@ -656,7 +669,7 @@ __device__ __forceinline__ void prep_q_compute(const Ctx& c, const DeviceItem& i
     }
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
+  for (int u = 0; u < U; ++u) {
     const __nv_bfloat162* a2 = reinterpret_cast<const __nv_bfloat162*>(&a[u]);
     const __nv_bfloat162* b2 = reinterpret_cast<const __nv_bfloat162*>(&b[u]);
 #pragma unroll
@@ -667,13 +680,14 @@ __device__ __forceinline__ void prep_q_compute(const Ctx& c, const DeviceItem& i
     }
   }
 }
-__device__ __forceinline__ void prep_q_store(const Ctx& c, const DeviceItem& it, uint32_t qbuf, int rank, int e0, const QUnits& qu,
+template <int NT = 128, int U = 4>
+__device__ __forceinline__ void prep_q_store(const Ctx& c, const DeviceItem& it, uint32_t qbuf, int rank, int e0, const QUnits<U>& qu,
                                              bool tile128 = false) {
-  const int G = c.n_q_heads / c.n_kv_heads;
+  const int G = c.G;
   const int M = it.n_q_tok * G, R = tile128 ? 128 : (M <= 32 ? 32 : (M <= 64 ? 64 : 128)), KS = (c.m64 && !tile128 ? 64 : 128) / R;
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int e = e0 + rank + u * 128, r = e >> 3, ch = e & 7;
+  for (int u = 0; u < U; ++u) {
+    const int e = e0 + rank + u * NT, r = e >> 3, ch = e & 7;
     if (e >= R * 8) break;
     for (int jj = 0; jj < KS; ++jj) {
       const uint32_t addr = qbuf + (jj * R + r) * 128 + ((ch ^ (r & 7)) << 4);
@@ -684,76 +698,109 @@ __device__ __forceinline__ void prep_q_store(const Ctx& c, const DeviceItem& it,
     }
   }
 }
+template <int NT = 128, int U = 4>
 __device__ __forceinline__ void prep_q(const Ctx& c, const DeviceItem& it, uint32_t qbuf, int rank, int e0 = 0) {
-  QUnits qu;
-  prep_q_compute(c, it, rank, e0, qu);
-  prep_q_store(c, it, qbuf, rank, e0, qu);
+  QUnits<U> qu;
+  prep_q_compute<NT, U>(c, it, rank, e0, qu);
+  prep_q_store<NT, U>(c, it, qbuf, rank, e0, qu);
 }
 
 // Fused step (aspd_branch_step / aspd_serial_step): the rows this step adds to pages that THIS CTA
-// reads are written into the pools at the start of the kernel, K rotated at the token's position
-// (cos/sin table of the plan) and V as is.  CTAs that read the same page write identical bytes, so
-// no cross-CTA ordering is needed.  One unit = one 16-byte chunk pair of K (8 per row) or one
-// 16-byte chunk of V (16 per row).  Called by the 128 epilogue threads; the loads of a batch of
-// units are all issued before its first store.
-__device__ __forceinline__ void append_new_rows(const Ctx& c, int rank, int d0, int n_units, const int4 (&first)[2]) {
-  for (int u0 = rank; u0 < n_units; u0 += 128 * 2) {
-    int4 d[2];
-    uint4 a[2], b[2];
+// reads are written into the pools at the start of the kernel, K rotated at the token's position (cos/sin table
+// of the plan) and V as is.  CTAs that read the same page write identical bytes, so no cross-CTA ordering is
+// needed.  STASH: the rows are also kept in shared memory, from where the producers put them into tiles that they
+// have copied without waiting for the pools' rows (patch_tile).
+// Called by the four epilogue warps while the softmax warps prepare the first query tile.  A warp takes two rows
+// at a time, lanes 0-15 the 16-byte chunks of K (with their partner chunks, half a row away), lanes 16-31 those of
+// V; all pieces of both rows are requested before the first is used.
+template <bool STASH>
+__device__ __forceinline__ void append_new_rows(const Ctx& c, uint32_t base, int warp_rank, int lane, int4 mine, int n_rows) {
+  const int ch = lane & 15;
+  const bool is_v = lane >= 16;
+#pragma unroll 1
+  for (int e0 = warp_rank; e0 < n_rows; e0 += 8) {
+    uint4 own[2], other[2];
     float4 w[2][4];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      const int u = u0 + k * 128;
-      d[k] = first[k];                                         // the first batch was fetched during set-up
-      if (u0 != rank) { d[k] = make_int4(0, 0, 0, 0); if (u < n_units) d[k] = c.pd.dirty[d0 + u / 24]; }   // (page, KV head, token, row)
+      const int e = min(e0 + 4 * k, n_rows - 1), head = __shfl_sync(0xffffffffu, mine.y, e), tok = __shfl_sync(0xffffffffu, mine.z, e);
+      const __nv_bfloat16* src = (is_v ? c.v_new : c.k_new) + ((size_t)tok * c.n_kv_heads + head) * 128;
+      own[k] = *reinterpret_cast<const uint4*>(src + ch * 8);
+      other[k] = *reinterpret_cast<const uint4*>(src + (ch ^ 8) * 8);
+      const float4* cs = reinterpret_cast<const float4*>(c.pd.q_cs + (size_t)tok * 64 + (ch & 7) * 8);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[k][i] = cs[i];
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      const int u = u0 + k * 128, sub = u % 24;
-      a[k] = make_uint4(0, 0, 0, 0); b[k] = a[k];
-      if (u >= n_units) continue;
-      const size_t src = ((size_t)d[k].z * c.n_kv_heads + d[k].y) * 128;
-      if (sub < 8) {
-        a[k] = *reinterpret_cast<const uint4*>(c.k_new + src + sub * 8);
-        b[k] = *reinterpret_cast<const uint4*>(c.k_new + src + 64 + sub * 8);
-        const float4* cs = reinterpret_cast<const float4*>(c.pd.q_cs + (size_t)d[k].z * 64 + sub * 8);
+      const int e = min(e0 + 4 * k, n_rows - 1);                 // (a row that is not there: the last one again, same bytes)
+      uint32_t r[4] = {own[k].x, own[k].y, own[k].z, own[k].w};
+      const __nv_bfloat162* a2 = reinterpret_cast<const __nv_bfloat162*>(&own[k]);
+      const __nv_bfloat162* b2 = reinterpret_cast<const __nv_bfloat162*>(&other[k]);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) w[k][i] = cs[i];
-      } else {
-        a[k] = *reinterpret_cast<const uint4*>(c.v_new + src + (sub - 8) * 8);
+      for (int i = 0; i < 4; ++i) {
+        // first half of the row: x0 cos - x1 sin; second half: x1 cos + x0 sin
+        const float2 x = __bfloat1622float2(a2[i]), y = __bfloat1622float2(b2[i]);
+        const float s0 = ch < 8 ? -w[k][i].y : w[k][i].y, s1 = ch < 8 ? -w[k][i].w : w[k][i].w;
+        if (!is_v) r[i] = pack_bf16(x.x * w[k][i].x + y.x * s0, x.y * w[k][i].z + y.y * s1);
       }
-    }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int u = u0 + k * 128, sub = u % 24;
-      if (u >= n_units || !bounds_ok(c.pd, d[k].x, d[k].w, 16)) continue;
-      const size_t tile = ((size_t)d[k].x * c.n_kv_heads + d[k].y) * 4096;
-      if (sub < 8) {
-        const __nv_bfloat162* a2 = reinterpret_cast<const __nv_bfloat162*>(&a[k]);
-        const __nv_bfloat162* b2 = reinterpret_cast<const __nv_bfloat162*>(&b[k]);
-        uint32_t lo[4], hi[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float2 x0 = __bfloat1622float2(a2[i]), x1 = __bfloat1622float2(b2[i]);
-          lo[i] = pack_bf16(x0.x * w[k][i].x - x1.x * w[k][i].y, x0.y * w[k][i].z - x1.y * w[k][i].w);
-          hi[i] = pack_bf16(x1.x * w[k][i].x + x0.x * w[k][i].y, x1.y * w[k][i].z + x0.y * w[k][i].w);
-        }
-        char* kt = const_cast<char*>(c.k_pool) + tile;
-        *reinterpret_cast<uint4*>(kt + tile_offset(d[k].w, sub * 16, 256)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-        *reinterpret_cast<uint4*>(kt + tile_offset(d[k].w, 128 + sub * 16, 256)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-      } else {
-        *reinterpret_cast<uint4*>(const_cast<char*>(c.v_pool) + tile + tile_offset(d[k].w, (sub - 8) * 16, 256)) = a[k];
-      }
+      const int page = __shfl_sync(0xffffffffu, mine.x, e), head = __shfl_sync(0xffffffffu, mine.y, e), row = __shfl_sync(0xffffffffu, mine.w, e) & 255;
+      if constexpr (STASH)
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row_stash(base, e) + lane * 16), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+      if (bounds_ok(c.pd, page, row, 16))
+        *reinterpret_cast<uint4*>(const_cast<char*>(is_v ? c.v_pool : c.k_pool) + ((size_t)page * c.n_kv_heads + head) * 4096 +
+                                  tile_offset(row, ch * 16, 256)) = make_uint4(r[0], r[1], r[2], r[3]);
     }
   }
-  asm volatile("fence.proxy.async;" ::: "memory");   // generic-proxy stores before the producers' async-proxy copies
+}
+
+// The step's new rows inside tile g of the CTA (K tile for kv = 0, V tile for 1), by the producer warp that has
+// copied the tile's pages as they were: the rows are put over what was copied, and the MMA issuer waits for the
+// slot's patch barrier before it uses such a tile.  So a page with new rows is fetched beside the append and not
+// behind it.  For plans of at most two tiles per CTA, whose time is that chain (one request of 2 k tokens, four
+// branches: 9.4 against 10.5 us a layer); with more tiles a producer that has a tile to patch gets late with its
+// next requests (32 requests, 10 tiles per CTA and more: 53.3 against 48.4 us).
+// `mine`: lane l holds dirty entry l of the CTA, which carries above its row the page's index in its tile and the
+// tile's number among the CTA's.  16 lanes take a row's 256 bytes.  The producer calls this after it has requested
+// the next tile's copies and before it waits for the slot again, so the phase it asks about is the latest.
+__device__ __forceinline__ bool patch_tile(uint32_t base, uint32_t bars, volatile int* ab, int kv, int g, int4 mine, int n_rows, int lane) {
+  static_assert(kMostFusedRows <= 32, "one entry per lane");
+  const uint32_t full_mask = 0xffffffffu, mask = __ballot_sync(full_mask, lane < n_rows && (mine.w >> 16) == g);
+  if (mask == 0) return true;
+  const int begin = __ffs(mask) - 1, end = begin + __popc(mask), sl = g & 1, ch = lane & 15;
+  if (!__all_sync(full_mask, mbar_wait(bars + 8 * A_DONE, 0, ab) && mbar_wait(bars + 8 * ((kv ? V_FULL : K_FULL) + sl), (g >> 1) & 1, ab))) return false;
+  const uint32_t tile = base + (kv ? OFF_V : OFF_K) + sl * kTileBytes;
+#pragma unroll 1
+  for (int from = begin; from < end; from += 2) {
+    const int e = from + (lane >> 4), w = __shfl_sync(full_mask, mine.w, e & 31);
+    if (e < end) {
+      uint4 x;
+      asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "r"(row_stash(base, e) + kv * 256 + ch * 16) : "memory");
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tile + ((w >> 8) & 255) * 4096 + tile_offset(w & 255, ch * 16, 256)), "r"(x.x),
+                   "r"(x.y), "r"(x.z), "r"(x.w) : "memory");
+    }
+  }
+  fence_async_smem();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(bars + 8 * ((kv ? V_PATCH : K_PATCH) + sl));
+  return true;
 }
 
 // --------------------------------------------------------------------------------- the kernel
 // WIDE: row blocks of up to 128 query rows (plans that deal whole streams to the CTAs); one
 // query tile instead of two, Misc in the place of the second.
-template <bool WIDE>
+// MODE: instances, not run-time switches, because a short launch is bound by fetching its instructions (a fifth of
+// all warp time on one request of 2 k tokens), and the code of a path that is not taken still separates the lines
+// of the one that is (145 KB with everything in one instance, 81 without the options: one request 9.6 -> 9.3 us a
+// layer, branch-open step 16.0 -> 14.7, serial step of 32 requests 45.3 -> 43.8).
+//   kPlain
+//   kOptions   what few callers ask for: scores with M = 64, records merged inside the kernel, whole streams dealt in
+//              narrow row blocks
+//   kPatch     kPlain for fused steps of plans that patch their tiles (patch_tile)
+enum { kPlain = 0, kOptions = 1, kPatch = 2 };
+template <bool WIDE, int MODE>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
+  constexpr bool OPT = MODE == kOptions, PATCH = MODE == kPatch;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -765,13 +812,18 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
   volatile int* ab = &misc->abort_flag;
   if (tid == 0) ASPD_CTA_STAMP(c, 0);
   if (tid == 0) pdl_launch_dependents();
-  const int4 head = c.pd.cta_head[blockIdx.x];
+  const int4 head = c.pd.cta_head[2 * blockIdx.x], head2 = c.pd.cta_head[2 * blockIdx.x + 1];
   const int item_begin = head.x, item_end = head.y;
   // Plan tables do not depend on earlier kernels of the stream: the CTA's items and, for the
   // producers, the first batch of page entries (whose place comes with the head entry, so that it
   // is the second load of the kernel, not the fourth) are fetched while the CTA is still setting up.
   int2 first_pages = make_int2(0, 0);
   if ((warp == W_KPROD || warp == W_VPROD) && lane < head.w) first_pages = c.pd.visit[head.z + lane];
+  // fused step: the CTA's new rows (plan data), an entry per lane of the warps that deal with them
+  const int dirty_rows = c.k_new != nullptr ? head2.y : 0;
+  const bool patch = PATCH && dirty_rows > 0;
+  int4 dirty = make_int4(0, 0, 0, -1);
+  if (warp >= W_KPROD && lane < dirty_rows) dirty = c.pd.dirty[head2.x + lane];
   {
     const int n_cached = min(item_end - item_begin, kItemCache);
     for (int e = tid; e < n_cached * (int)(sizeof(DeviceItem) / 4); e += kThreads)
@@ -784,7 +836,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
   }
 
   if (tid == 0) {
-    const int counts[NUM_BARS] = {1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 256, 256, 256, 1, 1, 1, 128, 128, 128, 128, 1, 1, 256, 256, 128};
+    const int counts[NUM_BARS] = {1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 256, 256, 256, 1, 1, 1, 128, 128, 256, 256, 1, 1, 256, 256, 1, 1, 1, 1, 128};
     for (int i = 0; i < NUM_BARS; ++i) mbar_init(bars + 8 * i, counts[i]);
     misc->abort_flag = 0;
     misc->mq_n = 0;
@@ -799,18 +851,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = misc->tmem_base;
-  // fused step: the epilogue threads fetch their first new-row entries now (plan data)
-  int dirty0 = 0, dirty_units = 0;
-  int4 dirty_first[2] = {make_int4(0, 0, 0, 0), make_int4(0, 0, 0, 0)};
-  if (warp >= W_EPI && c.k_new != nullptr) {
-    dirty0 = c.pd.cta_dirty0[blockIdx.x];
-    dirty_units = (c.pd.cta_dirty0[blockIdx.x + 1] - dirty0) * 24;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int u = (tid - W_EPI * 32) + k * 128;
-      if (u < dirty_units) dirty_first[k] = c.pd.dirty[dirty0 + u / 24];
-    }
-  }
   // everything above touches only the plan's own tables; inputs written by earlier kernels of
   // the stream (q, k_new, the pools, the workspace's previous readers) are used from here on.
   // With the plan's stable-cache promise the two producer warps go ahead and fetch pages that
@@ -821,17 +861,23 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
 
   if (warp < 8) {
     // =============================== softmax ===============================
+    // The first query tile, while the first K/V tiles are in flight and the epilogue threads write the new rows.
+    if (item_begin < item_end) {
+      prep_q<kSoftmaxThreads, WIDE ? 4 : 2>(c, misc->items[0], base + OFF_Q, tid);
+      fence_async_smem();
+      mbar_arrive(bars + 8 * Q_FULL);
+    }
     int g = 0, item_no = 0;
     for (int idx = item_begin; idx < item_end; ++idx, ++item_no) {
       const DeviceItem it = get_item(c, misc, idx, item_begin);
-      const int M = it.n_q_tok * (c.n_q_heads / c.n_kv_heads);
+      const int M = it.n_q_tok * c.G;
       bool ok;
       if constexpr (WIDE) {
         ok = M <= 32 ? softmax_item<32>(c, it, misc, bars, base + OFF_P, tmem, item_no, g)
            : M <= 64 ? softmax_item<64>(c, it, misc, bars, base + OFF_P, tmem, item_no, g)
                      : softmax_item_wide(c, it, misc, bars, base + OFF_P, tmem, item_no, g);
       } else {
-        if (c.m64)
+        if (OPT && c.m64)
           ok = M <= 32 ? softmax_item_m64<32>(c, it, misc, bars, base + OFF_P, tmem, item_no, g)
                        : softmax_item_m64<64>(c, it, misc, bars, base + OFF_P, tmem, item_no, g);
         else
@@ -850,7 +896,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
     const int kv = warp == W_KPROD ? 0 : 1;
     const char* pool = kv ? c.v_pool : c.k_pool;
     int g = 0;
-    bool ok = true, appended = false, waited = false;
+    bool ok = true, waited = false, appended = false;
     // (item, batch of 32 pages) pairs are walked as one sequence: `cur` holds the batch being
     // consumed, `nxt` the one after it, which may already belong to the next item.
     int2 nxt = first_pages;
@@ -877,15 +923,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
         if (lane >= npg) pg = make_int2(0, 0);
         if (lane < npg && !bounds_ok(c.pd, pg.x, 0, 16)) pg.x = 0;       // checking builds: flagged, page 0 read instead
         if (producer_runs_ahead && !waited && __any_sync(0xffffffffu, ((pg.y >> 8) & 31) != 0)) {
-          pdl_wait();                                  // new rows come from the previous kernel (or from this one)
+          pdl_wait();                                  // a row's neighbours may come from the previous kernel
           waited = true;
         }
-        if (c.k_new != nullptr && !appended && __any_sync(0xffffffffu, ((pg.y >> 8) & 31) != 0)) {
-          // fused append: this tile holds rows that are new this step; the append warp has written
-          // (or is writing) them -- wait for it once, before the first such page is copied
-          int okw = 1;
-          if (lane == 0) okw = mbar_wait(bars + 8 * A_DONE, 0, ab) ? 1 : 0;
-          if (!__shfl_sync(0xffffffffu, okw, 0)) { ok = false; break; }
+        if (!patch && !appended && dirty_rows > 0 && __any_sync(0xffffffffu, ((pg.y >> 8) & 31) != 0)) {
+          if (!__all_sync(0xffffffffu, mbar_wait(bars + 8 * A_DONE, 0, ab))) { ok = false; break; }
           appended = true;
         }
         const uint32_t full = bars + 8 * ((kv ? V_FULL : K_FULL) + sl), empty = bars + 8 * ((kv ? V_EMPTY : K_EMPTY) + sl);
@@ -914,8 +956,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
           bulk_copy(base + (kv ? OFF_V : OFF_K) + sl * kTileBytes + lane * 4096,
                     pool + ((size_t)pg.x * c.n_kv_heads + it.kv_head) * 4096, 4096, full);
         if (lane == 0) ASPD_STAMP(c, g, 13 + kv);
+        if (g > 0 && patch) ok = patch_tile(base, bars, ab, kv, g - 1, dirty, dirty_rows, lane);
       }
     }
+    if (ok && g > 0 && patch) patch_tile(base, bars, ab, kv, g - 1, dirty, dirty_rows, lane);
   } else if (warp == W_MMA) {
     // =================================== MMA issuer ===================================
     // The tiles of all items form one pipeline: S of tile g is issued before P.V of tile g - 1,
@@ -926,15 +970,23 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
       const uint32_t full_mask = 0xffffffffu;
       const uint32_t tmem_u = __shfl_sync(full_mask, tmem, 0);
       const uint32_t base_u = __shfl_sync(full_mask, base, 0), bars_u = base_u + off_misc;
-      struct TileRef { int npg, first, last, qb, ob, item_no; };   // qb: query tile (always 0 in the wide kernel)
+      struct TileRef { int npg, first, last, qb, ob, item_no, fresh; };   // qb: query tile (always 0 in the wide kernel); fresh:
+                                                                          // 1 + number among the slot's tiles with new rows (0: none)
       auto q_fill = [](int item_no) { return WIDE ? item_no : item_no >> 1; };   // how often the item's query tile was filled before
       auto wait_all = [&](uint32_t bar, uint32_t parity) { return __all_sync(full_mask, mbar_wait(bar, parity, ab)) != 0; };
-      const uint32_t mma_m = c.m64 ? 64u : 128u;
-      const uint32_t idesc_pv = instr_desc(128, 1, (c.m64 || c.pv64) ? 64u : 128u);
-      auto issue_s = [&](const TileRef& tr, int g) -> bool {
+      const uint32_t mma_m = OPT && c.m64 ? 64u : 128u;
+      const uint32_t idesc_pv = instr_desc(128, 1, ((OPT && c.m64) || c.pv64) ? 64u : 128u);
+      int n_fresh0 = 0, n_fresh1 = 0;              // tiles with new rows so far, in either slot
+      auto issue_s = [&](TileRef& tr, int g) -> bool {
         const int sb = g & 1;
         if (tr.first && !wait_all(bars_u + 8 * (Q_FULL + tr.qb), q_fill(tr.item_no) & 1)) return false;
         if (!wait_all(bars_u + 8 * (K_FULL + sb), (g >> 1) & 1)) return false;
+        if (patch) {                               // new rows in the tile's pages: the producers put them in
+          if (__any_sync(full_mask, lane < tr.npg && ((misc->nval[g & 3][lane & 7] >> 8) & 31) != 0)) {
+            tr.fresh = sb ? ++n_fresh1 : ++n_fresh0;
+            if (!wait_all(bars_u + 8 * (K_PATCH + sb), (tr.fresh - 1) & 1)) return false;
+          }
+        }
         if (lane == 0) ASPD_STAMP(c, g, 15);
         if (!wait_all(bars_u + 8 * (S_EMPTY + sb), ((g >> 1) & 1) ^ 1)) return false;
         tc_fence_after();
@@ -954,6 +1006,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
         if (!wait_all(bars_u + 8 * P_FULL, g & 1)) return false;
         if (lane == 0) ASPD_STAMP(c, g, 11);
         if (!wait_all(bars_u + 8 * (V_FULL + (g & 1)), (g >> 1) & 1)) return false;
+        if (tr.fresh && !wait_all(bars_u + 8 * (V_PATCH + (g & 1)), (tr.fresh - 1) & 1)) return false;
         if (tr.first && !wait_all(bars_u + 8 * (O_EMPTY + tr.ob), ((tr.item_no >> 1) & 1) ^ 1)) return false;
         tc_fence_after();
         const uint32_t pbuf = base_u + OFF_P, vbuf = base_u + OFF_V + (g & 1) * kTileBytes;
@@ -968,12 +1021,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
       };
       int g = 0, item_no = 0;
       bool ok = true, have_prev = false;
-      TileRef prev = {0, 0, 0, 0, 0, 0};
+      TileRef prev = {0, 0, 0, 0, 0, 0, 0};
       const int ib = __shfl_sync(full_mask, item_begin, 0), ie = __shfl_sync(full_mask, item_end, 0);
       for (int idx = ib; idx < ie && ok; ++idx, ++item_no) {
         const int n_pages = __shfl_sync(full_mask, get_item(c, misc, idx, ib).n_pages, 0), n_tiles = (n_pages + 7) >> 3;
         for (int t = 0; t < n_tiles && ok; ++t, ++g) {
-          const TileRef cur = {min(8, n_pages - t * 8), t == 0, t == n_tiles - 1, WIDE ? 0 : item_no & 1, item_no & 1, item_no};
+          TileRef cur = {min(8, n_pages - t * 8), t == 0, t == n_tiles - 1, WIDE ? 0 : item_no & 1, item_no & 1, item_no, 0};
           ok = issue_s(cur, g);
           if (ok && have_prev) ok = issue_pv(prev, g - 1);
           prev = cur;
@@ -988,22 +1041,23 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
     // One (m, l, O) record per query row of every item, written while the other warps are
     // already working on the next item (O and the statistics are double-buffered by item).
     const int et = tid - W_EPI * 32, ew = warp - W_EPI;   // TMEM lane quadrant = warp % 4 = ew
-    const int G = c.n_q_heads / c.n_kv_heads;
+    const int G = c.G;
     int item_no = 0;
     bool dead = false;
-    if (c.k_new != nullptr) append_new_rows(c, et, dirty0, dirty_units, dirty_first);
-    mbar_arrive(bars + 8 * A_DONE);
-    if (item_begin < item_end) {                   // the first query tile, while the first K/V tiles are in flight
-      prep_q(c, get_item(c, misc, item_begin, item_begin), base + OFF_Q, et);
-      if constexpr (WIDE) prep_q(c, get_item(c, misc, item_begin, item_begin), base + OFF_Q, et, 512);
-      fence_async_smem();
-      mbar_arrive(bars + 8 * Q_FULL);
+    if (dirty_rows > 0) {
+      append_new_rows<PATCH>(c, base, ew, lane, dirty, dirty_rows);
+      // generic-proxy stores before async-proxy copies: this launch's (unless the tiles are patched) and later ones'
+      if (patch) mbar_arrive(bars + 8 * A_DONE);
+      asm volatile("fence.proxy.async;" ::: "memory");
+      if (!patch) mbar_arrive(bars + 8 * A_DONE);
     }
+    // The softmax threads have prepared the first item's query tile.  Every fill of a query buffer is announced by
+    // 256 arrivals, as many as that first one: two for each of these threads.
     for (int idx = item_begin; idx < item_end; ++idx, ++item_no) {
       const DeviceItem it = get_item(c, misc, idx, item_begin);
-      const bool m64 = !WIDE && (c.m64 || c.pv64);  // O from an M = 64 MMA: row 16 q + i sits in lane i < 16 of quadrant q
+      const bool m64 = !WIDE && ((OPT && c.m64) || c.pv64);  // O from an M = 64 MMA: row 16 q + i sits in lane i < 16 of quadrant q
       const int ob = item_no & 1, M = it.n_q_tok * G, R = M <= 32 ? 32 : (M <= 64 ? 64 : 128),
-                KS = ((!WIDE && c.m64) ? 64 : 128) / R;                // replicas in the softmax threads' layout
+                KS = ((OPT && c.m64) ? 64 : 128) / R;                // replicas in the softmax threads' layout
       if (idx + 1 < item_end) {                    // the next item's query tile: into the other buffer, or (wide
         const int qn = WIDE ? 0 : (item_no + 1) & 1;   // kernel) into the only one once this item's last S is issued
         const int fills = WIDE ? item_no + 1 : (item_no + 1) >> 1;
@@ -1011,7 +1065,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
           // the only query tile is free once this item's last S has been issued: rotate the next
           // item's rows into registers first, so that only the stores are left for after the wait
           const DeviceItem nx = get_item(c, misc, idx + 1, item_begin);
-          QUnits q0, q1;
+          QUnits<4> q0, q1;
           prep_q_compute(c, nx, et, 0, q0);
           prep_q_compute(c, nx, et, 512, q1);
           dead |= !mbar_wait(bars + 8 * (Q_EMPTY + qn), (fills & 1) ^ 1, ab);
@@ -1022,23 +1076,23 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
           prep_q(c, get_item(c, misc, idx + 1, item_begin), base + OFF_Q + qn * kTileBytes, et);
         }
         fence_async_smem();
-        mbar_arrive(bars + 8 * (Q_FULL + qn));
+        mbar_arrive(bars + 8 * (Q_FULL + qn), 2);
       }
-      dead |= !mbar_wait(bars + 8 * (E_FULL + ob), (item_no >> 1) & 1, ab);
-      dead |= !mbar_wait(bars + 8 * (O_FULL + ob), (item_no >> 1) & 1, ab);
-      tc_fence_after();
       // where the item's result goes: a record for the merge, or -- when the item is the row's whole key
       // stream -- the normalised output itself
       // (the wide variant only serves plans that deal whole streams: always direct, never a merge)
-      const bool merging = !WIDE && c.merge_out != nullptr;
-      const bool direct = c.out != nullptr || (merging && it.n_parts == 1);
+      const bool merging = OPT && c.merge_out != nullptr;
+      const bool direct = WIDE ? c.out != nullptr : OPT && (c.out != nullptr || (merging && it.n_parts == 1));
       __nv_bfloat16* const out_base = c.out != nullptr ? c.out : c.merge_out;
+      const int r = m64 ? ((et & 31) < 16 ? ew * 16 + (et & 31) : 1 << 20) : et;   // row of O held by this thread's TMEM lane
+      int rec = 0;
+      const int tl = token_of(c, r & 255);
+      if (r < M && !direct) rec = (c.pd.part_base[(it.q_tok0 + tl) * c.n_kv_heads + it.kv_head] + it.part_slot) * G + r - tl * G;
+      dead |= !mbar_wait(bars + 8 * (E_FULL + ob), (item_no >> 1) & 1, ab);
+      dead |= !mbar_wait(bars + 8 * (O_FULL + ob), (item_no >> 1) & 1, ab);
+      tc_fence_after();
       if (ew < R / (m64 ? 16 : 32)) {
-        const int r = m64 ? ((et & 31) < 16 ? ew * 16 + (et & 31) : 1 << 20) : et;   // row of O held by this thread's TMEM lane
-        size_t rec = 0;
         if (r < M && !direct) {
-          const int tok = it.q_tok0 + r / G;
-          rec = (size_t)(c.pd.part_base[tok * c.n_kv_heads + it.kv_head] + it.part_slot) * G + r % G;
           float lt = 0.f;
           for (int jj = 0; jj < KS; ++jj) lt += misc->fin_l[ob][jj * R + r] + misc->fin_l[ob][128 + jj * R + r];
           float mr = R == 128 ? reinterpret_cast<const float*>(misc + 1)[ob * 128 + r] : misc->fin_m[ob][r];
@@ -1052,7 +1106,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
           float lt = 0.f;
           for (int jj = 0; jj < KS; ++jj) lt += misc->fin_l[ob][jj * R + r] + misc->fin_l[ob][128 + jj * R + r];
           inv_l = lt > 0.f ? 1.f / lt : 0.f;
-          orow = out_base + ((size_t)(it.q_tok0 + r / G) * c.n_q_heads + it.kv_head * G + r % G) * 128;
+          orow = out_base + ((size_t)(it.q_tok0 + tl) * c.n_q_heads + it.kv_head * G + r - tl * G) * 128;
         }
 #pragma unroll 1
         for (int q4 = 0; q4 < 4; ++q4) {
@@ -1068,7 +1122,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
                                     pack_bf16(o[8 * i + 4] * inv_l, o[8 * i + 5] * inv_l), pack_bf16(o[8 * i + 6] * inv_l, o[8 * i + 7] * inv_l));
             }
           } else if (r < M && !dead) {
-            float4* dst = reinterpret_cast<float4*>(c.pd.ws_o + rec * 128 + q4 * 32);
+            float4* dst = reinterpret_cast<float4*>(c.pd.ws_o + (size_t)rec * 128 + q4 * 32);
 #pragma unroll
             for (int i = 0; i < 8; ++i) dst[i] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
           }
@@ -1119,7 +1173,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
   }
   // single-launch plans: the pairs whose last record this CTA stored are merged now, by all warps
-  if (!WIDE && c.merge_out != nullptr && !*ab) drain_merge_queue(c, misc, warp, kThreads / 32, lane);
+  if (OPT && c.merge_out != nullptr && !*ab) drain_merge_queue(c, misc, warp, kThreads / 32, lane);
   if (tid == 0) ASPD_CTA_STAMP(c, 7);
 }
 
@@ -1173,9 +1227,11 @@ static int launch_tc(const aspd_plan* p, const void* q, const void* k_new, const
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return ASPD_ERR_CUDA;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    if (cudaFuncSetAttribute(attn_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(attn_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(attn_tc_w2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytesW2) != cudaSuccess)
+    auto attr = [](auto* kernel, size_t bytes) {
+      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+    };
+    if (!attr(attn_tc_kernel<false, kPlain>, kSmemBytes) || !attr(attn_tc_kernel<false, kOptions>, kSmemBytes) ||
+        !attr(attn_tc_kernel<false, kPatch>, kSmemBytes) || !attr(attn_tc_kernel<true, kPlain>, kSmemBytes) || !attr(attn_tc_w2_kernel, kSmemBytesW2))
       return ASPD_ERR_CUDA;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
@@ -1195,6 +1251,8 @@ static int launch_tc(const aspd_plan* p, const void* q, const void* k_new, const
   c.n_items = p->n_items;
   c.n_q_heads = sh.n_q_heads;
   c.n_kv_heads = sh.n_kv_heads;
+  c.G = sh.n_q_heads / sh.n_kv_heads;
+  c.inv_g = (65536 + c.G - 1) / c.G;
   c.scale_log2 = sh.sm_scale * kLog2e;
   c.early_fetch = p->stable_cache;
   c.stagger_start = p->stagger_start;
@@ -1207,8 +1265,10 @@ static int launch_tc(const aspd_plan* p, const void* q, const void* k_new, const
     c.k_new = nullptr; c.v_new = nullptr;
     return launch_pdl(kPdlAttn, attn_tc_w2_kernel, dim3(p->n_ctas), dim3(kThreads), kSmemBytesW2, s, c) == cudaSuccess ? ASPD_OK : ASPD_ERR_CUDA;
   }
-  const cudaError_t e = p->wide ? launch_pdl(kPdlAttn, attn_tc_kernel<true>, dim3(p->n_ctas), dim3(kThreads), kSmemBytes, s, c)
-                                : launch_pdl(kPdlAttn, attn_tc_kernel<false>, dim3(p->n_ctas), dim3(kThreads), kSmemBytes, s, c);
+  auto* kernel = p->wide ? attn_tc_kernel<true, kPlain>
+                 : c.m64 || c.merge_out != nullptr || c.out != nullptr ? attn_tc_kernel<false, kOptions>
+                 : c.k_new != nullptr && p->patch_tiles ? attn_tc_kernel<false, kPatch> : attn_tc_kernel<false, kPlain>;
+  const cudaError_t e = launch_pdl(kPdlAttn, kernel, dim3(p->n_ctas), dim3(kThreads), kSmemBytes, s, c);
   return e == cudaSuccess ? ASPD_OK : ASPD_ERR_CUDA;
 }
 

@@ -65,7 +65,7 @@ __device__ __forceinline__ DeviceItem get_item_w2(const Ctx& c, const MiscW2* mi
 __device__ __forceinline__ void softmax_group_w2(const Ctx& c, MiscW2* misc, uint32_t bars, uint32_t base, uint32_t tmem, int item_begin,
                                                  int item_end, int grp, int tpt) {
   const int tid = threadIdx.x, warp = tid >> 5, r = tid & 127;
-  const int G = c.n_q_heads / c.n_kv_heads;
+  const int G = c.G;
   volatile int* ab = &misc->abort_flag;
   const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
   const uint32_t s_base = tmem + lane_addr + COL_S + grp * 128, o_base = tmem + lane_addr + COL_O + grp * 128;
@@ -80,7 +80,7 @@ __device__ __forceinline__ void softmax_group_w2(const Ctx& c, MiscW2* misc, uin
     const int n_tiles = (it.n_pages + 7) >> 3;
     const int n_tok = min(tpt, it.n_q_tok - grp * tpt);
     if (n_tok <= 0) { g += n_tiles; continue; }                // the block has no second tile
-    const int M = n_tok * G, tok = it.q_tok0 + grp * tpt + r / G;
+    const int tl = token_of(c, r), M = n_tok * G, tok = it.q_tok0 + grp * tpt + tl;
     int4 vis = make_int4(0, 0, 0, 0);                          // padding rows see nothing
     if (r < M) vis = c.pd.tok_vis[tok];
     float m_ref = 0.f, l = 0.f;                                 // see the one-tile variant: the reference starts at 0
@@ -240,7 +240,7 @@ __device__ __forceinline__ void softmax_group_w2(const Ctx& c, MiscW2* misc, uin
     ++ic;
     {
       const float inv_l = l > 0.f ? 1.f / l : 0.f;
-      __nv_bfloat16* orow = c.out + ((size_t)tok * c.n_q_heads + it.kv_head * G + r % G) * 128;
+      __nv_bfloat16* orow = c.out + ((size_t)tok * c.n_q_heads + it.kv_head * G + r - tl * G) * 128;
 #pragma unroll 1
       for (int q4 = 0; q4 < 4; ++q4) {
         float o[32];
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_w2_kernel(Ctx c) {
   volatile int* ab = &misc->abort_flag;
   if (tid == 0) ASPD_CTA_STAMP(c, 0);
   if (tid == 0) pdl_launch_dependents();
-  const int4 head = c.pd.cta_head[blockIdx.x];
+  const int4 head = c.pd.cta_head[2 * blockIdx.x];
   const int item_begin = head.x, item_end = head.y;
   int2 first_pages = make_int2(0, 0);
   if ((warp == W_KPROD || warp == W_VPROD) && lane < head.w) first_pages = c.pd.visit[head.z + lane];
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_w2_kernel(Ctx c) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = misc->tmem_base;
-  const int G = c.n_q_heads / c.n_kv_heads, tpt = 128 / G;      // tokens per query tile
+  const int G = c.G, tpt = 128 / G;      // tokens per query tile
   // inputs written by earlier kernels of the stream are used from here on; with the plan's
   // stable-cache promise the producers go ahead (such plans never carry new rows in their pages'
   // entries only when the step was appended by an earlier kernel: they wait before the first such page)
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_w2_kernel(Ctx c) {
         if (sub.n_q_tok <= 0) break;
 #pragma unroll 1
         for (int e0 = 0; e0 < 1024; e0 += 512) {
-          QUnits qu;
+          QUnits<4> qu;
           prep_q_compute(c, sub, et, e0, qu, true);
           if (!waited_q) {      // the tiles are free once the previous item's last scores have been issued
             dead |= !mbar_wait(bars + 8 * WQ_EMPTY, (item_no & 1) ^ 1, ab);

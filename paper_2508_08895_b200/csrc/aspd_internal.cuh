@@ -13,6 +13,7 @@ namespace aspd {
 
 constexpr int kMaxRowsPerItem = 64;   // query rows (tokens x group heads) one work item carries
 constexpr int kMaxRowsWide = 128;     // ... in a plan that deals whole streams to the tensor-core kernel's CTAs
+constexpr int kMostFusedRows = 20;   // new rows per CTA up to which the attention pass writes them itself
 constexpr int kCausalAll = 1 << 29;   // prefix end of a token that sees its whole key stream
 
 // ---------------------------------------------------------------------------------------
@@ -41,12 +42,13 @@ struct DeviceItem {       // mirrors aspd_item_t, 40 bytes
 
 struct PlanDevice {       // pointers into the plan's single device allocation
   const DeviceItem* items;
-  const int4* cta_head;        // [n_ctas] (first item, end item, page0 and n_pages of the first item): everything a CTA
-                               // needs to request its first pages comes with one load
+  const int4* cta_head;        // [n_ctas][2] (first item, end item, page0 and n_pages of the first item) and (first entry of
+                               // `dirty`, number of entries, -, -): everything a CTA needs to request its first pages
+                               // and rows comes with one line
   const int2* visit;           // key streams, per page to read: (physical page, valid rows | new rows << 8 |
                                // first new token << 13); the new rows are the last valid rows of the page
-  const int32_t* cta_dirty0;   // [n_ctas + 1] range of `dirty` that CTA c must write before reading (fused step)
-  const int4* dirty;           // (physical page, KV head, new token, row) of every new row in a CTA's pages
+  const int4* dirty;           // of every new row in a CTA's pages: (physical page, KV head, new token, row | index of the page
+                               // in its 128-key tile << 8 | number of the tile among the CTA's << 16)
   const int4* tok_vis;         // [n_new] (pe, lo, hi, -): visible stream keys are [0, pe) and [lo, hi)
   const int2* row_blocks;      // [n_row_blocks] (first new token, number of tokens)
   const int32_t* tok_page;     // [n_new] physical page the new token's K/V goes to
@@ -86,7 +88,7 @@ namespace aspd {
 // Byte offsets of the plan's tables inside its device block, and how many entries the
 // length-dependent ones have room for.
 struct PlanLayout {
-  size_t o_items = 0, o_cta = 0, o_visit = 0, o_cdirty = 0, o_dirty = 0, o_tpage = 0, o_trow = 0, o_tpos = 0, o_tvis = 0,
+  size_t o_items = 0, o_cta = 0, o_visit = 0, o_dirty = 0, o_tpage = 0, o_trow = 0, o_tpos = 0, o_tvis = 0,
          o_rb = 0, o_pbase = 0, o_freq = 0, o_status = 0, o_arrive = 0, upload_bytes = 0, cleared_end = 0, o_qcs = 0, o_wso = 0, o_wsml = 0, o_stq = 0,
          o_stk = 0, o_stv = 0, o_sto = 0, o_stp = 0, device_bytes = 0;
   size_t cap_items = 0, cap_visit = 0, cap_dirty = 0, cap_partials = 0, n_row_blocks = 0, n_part_base = 0;
@@ -126,6 +128,7 @@ struct aspd_plan {
   int dec = 0;                     // tensor-core plan of a shape that aspd_attn_dec.cu serves (head_dim 64, pages of 8 or 32)
   int max_rows = 0;                // largest number of query rows of an item
   int stagger_start = 0;           // few tiles per CTA: order the requests of a CTA's first tiles (see the producers)
+  int patch_tiles = 0;             // at most two tiles per CTA: a fused step puts the new rows into the tiles (see patch_tile)
   int single_launch = 0;           // stream-K plan of the tensor-core kernel whose last-arriving CTAs merge the records themselves
   int64_t n_pool_pages = 0;
   int64_t kv_tokens_read = 0;
@@ -205,7 +208,8 @@ int launch_read_token(const aspd_shape_t* shape, const void* pool, int64_t page,
 inline void fill_cta_head(const aspd_plan* p, int4* dst) {
   for (int c = 0; c < p->n_ctas; ++c) {
     const int b = p->cta_item0[c], e = p->cta_item0[c + 1];
-    dst[c] = make_int4(b, e, b < e ? p->items[b].page0 : 0, b < e ? p->items[b].n_pages : 0);
+    dst[2 * c] = make_int4(b, e, b < e ? p->items[b].page0 : 0, b < e ? p->items[b].n_pages : 0);
+    dst[2 * c + 1] = make_int4(p->cta_dirty0[c], p->cta_dirty0[c + 1] - p->cta_dirty0[c], 0, 0);
   }
 }
 inline int esize_of(int dtype) { return dtype == ASPD_DTYPE_BF16 ? 2 : 4; }

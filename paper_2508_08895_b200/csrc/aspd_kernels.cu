@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(kGenThreads, 2) attn_generic_kernel(PlanDevice
   extern __shared__ __align__(1024) uint8_t gen_smem[];
   GenSmem<T, D>& sm = *reinterpret_cast<GenSmem<T, D>*>(gen_smem);
   pdl_launch_dependents();
-  const int4 head = pd.cta_head[blockIdx.x];
+  const int4 head = pd.cta_head[2 * blockIdx.x];
   DeviceItem it = {};
   if (head.x < head.y) it = pd.items[head.x];
   pdl_wait();

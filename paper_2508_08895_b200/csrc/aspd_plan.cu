@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <chrono>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -65,8 +66,15 @@ int block_acquire(size_t bytes, size_t host_need, cudaStream_t s, PlanBlock* out
       if (oldest < 0) oldest = i;
       if ((best < 0 || g_blocks[i].bytes < g_blocks[best].bytes) && cudaEventQuery(g_blocks[i].upload_done) == cudaSuccess) best = i;
     }
-    // every fitting block still has its copy queued: with a couple of them parked the host is simply
-    // ahead of the GPU and waits for the oldest one instead of allocating more
+    // Every fitting block still has its copy queued.  A new block (device and page-locked memory) takes the host the
+    // better part of a millisecond, so a copy that is about to finish is waited for first; and with a couple of
+    // blocks parked the host is simply ahead of the GPU and waits for the oldest one instead of allocating more.
+    if (best < 0 && fitting == 1) {
+      const auto until = std::chrono::steady_clock::now() + std::chrono::microseconds(300);
+      do {
+        if (cudaEventQuery(g_blocks[oldest].upload_done) == cudaSuccess) best = oldest;
+      } while (best < 0 && std::chrono::steady_clock::now() < until);
+    }
     if (best < 0 && fitting >= 2 && cudaEventSynchronize(g_blocks[oldest].upload_done) == cudaSuccess) best = oldest;
     if (best >= 0) {
       PlanBlock b;
@@ -659,7 +667,6 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   // writes them in batches at the start of the kernel; with many new rows per CTA (a branch-open step) the
   // separate append kernel is the faster way, and such plans carry no list.  (The few pages that hold new rows
   // are found once, not once per KV head and CTA.)
-  constexpr int kMostFused = 20;
   std::vector<int4> dirty;
   std::vector<int32_t> cta_dirty0(n_ctas + 1, 0);
   p->fuse_append = (kernel == ASPD_KERNEL_MMA && !shared_mask && tok_field_fits && p->wide != 2) ? 1 : 0;
@@ -669,15 +676,20 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
       if ((visit[i].y >> 8) & 31) fresh.push_back((int)i);
     for (int c = 0; c < n_ctas && p->fuse_append; ++c) {
       cta_dirty0[c] = (int)dirty.size();
+      const int ppt = 128 / ps;                    // pages of a tile
+      int tile0 = 0;                               // number of the item's first tile among the CTA's
       for (int i = cta_item0[c]; i < cta_item0[c + 1]; ++i) {
         const DeviceItem& it = p->items[i];
         for (auto e = std::lower_bound(fresh.begin(), fresh.end(), it.page0); e != fresh.end() && *e < it.page0 + it.n_pages; ++e) {
           const int2 v = visit[*e];
           const int cnt = (v.y >> 8) & 31, tok0 = v.y >> 13, row0 = (v.y & 255) - cnt;
-          for (int k = 0; k < cnt; ++k) dirty.push_back(make_int4(v.x, it.kv_head, tok0 + k, row0 + k));
+          const int pg = *e - it.page0, place = (pg % ppt) << 8 | (tile0 + pg / ppt) << 16;
+          for (int k = 0; k < cnt; ++k) dirty.push_back(make_int4(v.x, it.kv_head, tok0 + k, (row0 + k) | place));
         }
+        tile0 += (it.n_pages + ppt - 1) / ppt;
       }
-      if ((int)dirty.size() - cta_dirty0[c] > kMostFused) p->fuse_append = 0;
+      // (32 767 tiles: what the number's field holds)
+      if ((int)dirty.size() - cta_dirty0[c] > kMostFusedRows || tile0 > 32767) p->fuse_append = 0;
     }
     cta_dirty0[n_ctas] = (int)dirty.size();
     if (!p->fuse_append) { dirty.clear(); std::fill(cta_dirty0.begin(), cta_dirty0.end(), 0); }
@@ -688,12 +700,13 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   // down, stays as it is); 0: both with M = 128
   p->m64 = (kernel == ASPD_KERNEL_MMA && !deal_streams && !p->dec) ? (tune.mma_m == 64 ? 1 : tune.mma_m == 128 ? 0 : 2) : 0;
   p->stagger_start = (!deal_streams && total_pages <= 6L * 8 * n_ctas) ? 1 : 0;       // at most six 128-key tiles per CTA
+  p->patch_tiles = (!deal_streams && total_pages <= 2L * 8 * n_ctas) ? 1 : 0;
   // Merging inside the attention kernel is an option, not the default.  Measured on every workload of
   // the benchmark, the CTA that stores a pair's last record is a CTA at the very end of its own work,
   // so its fence, count and merge (1.5 us + one memory round trip per 16 rows of the pairs it ended
   // up with; all rows of a stream cut into dozens of parts land on one CTA) lengthen the kernel by
   // more than the combine launch costs, whose blocks are resident and waiting when the pass ends.
-  p->single_launch = (kernel == ASPD_KERNEL_MMA && !deal_streams && !p->dec && tune.combine == ASPD_COMBINE_FUSED) ? 1 : 0;
+  p->single_launch = (kernel == ASPD_KERNEL_MMA && !deal_streams && !p->dec && tune.combine == ASPD_COMBINE_FUSED && max_tok <= 16) ? 1 : 0;   // 16: an item's tokens in the merge queue
   for (size_t i = 0; i < n_parts.size(); ++i) part_base[i + 1] = part_base[i] + n_parts[i];
   p->n_items = (int)p->items.size();
   p->n_partials = part_base[n_parts.size()];
@@ -728,9 +741,8 @@ static void plan_layout(const aspd_plan* p, double slack, aspd::PlanLayout* L) {
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   L->o_items = take(sizeof(DeviceItem) * L->cap_items);
-  L->o_cta = take(sizeof(int4) * std::max(1, p->n_ctas));
+  L->o_cta = take(2 * sizeof(int4) * std::max(1, p->n_ctas));
   L->o_visit = take(sizeof(int2) * L->cap_visit);
-  L->o_cdirty = take(sizeof(int32_t) * (p->n_ctas + 1));
   L->o_dirty = take(sizeof(int4) * L->cap_dirty);
   L->o_tpage = take(sizeof(int32_t) * std::max(1, n_new));
   L->o_trow = take(sizeof(int32_t) * std::max(1, n_new));
@@ -761,12 +773,11 @@ static void plan_layout(const aspd_plan* p, double slack, aspd::PlanLayout* L) {
 // the cos/sin table there.  The caller has made sure that the buffer's previous copy has completed.
 static int plan_upload(aspd_plan* p, cudaStream_t s, bool clear) {
   const aspd::PlanLayout& L = p->layout;
-  const int n_new = p->n_new, d = p->shape.head_dim, n_ctas = p->n_ctas;
+  const int n_new = p->n_new, d = p->shape.head_dim;
   uint8_t* blob = static_cast<uint8_t*>(p->block.host);
   if (!p->items.empty()) memcpy(blob + L.o_items, p->items.data(), sizeof(DeviceItem) * p->items.size());
   fill_cta_head(p, reinterpret_cast<int4*>(blob + L.o_cta));
   if (!p->visit.empty()) memcpy(blob + L.o_visit, p->visit.data(), sizeof(int2) * p->visit.size());
-  memcpy(blob + L.o_cdirty, p->cta_dirty0.data(), sizeof(int32_t) * (n_ctas + 1));
   if (!p->dirty.empty()) memcpy(blob + L.o_dirty, p->dirty.data(), sizeof(int4) * p->dirty.size());
   if (n_new) {
     memcpy(blob + L.o_tpage, p->tok_page.data(), sizeof(int32_t) * n_new);
@@ -801,7 +812,6 @@ static int plan_to_device(aspd_plan* p, cudaStream_t s) {
   p->dev.items = (const DeviceItem*)(b8 + L.o_items);
   p->dev.cta_head = (const int4*)(b8 + L.o_cta);
   p->dev.visit = (const int2*)(b8 + L.o_visit);
-  p->dev.cta_dirty0 = (const int32_t*)(b8 + L.o_cdirty);
   p->dev.dirty = (const int4*)(b8 + L.o_dirty);
   p->dev.tok_vis = (const int4*)(b8 + L.o_tvis);
   p->dev.row_blocks = (const int2*)(b8 + L.o_rb);

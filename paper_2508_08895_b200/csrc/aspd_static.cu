@@ -60,7 +60,7 @@ extern "C" int aspd_attn_static(const aspd_plan_t* plan, const void* q, const vo
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   const size_t o_items = take(sizeof(DeviceItem) * plan->items.size());
-  const size_t o_cta = take(sizeof(int4) * (size_t)(plan->n_ctas > 0 ? plan->n_ctas : 1));
+  const size_t o_cta = take(2 * sizeof(int4) * (size_t)(plan->n_ctas > 0 ? plan->n_ctas : 1));
   const size_t o_visit = take(sizeof(int2) * plan->visit.size());
   const size_t o_tvis = take(sizeof(int4) * plan->tok_vis.size());
   const size_t o_rb = take(sizeof(int2) * plan->row_blocks.size());
