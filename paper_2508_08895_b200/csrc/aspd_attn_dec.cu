@@ -256,7 +256,6 @@ __device__ __forceinline__ void prep_q(const Ctx& c, const DeviceItem& it, uint3
   }
   fence_async_smem();
 }
-__host__ __device__ inline int padded_rows(int m) { return m <= 16 ? 16 : m <= 32 ? 32 : 64; }
 // One arrival per warp: what its lanes wrote before is ordered by the warp barrier.
 __device__ __forceinline__ void warp_arrive(uint32_t bar, int lane) {
   __syncwarp();
@@ -439,7 +438,9 @@ __device__ __forceinline__ void finish_item(const Ctx& c, const DeviceItem& it, 
 }
 
 // -------------------------------------------------------------------------------------------- the kernel
-template <int D>
+// NR: rows that the plan's largest row block is padded to; its smaller blocks are padded as far.  (One instance that
+// chose per item was 161 KB of code, and a short launch waits for its instructions: FIGURE)
+template <int D, int NR>
 __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
@@ -484,7 +485,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
     int g = 0, item_no = 0;
     // the item's query tile, its tokens' ranges and where its rows go
     auto start_item = [&](const DeviceItem& it, int par) {
-      const int m = it.n_q_tok * G, nr = padded_rows(m);
+      const int m = it.n_q_tok * G;
       int4 vis = make_int4(0, 0, 0, 0);
       int row_out = 0;
       if (tid < it.n_q_tok) vis = c.pd.tok_vis[it.q_tok0 + tid];
@@ -493,9 +494,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
         row_out = c.out != nullptr ? tok * c.n_q_heads + it.kv_head * G + tid % G
                                    : (c.pd.part_base[tok * c.n_kv_heads + it.kv_head] + it.part_slot) * G + tid % G;
       }
-      if (nr == 16) prep_q<D, 16>(c, it, base + c.off_q, tid);
-      else if (nr == 32) prep_q<D, 32>(c, it, base + c.off_q, tid);
-      else prep_q<D, 64>(c, it, base + c.off_q, tid);
+      prep_q<D, NR>(c, it, base + c.off_q, tid);
       if (tid < it.n_q_tok) misc->vis[par][tid] = vis;
       if (tid < m) misc->row_out[par][tid] = row_out;
       warp_arrive(bars + 8 * Q_FULL, lane);
@@ -503,24 +502,18 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
     if (item_begin < item_end) start_item(first, 0);
     for (int idx = item_begin; idx < item_end; ++idx, ++item_no) {
       const DeviceItem it = idx == item_begin ? first : c.pd.items[idx];
-      const int nr = padded_rows(it.n_q_tok * G), par = item_no & 1;
+      const int par = item_no & 1;
       named_sync(1, kSmThreads);                                  // the item's ranges are there
-      auto whole_item = [&](auto tag) {
-        constexpr int NR = decltype(tag)::value;
-        dead |= !softmax_item<D, NR>(c, it, misc, bars, base + c.off_p, tmem, par, g);
-        if (idx + 1 < item_end) {                                 // the next query tile as soon as this item's last scores are issued
-          dead |= !mbar_wait(bars + 8 * Q_EMPTY, item_no & 1, ab);
-          start_item(c.pd.items[idx + 1], par ^ 1);
-        }
-        dead |= !mbar_wait(bars + 8 * O_FULL, item_no & 1, ab);
-        tc_fence_after();
-        named_sync(1, kSmThreads);                                // the row sums of all quadrants
-        finish_item<D, NR>(c, it, misc, tmem, par, dead || *ab);
-        tc_fence_before();
-      };
-      if (nr == 16) whole_item(std::integral_constant<int, 16>());
-      else if (nr == 32) whole_item(std::integral_constant<int, 32>());
-      else whole_item(std::integral_constant<int, 64>());
+      dead |= !softmax_item<D, NR>(c, it, misc, bars, base + c.off_p, tmem, par, g);
+      if (idx + 1 < item_end) {                                   // the next query tile as soon as this item's last scores are issued
+        dead |= !mbar_wait(bars + 8 * Q_EMPTY, item_no & 1, ab);
+        start_item(c.pd.items[idx + 1], par ^ 1);
+      }
+      dead |= !mbar_wait(bars + 8 * O_FULL, item_no & 1, ab);
+      tc_fence_after();
+      named_sync(1, kSmThreads);                                  // the row sums of all quadrants
+      finish_item<D, NR>(c, it, misc, tmem, par, dead || *ab);
+      tc_fence_before();
       if (named_sync_or(1, kSmThreads, dead || *ab)) break;
     }
   } else if (producer) {
@@ -595,7 +588,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
     int g = 0, item_no = 0;
     bool ok = true;
     for (int idx = ib; idx < ie && ok; ++idx, ++item_no) {
-      const int n_pages = __shfl_sync(fm, c.pd.items[idx].n_pages, 0), nr = padded_rows(__shfl_sync(fm, c.pd.items[idx].n_q_tok, 0) * G);
+      const int n_pages = __shfl_sync(fm, c.pd.items[idx].n_pages, 0);
       const int n_tiles = (n_pages + ppt - 1) / ppt;
       for (int t = 0; t < n_tiles && ok; ++t, ++g) {
         if (warp == W_S) {
@@ -605,11 +598,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
           if (!ok) break;
           tc_fence_after();
           const uint64_t a = smem_desc(base_u + sl * kTileBytes, 16, kRowGroup), b = smem_desc(base_u + c.off_q, 16, 1024);
-          const uint32_t idesc = instr_desc((uint32_t)nr, 0), d = tmem_u + COL_S + sb * 64;
+          const uint32_t idesc = instr_desc(NR, 0), d = tmem_u + COL_S + sb * 64;
 #pragma unroll
-          for (int pc = 0; pc < kPieces; ++pc) {                 // the queries' pieces lie nr * D * 2 bytes apart
-            tc_mma_k64_lane0(d, a, b + pc * (nr * D / 8), idesc, pc);
-            if constexpr (D == 128) tc_mma_k64_lane0(d, a + 64, b + pc * (nr * D / 8) + nr * 8, idesc, 1);   // second span: 1024 B further in K, nr * 128 B in Q
+          for (int pc = 0; pc < kPieces; ++pc) {                 // the queries' pieces lie NR * D * 2 bytes apart
+            tc_mma_k64_lane0(d, a, b + pc * (NR * D / 8), idesc, pc);
+            if constexpr (D == 128) tc_mma_k64_lane0(d, a + 64, b + pc * (NR * D / 8) + NR * 8, idesc, 1);   // second span: 1024 B further in K, NR * 128 B in Q
           }
           tc_commit_lane0(bars_u + 8 * (S_FULL + sb));
           tc_commit_lane0(bars_u + 8 * (K_EMPTY + sl));
@@ -621,12 +614,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
           if (!ok) break;
           tc_fence_after();
           const uint64_t a = smem_desc(base_u + c.off_v + sl * kTileBytes, 1024, kRowGroup);
-          const uint64_t b = nr == 64 ? p_desc<64>(base_u + c.off_p) : nr == 32 ? p_desc<32>(base_u + c.off_p) : p_desc<16>(base_u + c.off_p);
+          const uint64_t b = p_desc<NR>(base_u + c.off_p);
           // both operands MN-major; 16 keys are two groups of 8 in either
-          const uint32_t idesc = instr_desc((uint32_t)nr, 1, D) | (1u << 15);
+          const uint32_t idesc = instr_desc(NR, 1, D) | (1u << 15);
 #pragma unroll
           for (int pc = 0; pc < kPieces; ++pc)
-            tc_mma_keys_lane0(tmem_u + COL_O, a, b + pc * (kTile * nr / 8), 2 * kRowGroup >> 4, nr * 2, idesc, t > 0 || pc > 0 ? 1u : 0u, steps);
+            tc_mma_keys_lane0(tmem_u + COL_O, a, b + pc * (kTile * NR / 8), 2 * kRowGroup >> 4, NR * 2, idesc, t > 0 || pc > 0 ? 1u : 0u, steps);
           tc_commit_lane0(bars_u + 8 * P_EMPTY);
           tc_commit_lane0(bars_u + 8 * (V_EMPTY + sl));
           if (t == n_tiles - 1) tc_commit_lane0(bars_u + 8 * O_FULL);
@@ -666,18 +659,19 @@ inline uint32_t smem_layout(int D, int nr, Ctx* c) {
   return c->off_misc + (uint32_t)sizeof(DecMisc) + 1024;
 }
 
-template <int D>
-cudaError_t launch(const aspd_plan* p, const Ctx& c, uint32_t smem, cudaStream_t s) {
+template <int D, int NR>
+cudaError_t launch(const aspd_plan* p, Ctx& c, cudaStream_t s) {
   static bool configured[64] = {};                 // the attribute belongs to the (function, device) pair
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    e = cudaFuncSetAttribute(attn_dec_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    e = cudaFuncSetAttribute(attn_dec_kernel<D, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
-  return launch_pdl(kPdlAttn, attn_dec_kernel<D>, dim3(p->n_ctas), dim3(kThreads), smem, s, c);
+  const uint32_t smem = smem_layout(D, NR, &c);
+  return launch_pdl(kPdlAttn, attn_dec_kernel<D, NR>, dim3(p->n_ctas), dim3(kThreads), smem, s, c);
 }
 
 }  // namespace
@@ -695,8 +689,9 @@ int launch_attn_dec(const aspd_plan* p, const void* q, const void* k_new, const 
   c.n_q_heads = sh.n_q_heads; c.n_kv_heads = sh.n_kv_heads; c.page_size = sh.page_size;
   c.scale_log2 = sh.sm_scale * kLog2e;
   c.early_fetch = p->stable_cache;
-  const uint32_t smem = smem_layout(sh.head_dim, padded_rows(p->max_rows), &c);
-  const cudaError_t e = sh.head_dim == 64 ? launch<64>(p, c, smem, s) : launch<128>(p, c, smem, s);
+  const int nr = padded_rows(p->max_rows);
+  const cudaError_t e = sh.head_dim == 64 ? (nr == 16 ? launch<64, 16>(p, c, s) : nr == 32 ? launch<64, 32>(p, c, s) : launch<64, 64>(p, c, s))
+                                          : (nr == 16 ? launch<128, 16>(p, c, s) : nr == 32 ? launch<128, 32>(p, c, s) : launch<128, 64>(p, c, s));
   return e == cudaSuccess ? ASPD_OK : ASPD_ERR_CUDA;
 }
 

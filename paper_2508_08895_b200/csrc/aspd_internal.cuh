@@ -185,6 +185,7 @@ int launch_attn_generic(const aspd_plan* p, const void* q, const void* k_pool, c
 // kernel itself when the plan has one item per (token, KV head) (ignored otherwise)
 int launch_attn_mma(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool, void* out,
                     cudaStream_t s);
+inline int padded_rows(int m) { return m <= 16 ? 16 : m <= 32 ? 32 : 64; }   // N of that kernel's MMAs
 // the same for plans with p->dec; k_new / v_new non-null: the step's new rows are written first
 int launch_attn_dec(const aspd_plan* p, const void* q, const void* k_new, const void* v_new, const void* k_pool, const void* v_pool,
                     void* out, cudaStream_t s);

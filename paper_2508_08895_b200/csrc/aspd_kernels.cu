@@ -425,7 +425,9 @@ __device__ __forceinline__ void generic_item(const PlanDevice& pd, const DeviceI
   }
 }
 
-template <typename T, int D>
+// (RPW for the plan's largest row block: an instance that chose per item was 65 to 79 KB of code, and a short launch
+// waits for its instructions.)
+template <typename T, int D, int RPW>
 __global__ void __launch_bounds__(kGenThreads, 2) attn_generic_kernel(PlanDevice pd, const T* __restrict__ q, const T* __restrict__ k_pool,
                                                                       const T* __restrict__ v_pool, int n_q_heads, int n_kv_heads,
                                                                       int page_size, float scale_log2) {
@@ -438,13 +440,7 @@ __global__ void __launch_bounds__(kGenThreads, 2) attn_generic_kernel(PlanDevice
   pdl_wait();
   for (int idx = head.x; idx < head.y; ++idx) {
     if (idx > head.x) it = pd.items[idx];
-    const int rows = it.n_q_tok * (n_q_heads / n_kv_heads);
-#define ASPD_GEN_ITEM(RPW) generic_item<T, D, RPW>(pd, it, sm, q, k_pool, v_pool, n_q_heads, n_kv_heads, page_size, scale_log2)
-    if (rows <= 8) ASPD_GEN_ITEM(1);
-    else if (rows <= 16) ASPD_GEN_ITEM(2);
-    else if (rows <= 32) ASPD_GEN_ITEM(4);
-    else ASPD_GEN_ITEM(8);
-#undef ASPD_GEN_ITEM
+    generic_item<T, D, RPW>(pd, it, sm, q, k_pool, v_pool, n_q_heads, n_kv_heads, page_size, scale_log2);
   }
 }
 
@@ -492,19 +488,25 @@ int launch_append(const aspd_plan* p, const void* k_new, const void* v_new, cons
                               sh.n_kv_heads, sh.head_dim, sh.page_size, p->dev));
 }
 
-template <typename T, int D>
-static int launch_generic(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool, cudaStream_t s) {
+template <typename T, int D, int RPW>
+static int launch_generic_rows(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool, cudaStream_t s) {
   static bool configured[64] = {};                 // the attribute belongs to the (function, device) pair
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return ASPD_ERR_CUDA;
   if (dev < 0 || dev >= 64 || !configured[dev]) {
-    if (cudaFuncSetAttribute(attn_generic_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GenSmem<T, D>)) != cudaSuccess)
+    if (cudaFuncSetAttribute(attn_generic_kernel<T, D, RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GenSmem<T, D>)) != cudaSuccess)
       return ASPD_ERR_CUDA;
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   const aspd_shape_t& sh = p->shape;
-  return status_of(launch_pdl(kPdlAttn, attn_generic_kernel<T, D>, dim3(p->n_ctas), dim3(kGenThreads), sizeof(GenSmem<T, D>), s, p->dev,
+  return status_of(launch_pdl(kPdlAttn, attn_generic_kernel<T, D, RPW>, dim3(p->n_ctas), dim3(kGenThreads), sizeof(GenSmem<T, D>), s, p->dev,
                               (const T*)q, (const T*)k_pool, (const T*)v_pool, sh.n_q_heads, sh.n_kv_heads, sh.page_size, sh.sm_scale * kLog2e));
+}
+template <typename T, int D>
+static int launch_generic(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool, cudaStream_t s) {
+  const int m = p->max_rows;                       // eight warps
+  return m <= 8 ? launch_generic_rows<T, D, 1>(p, q, k_pool, v_pool, s) : m <= 16 ? launch_generic_rows<T, D, 2>(p, q, k_pool, v_pool, s)
+       : m <= 32 ? launch_generic_rows<T, D, 4>(p, q, k_pool, v_pool, s) : launch_generic_rows<T, D, 8>(p, q, k_pool, v_pool, s);
 }
 
 int launch_attn_generic(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool, cudaStream_t s) {
