@@ -672,7 +672,7 @@ cudaError_t launch(const aspd_plan* p, Ctx& c, cudaStream_t s) {
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   const uint32_t smem = smem_layout(D, NR, &c);
-  return launch_pdl(kPdlAttn, attn_dec_kernel<D, NR>, dim3(p->n_ctas), dim3(kThreads), smem, s, c);
+  return launch_pdl(attn_dec_kernel<D, NR>, dim3(p->n_ctas), dim3(kThreads), smem, s, c);
 }
 
 }  // namespace

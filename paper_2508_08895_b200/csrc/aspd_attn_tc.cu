@@ -1263,12 +1263,12 @@ static int launch_tc(const aspd_plan* p, const void* q, const void* k_new, const
   if (p->wide == 2) {                       // row blocks of two query tiles: final outputs only
     if (c.out == nullptr) return ASPD_ERR_UNSUPPORTED;
     c.k_new = nullptr; c.v_new = nullptr;
-    return launch_pdl(kPdlAttn, attn_tc_w2_kernel, dim3(p->n_ctas), dim3(kThreads), kSmemBytesW2, s, c) == cudaSuccess ? ASPD_OK : ASPD_ERR_CUDA;
+    return launch_pdl(attn_tc_w2_kernel, dim3(p->n_ctas), dim3(kThreads), kSmemBytesW2, s, c) == cudaSuccess ? ASPD_OK : ASPD_ERR_CUDA;
   }
   auto* kernel = p->wide ? attn_tc_kernel<true, kPlain>
                  : c.m64 || c.merge_out != nullptr || c.out != nullptr ? attn_tc_kernel<false, kOptions>
                  : c.k_new != nullptr && p->patch_tiles ? attn_tc_kernel<false, kPatch> : attn_tc_kernel<false, kPlain>;
-  const cudaError_t e = launch_pdl(kPdlAttn, kernel, dim3(p->n_ctas), dim3(kThreads), kSmemBytes, s, c);
+  const cudaError_t e = launch_pdl(kernel, dim3(p->n_ctas), dim3(kThreads), kSmemBytes, s, c);
   return e == cudaSuccess ? ASPD_OK : ASPD_ERR_CUDA;
 }
 

@@ -468,6 +468,7 @@ __global__ void read_token_kernel(const T* pool, size_t tile, int row, int head_
   out[e] = to_f32(*reinterpret_cast<const T*>(reinterpret_cast<const char*>(pool) + tile + tile_offset(row, e * sizeof(T), head_dim * sizeof(T))));
 }
 
+constexpr int kCombineClaim = 115 * 1024;        // more than half of the 228 KB of an SM
 inline int check_launch() { return cudaGetLastError() == cudaSuccess ? ASPD_OK : ASPD_ERR_CUDA; }
 inline int status_of(cudaError_t e) { return e == cudaSuccess ? ASPD_OK : ASPD_ERR_CUDA; }
 
@@ -480,10 +481,10 @@ int launch_append(const aspd_plan* p, const void* k_new, const void* v_new, cons
   const dim3 grid((unsigned)(((long)p->n_new * sh.n_kv_heads * chunks + kAppendThreads - 1) / kAppendThreads)), block(kAppendThreads);
   const float2* cs = pos == p->dev.tok_pos ? p->dev.q_cs : nullptr;
   if (sh.dtype == ASPD_DTYPE_BF16)
-    return status_of(launch_pdl(kPdlAppend, append_kernel<__nv_bfloat16>, grid, block, 0, s, (const __nv_bfloat16*)k_new,
+    return status_of(launch_pdl(append_kernel<__nv_bfloat16>, grid, block, 0, s, (const __nv_bfloat16*)k_new,
                                 (const __nv_bfloat16*)v_new, pos, cs, p->dev.tok_page, p->dev.tok_row, p->dev.inv_freq,
                                 (__nv_bfloat16*)k_pool, (__nv_bfloat16*)v_pool, p->n_new, sh.n_kv_heads, sh.head_dim, sh.page_size, p->dev));
-  return status_of(launch_pdl(kPdlAppend, append_kernel<float>, grid, block, 0, s, (const float*)k_new, (const float*)v_new, pos, cs,
+  return status_of(launch_pdl(append_kernel<float>, grid, block, 0, s, (const float*)k_new, (const float*)v_new, pos, cs,
                               p->dev.tok_page, p->dev.tok_row, p->dev.inv_freq, (float*)k_pool, (float*)v_pool, p->n_new,
                               sh.n_kv_heads, sh.head_dim, sh.page_size, p->dev));
 }
@@ -499,7 +500,7 @@ static int launch_generic_rows(const aspd_plan* p, const void* q, const void* k_
     if (dev >= 0 && dev < 64) configured[dev] = true;
   }
   const aspd_shape_t& sh = p->shape;
-  return status_of(launch_pdl(kPdlAttn, attn_generic_kernel<T, D, RPW>, dim3(p->n_ctas), dim3(kGenThreads), sizeof(GenSmem<T, D>), s, p->dev,
+  return status_of(launch_pdl(attn_generic_kernel<T, D, RPW>, dim3(p->n_ctas), dim3(kGenThreads), sizeof(GenSmem<T, D>), s, p->dev,
                               (const T*)q, (const T*)k_pool, (const T*)v_pool, sh.n_q_heads, sh.n_kv_heads, sh.page_size, sh.sm_scale * kLog2e));
 }
 template <typename T, int D>
@@ -524,23 +525,36 @@ int launch_qcs(const aspd_plan* p, cudaStream_t s) {
   return check_launch();
 }
 
+template <typename T, int D>
+static int launch_combine_of(const aspd_plan* p, void* out, cudaStream_t s) {
+  const aspd_shape_t& sh = p->shape;
+  static int sms[64] = {};                         // per device: SMs, known once the kernel has been configured there
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return ASPD_ERR_CUDA;
+  int n_sms = dev >= 0 && dev < 64 ? sms[dev] : 0;
+  if (n_sms == 0) {
+    if (cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(combine_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombineClaim) != cudaSuccess)
+      return ASPD_ERR_CUDA;
+    if (dev >= 0 && dev < 64) sms[dev] = n_sms;
+  }
+  // The launch attribute lets the blocks wait on the SMs while the attention pass ends, so that the merge starts
+  // without the latency of a launch.  They come to the SMs as those fall free, as many as fit: all 56 of one long
+  // request onto the first SM or two, whose memory pipes then do all the work.  So the blocks of a grid that has an
+  // SM for each claim, without using it, more than half of an SM's shared memory.  A pass of layers launched from
+  // the host, in us, without the attribute / with it / with the claim as well: four branches over 2 k tokens 360 /
+  // 330 / 306, one token after another over 1 k 255 / 213 / 213, eight branches over 16 k 517 / 627 / 495, eight
+  // requests with heads of 64 410 / 402 / 364.  A grid larger than the chip spreads anyway, and would run in waves
+  // (six branches opened with twelve tokens each, 504 blocks: 480 / 438 / 524).
+  const int blocks = (p->n_new * sh.n_q_heads + 3) / 4;
+  const size_t claim = blocks <= n_sms ? kCombineClaim : 0;
+  return status_of(launch_pdl(combine_kernel<T, D>, dim3(blocks), dim3(128), claim, s, p->dev, (T*)out, p->n_new, sh.n_q_heads, sh.n_kv_heads));
+}
+
 int launch_combine(const aspd_plan* p, void* out, cudaStream_t s) {
   const aspd_shape_t& sh = p->shape;
-  const int warps = p->n_new * sh.n_q_heads;
-  const dim3 block(128), grid((warps + 3) / 4);
-  // Measured: with the attribute the combine's blocks wait on the SMs while the attention pass
-  // ends, which wins a little on a large step (serving mix: 48.6 against 49.2 us per layer) and
-  // loses a lot on small ones (long context, one request: 24.9 against 17.6; also with the rows in a
-  // few blocks of 32 warps, so that only a few SMs hold combine blocks: 24.7 against 18.2), so it
-  // follows the step's size.
-  const int which = p->algorithmic_bytes >= (128LL << 20) ? (kPdlCombine | kPdlCombineLarge) : kPdlCombine;
-#define ASPD_CMB(T, D) \
-  return status_of(launch_pdl(which, combine_kernel<T, D>, grid, block, 0, s, p->dev, (T*)out, p->n_new, sh.n_q_heads, sh.n_kv_heads))
-  if (sh.dtype == ASPD_DTYPE_BF16 && sh.head_dim == 128) ASPD_CMB(__nv_bfloat16, 128);
-  else if (sh.dtype == ASPD_DTYPE_BF16) ASPD_CMB(__nv_bfloat16, 64);
-  else if (sh.head_dim == 128) ASPD_CMB(float, 128);
-  else ASPD_CMB(float, 64);
-#undef ASPD_CMB
+  if (sh.dtype == ASPD_DTYPE_BF16) return sh.head_dim == 128 ? launch_combine_of<__nv_bfloat16, 128>(p, out, s) : launch_combine_of<__nv_bfloat16, 64>(p, out, s);
+  return sh.head_dim == 128 ? launch_combine_of<float, 128>(p, out, s) : launch_combine_of<float, 64>(p, out, s);
 }
 
 int launch_rerotate(const aspd_shape_t* sh, void* k_pool, const int32_t* pages, const int32_t* rows, const int32_t* delta,
@@ -550,9 +564,9 @@ int launch_rerotate(const aspd_shape_t* sh, void* k_pool, const int32_t* pages, 
   InvFreq table;
   for (int i = 0; i < sh->head_dim / 2; ++i) table.f[i] = pow((double)sh->rope_theta, -2.0 * i / (double)sh->head_dim);
   if (sh->dtype == ASPD_DTYPE_BF16)
-    return status_of(launch_pdl(kPdlAppend, rerotate_kernel<__nv_bfloat16>, grid, block, 0, s, (__nv_bfloat16*)k_pool, pages, rows,
+    return status_of(launch_pdl(rerotate_kernel<__nv_bfloat16>, grid, block, 0, s, (__nv_bfloat16*)k_pool, pages, rows,
                                 delta, table, n, sh->n_kv_heads, sh->head_dim, sh->page_size));
-  return status_of(launch_pdl(kPdlAppend, rerotate_kernel<float>, grid, block, 0, s, (float*)k_pool, pages, rows, delta,
+  return status_of(launch_pdl(rerotate_kernel<float>, grid, block, 0, s, (float*)k_pool, pages, rows, delta,
                               table, n, sh->n_kv_heads, sh->head_dim, sh->page_size));
 }
 
@@ -580,10 +594,10 @@ int launch_rerotate_ranges(const aspd_shape_t* sh, void* const* k_pools, int n_l
       const dim3 grid((unsigned)rr.unit0[rr.n], (unsigned)nl), block((unsigned)(ps * chunks));
       cudaError_t e;
       if (sh->dtype == ASPD_DTYPE_BF16)
-        e = launch_pdl(kPdlAppend, rerotate_ranges_kernel<__nv_bfloat16>, grid, block, 0, s, pools, page_table, rr, table, sh->n_kv_heads,
+        e = launch_pdl(rerotate_ranges_kernel<__nv_bfloat16>, grid, block, 0, s, pools, page_table, rr, table, sh->n_kv_heads,
                        sh->head_dim, ps);
       else
-        e = launch_pdl(kPdlAppend, rerotate_ranges_kernel<float>, grid, block, 0, s, pools, page_table, rr, table, sh->n_kv_heads,
+        e = launch_pdl(rerotate_ranges_kernel<float>, grid, block, 0, s, pools, page_table, rr, table, sh->n_kv_heads,
                        sh->head_dim, ps);
       if (e != cudaSuccess) return ASPD_ERR_CUDA;
     }

@@ -845,8 +845,7 @@ int aspd_plan_update(aspd_plan_t* p, const aspd_request_t* req, const aspd_branc
   const aspd::PlanLayout& L = p->layout;
   if (t->n_new != p->n_new || t->n_ctas != p->n_ctas || t->kernel != p->kernel || t->wide != p->wide || t->dealt != p->dealt ||
       t->fuse_append != p->fuse_append || t->shared_mask != p->shared_mask || t->single_launch != p->single_launch || t->m64 != p->m64 || (p->dec && padded_rows(t->max_rows) != padded_rows(p->max_rows)) || t->kernel != ASPD_KERNEL_MMA ||
-      t->row_blocks.size() != L.n_row_blocks || t->part_base.size() != L.n_part_base ||
-      (t->algorithmic_bytes >= (128LL << 20)) != (p->algorithmic_bytes >= (128LL << 20))) {   // the combine's launch attribute
+      t->row_blocks.size() != L.n_row_blocks || t->part_base.size() != L.n_part_base) {
     delete t;
     return ASPD_ERR_UNSUPPORTED;
   }
