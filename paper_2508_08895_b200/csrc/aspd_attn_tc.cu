@@ -712,18 +712,23 @@ __device__ __forceinline__ void prep_q(const Ctx& c, const DeviceItem& it, uint3
 // have copied without waiting for the pools' rows (patch_tile).
 // Called by the four epilogue warps while the softmax warps prepare the first query tile.  A warp takes two rows
 // at a time, lanes 0-15 the 16-byte chunks of K (with their partner chunks, half a row away), lanes 16-31 those of
-// V; all pieces of both rows are requested before the first is used.
+// V; all pieces of both rows are requested before the first is used.  `mine`: lane l holds entry l; more than 32
+// (CTAs with many tiles, which come to those rows much later) are fetched as they are needed.
 template <bool STASH>
-__device__ __forceinline__ void append_new_rows(const Ctx& c, uint32_t base, int warp_rank, int lane, int4 mine, int n_rows) {
+__device__ __forceinline__ void append_new_rows(const Ctx& c, uint32_t base, int warp_rank, int lane, int4 mine, int dirty0, int n_rows) {
   const int ch = lane & 15;
   const bool is_v = lane >= 16;
 #pragma unroll 1
   for (int e0 = warp_rank; e0 < n_rows; e0 += 8) {
+    if (!STASH && (e0 & 31) == warp_rank && e0 >= 32) {          // the next 32 entries
+      const int i = (e0 & ~31) + lane;
+      if (i < n_rows) mine = c.pd.dirty[dirty0 + i];
+    }
     uint4 own[2], other[2];
     float4 w[2][4];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      const int e = min(e0 + 4 * k, n_rows - 1), head = __shfl_sync(0xffffffffu, mine.y, e), tok = __shfl_sync(0xffffffffu, mine.z, e);
+      const int e = min(e0 + 4 * k, n_rows - 1), head = __shfl_sync(0xffffffffu, mine.y, e & 31), tok = __shfl_sync(0xffffffffu, mine.z, e & 31);
       const __nv_bfloat16* src = (is_v ? c.v_new : c.k_new) + ((size_t)tok * c.n_kv_heads + head) * 128;
       own[k] = *reinterpret_cast<const uint4*>(src + ch * 8);
       other[k] = *reinterpret_cast<const uint4*>(src + (ch ^ 8) * 8);
@@ -744,7 +749,7 @@ __device__ __forceinline__ void append_new_rows(const Ctx& c, uint32_t base, int
         const float s0 = ch < 8 ? -w[k][i].y : w[k][i].y, s1 = ch < 8 ? -w[k][i].w : w[k][i].w;
         if (!is_v) r[i] = pack_bf16(x.x * w[k][i].x + y.x * s0, x.y * w[k][i].z + y.y * s1);
       }
-      const int page = __shfl_sync(0xffffffffu, mine.x, e), head = __shfl_sync(0xffffffffu, mine.y, e), row = __shfl_sync(0xffffffffu, mine.w, e) & 255;
+      const int page = __shfl_sync(0xffffffffu, mine.x, e & 31), head = __shfl_sync(0xffffffffu, mine.y, e & 31), row = __shfl_sync(0xffffffffu, mine.w, e & 31) & 255;
       if constexpr (STASH)
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(row_stash(base, e) + lane * 16), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
       if (bounds_ok(c.pd, page, row, 16))
@@ -1045,7 +1050,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
     int item_no = 0;
     bool dead = false;
     if (dirty_rows > 0) {
-      append_new_rows<PATCH>(c, base, ew, lane, dirty, dirty_rows);
+      append_new_rows<PATCH>(c, base, ew, lane, dirty, head2.x, dirty_rows);
       // generic-proxy stores before async-proxy copies: this launch's (unless the tiles are patched) and later ones'
       if (patch) mbar_arrive(bars + 8 * A_DONE);
       asm volatile("fence.proxy.async;" ::: "memory");

@@ -13,7 +13,7 @@ namespace aspd {
 
 constexpr int kMaxRowsPerItem = 64;   // query rows (tokens x group heads) one work item carries
 constexpr int kMaxRowsWide = 128;     // ... in a plan that deals whole streams to the tensor-core kernel's CTAs
-constexpr int kMostFusedRows = 20;   // new rows per CTA up to which the attention pass writes them itself
+constexpr int kMostFusedRows = 20;   // new rows per CTA up to which the attention pass writes them itself (short CTAs; long ones write any number)
 constexpr int kCausalAll = 1 << 29;   // prefix end of a token that sees its whole key stream
 
 // ---------------------------------------------------------------------------------------

@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <functional>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -350,11 +351,11 @@ int aspd_visible_slots_masked(const aspd_request_t* req, const aspd_branch_t* br
 
 static int plan_to_device(aspd_plan* p, cudaStream_t s);
 
-// sm_count_override > 0: plan for a grid of that many SMs without asking the device (aspd_plan_update
-// re-plans on the host for the device the plan already lives on)
+// like: the plan that this one is to take the place of (aspd_plan_update re-plans on the host for the device that
+// plan lives on): the grid of its device, its way of splitting the streams and, as far as possible, of writing new rows
 static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req, const aspd_branch_t* br,
                             const int32_t* page_ids, int n_req, int64_t n_pool_pages, int mode, const int32_t* q_pos,
-                            const aspd_tuning_t* tuning, void* stream, int sm_count_override, aspd_plan_t** plan_out) {
+                            const aspd_tuning_t* tuning, void* stream, const aspd_plan* like, aspd_plan_t** plan_out) {
   if (!plan_out) return ASPD_ERR_INVALID_ARG;
   *plan_out = nullptr;
   int rc = check_shape(shape);
@@ -392,8 +393,8 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   p->host_only = tune.host_only; p->n_pool_pages = n_pool_pages; p->device_base = nullptr; p->device_bytes = 0;
   memset(&p->dev, 0, sizeof(p->dev));
   p->tune = tune;
-  p->sm_count = sm_count_override > 0 ? sm_count_override : 148;
-  if (!tune.host_only && sm_count_override <= 0) {
+  p->sm_count = like ? like->sm_count : 148;
+  if (!tune.host_only && !like) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -562,15 +563,46 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     const int want = tune.n_ctas > 0 ? tune.n_ctas : p->sm_count * (cores ? 2 : 1);
     return (int)std::max(1L, std::min((long)want, (pages + tile_pages - 1) / tile_pages));
   };
+  // Dealing the streams out whole, largest first, each to the CTA with the least so far.  A stream costs its pages and
+  // kDealItem more.  Returned: the largest share over the mean one.  (Rounds back and forth over the CTAs, as they were
+  // dealt before, left the first CTAs with a stream more and 8 to 12 % more pages: 160 requests, 212 us a layer
+  // against 204; the streams of masked prefill are so many that both come out even.)
+  std::vector<std::vector<int>> mine;
+  auto deal_out = [&](int n_ctas) {
+    constexpr double kDealItem = 8.0;
+    std::vector<int> order(streams.size());
+    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return streams[a].n_pages > streams[b].n_pages; });
+    mine.assign(n_ctas, {});
+    std::vector<std::pair<double, int>> load(n_ctas);                    // a heap, the CTA with the least on top
+    for (int c = 0; c < n_ctas; ++c) load[c] = {0.0, c};
+    double all = 0.0, most = 0.0;
+    for (int si : order) {
+      std::pop_heap(load.begin(), load.end(), std::greater<>());
+      auto& [cost, c] = load.back();
+      mine[c].push_back(si);
+      cost += kDealItem + streams[si].n_pages;
+      all += kDealItem + streams[si].n_pages;
+      most = std::max(most, cost);
+      std::push_heap(load.begin(), load.end(), std::greater<>());
+    }
+    return most * n_ctas / std::max(1.0, all);
+  };
   // With many more streams than CTAs (a step with many query tokens per branch: masked prefill,
-  // teacher forcing) nothing is cut: every stream is one item, and the streams are dealt to the
-  // CTAs in turn, longest requests first, so that at any moment all CTAs read the K/V pages of the
-  // same one or two requests (which then stay in L2) and every CTA gets one stream of each round.
+  // teacher forcing; a step of many requests) nothing is cut: every stream is one item whose CTA writes the output,
+  // and no records go through memory to a combine launch.  The longest requests come first, so that at any moment
+  // all CTAs read the K/V pages of the same one or two requests (which then stay in L2).
   // Every row block then gets a page sequence of its own, without the branch pages none of its
   // tokens sees, and the tensor-core kernel takes row blocks of up to 128 rows (its wide variant).
   // (only where the step fills the grid, or the caller chose the grid: a step of a few pages has few CTAs and many streams by default)
+  // From four streams per CTA on always; from two on where the shares come out even.  Requests of 0.5-8 k tokens, four
+  // KV heads, largest share over the mean one, us a layer dealt and cut: 100 requests 1.05, 134 and 146; 80 requests
+  // 1.08, 105 and 120; 60 requests 1.41 to 1.52, 87 to 93 and 85 to 87; 40 requests 1.97 to 2.3, 79 and 56 to 61.
+  constexpr double kDealSkew = 1.2;
   bool deal_streams = mode == ASPD_MODE_BRANCH && !shared_mask && tune.chunk_tokens == 0 &&
-                      (long)streams.size() >= 4L * ctas_for(total_pages) && (tune.n_ctas > 0 || ctas_for(total_pages) >= p->sm_count);
+                      (long)streams.size() >= 2L * ctas_for(total_pages) && (tune.n_ctas > 0 || ctas_for(total_pages) >= p->sm_count);
+  if (deal_streams && (long)streams.size() < 4L * ctas_for(total_pages)) deal_streams = deal_out(ctas_for(total_pages)) <= kDealSkew;
+  if (like) deal_streams = like->dealt != 0;
   p->wide = 0;
   if (deal_streams) {
     p->wide = (kernel == ASPD_KERNEL_MMA && wide_ok && kMaxRowsWide / G > max_tok) ? 1 : 0;
@@ -594,14 +626,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   std::vector<int32_t> n_parts((size_t)n_new * Hkv, 0), part_base((size_t)n_new * Hkv + 1, 0), cta_item0(n_ctas + 1, 0);
   p->dealt = deal_streams ? 1 : 0;
   if (deal_streams) {
-    std::vector<int> order(streams.size());
-    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return streams[a].n_pages > streams[b].n_pages; });
-    std::vector<std::vector<int>> mine(n_ctas);
-    for (size_t i = 0; i < order.size(); ++i) {
-      const int round = (int)(i / n_ctas), k = (int)(i % n_ctas);
-      mine[(round & 1) ? n_ctas - 1 - k : k].push_back(order[i]);       // back and forth: evens out the rounds
-    }
+    deal_out(n_ctas);
     for (int c = 0; c < n_ctas; ++c) {
       cta_item0[c] = (int)p->items.size();
       for (int si : mine[c]) {
@@ -669,7 +694,11 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   // are found once, not once per KV head and CTA.)
   std::vector<int4> dirty;
   std::vector<int32_t> cta_dirty0(n_ctas + 1, 0);
-  p->fuse_append = (kernel == ASPD_KERNEL_MMA && !shared_mask && tok_field_fits && p->wide != 2) ? 1 : 0;
+  p->fuse_append = (kernel == ASPD_KERNEL_MMA && !shared_mask && tok_field_fits && p->wide != 2 && !(like && !like->fuse_append)) ? 1 : 0;
+  // A CTA with that many tiles has its rows written long before it comes to the pages that hold them, so there any
+  // number is written at its start (160 requests, 740 new rows, up to 40 per CTA and head: 205 us a layer against
+  // 212 with the append kernel; 50 requests cut into parts: 70.2 against 71.5).
+  constexpr int kLongCta = 16;
   if (p->fuse_append) {
     std::vector<int> fresh;                        // entries of `visit` with new rows, ascending
     for (size_t i = 0; i < visit.size(); ++i)
@@ -689,7 +718,8 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
         tile0 += (it.n_pages + ppt - 1) / ppt;
       }
       // (32 767 tiles: what the number's field holds)
-      if ((int)dirty.size() - cta_dirty0[c] > kMostFusedRows || tile0 > 32767) p->fuse_append = 0;
+      const int rows = (int)dirty.size() - cta_dirty0[c];
+      if ((rows > kMostFusedRows && !(tile0 >= kLongCta && !p->dec) && !(like && !like->patch_tiles)) || tile0 > 32767) p->fuse_append = 0;
     }
     cta_dirty0[n_ctas] = (int)dirty.size();
     if (!p->fuse_append) { dirty.clear(); std::fill(cta_dirty0.begin(), cta_dirty0.end(), 0); }
@@ -725,7 +755,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
 int aspd_plan_create(const aspd_shape_t* shape, const aspd_request_t* req, const aspd_branch_t* br,
                      const int32_t* page_ids, int n_req, int64_t n_pool_pages, int mode, const int32_t* q_pos,
                      const aspd_tuning_t* tuning, void* stream, aspd_plan_t** plan_out) {
-  return plan_create_impl(shape, req, br, page_ids, n_req, n_pool_pages, mode, q_pos, tuning, stream, 0, plan_out);
+  return plan_create_impl(shape, req, br, page_ids, n_req, n_pool_pages, mode, q_pos, tuning, stream, nullptr, plan_out);
 }
 
 // ---- one device allocation, one staging blob ----------------------------------------------
@@ -840,7 +870,7 @@ int aspd_plan_update(aspd_plan_t* p, const aspd_request_t* req, const aspd_branc
   aspd_tuning_t tune = p->tune;
   tune.host_only = 1;
   aspd_plan* t = nullptr;
-  int rc = plan_create_impl(&p->shape, req, br, page_ids, n_req, p->n_pool_pages, p->mode, q_pos, &tune, nullptr, p->sm_count, &t);
+  int rc = plan_create_impl(&p->shape, req, br, page_ids, n_req, p->n_pool_pages, p->mode, q_pos, &tune, nullptr, p, &t);
   if (rc) return rc;
   const aspd::PlanLayout& L = p->layout;
   if (t->n_new != p->n_new || t->n_ctas != p->n_ctas || t->kernel != p->kernel || t->wide != p->wide || t->dealt != p->dealt ||
