@@ -625,6 +625,11 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   p->chunk_tokens = tune.chunk_tokens; p->n_ctas = n_ctas;
   std::vector<int32_t> n_parts((size_t)n_new * Hkv, 0), part_base((size_t)n_new * Hkv + 1, 0), cta_item0(n_ctas + 1, 0);
   p->dealt = deal_streams ? 1 : 0;
+  std::vector<int> fresh;                          // entries of `visit` with new rows, ascending
+  if (kernel == ASPD_KERNEL_MMA)
+    for (size_t i = 0; i < visit.size(); ++i)
+      if ((visit[i].y >> 8) & 31) fresh.push_back((int)i);
+  p->patch_tiles = (!deal_streams && total_pages <= 2L * 8 * n_ctas) ? 1 : 0;
   if (deal_streams) {
     deal_out(n_ctas);
     for (int c = 0; c < n_ctas; ++c) {
@@ -648,45 +653,79 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     // 0.35 % per row), so streams of requests with many branches weigh more
     const double kRowCost = 0.0035;
     auto page_cost = [&](const Stream& st) { return 1.0 + kRowCost * st.n_tok * G; };
+    // A CTA that comes to a page with new rows within its first 256 keys waits for them (its first tiles arrive while
+    // the kernel before this one still runs, the rows are written after it), unless the rows are put into the tiles
+    // (patch_tiles): it gets fewer pages, as many as it could have had by then.  Measured at 0 / 128 / 256 / 384 / 512
+    // keys, us a layer: one request of 16 k tokens and eight branches 16.9 / 16.5 / 16.4 / 16.1 / 16.3, 8 requests
+    // 18.8 / 18.5 / 18.1 / 18.0 / 18.8, 12 requests 22.2 / 22.0 / 21.7 / 22.4 / 23.0; 32 requests, whose CTAs have
+    // two dozen tiles each, 48.3 / 48.3 / 48.2 / 48.3 / 48.2.
+    const double kWait = (kernel == ASPD_KERNEL_MMA && !p->patch_tiles) ? 256.0 / ps : 0.0;
     // the share is re-derived from what is left whenever a CTA is closed, so rounding does not pile up
-    double cost_left = 0.0;
-    for (const Stream& st : streams) cost_left += page_cost(st) * st.n_pages;
-    long streams_left = (long)streams.size();
-    auto share_now = [&](int ctas_left) {
-      return (cost_left + kItemCost * ((double)streams_left + ctas_left)) / std::max(1, ctas_left);
-    };
-    double share = share_now(n_ctas);
-    int cta = 0;
-    double acc = 0.0;                              // cost already given to the current CTA
-    auto next_cta = [&]() { cta_item0[++cta] = (int)p->items.size(); acc = 0.0; share = share_now(n_ctas - cta); };
-    for (const Stream& st : streams) {
-      int at = 0, slot = 0;
-      const size_t first_item = p->items.size();
-      const double pc = page_cost(st);
-      --streams_left;
-      while (at < st.n_pages) {
-        double room = (share - acc - kItemCost) / pc;   // pages that still fit if an item starts here
-        if (room < 1.0 && acc > 0.0 && cta + 1 < n_ctas) { next_cta(); continue; }
-        long take = std::min<long>(st.n_pages - at, chunk_pages);
-        if (cta + 1 < n_ctas) take = std::min<long>(take, std::max<long>(1, (long)(room + 0.5)));
-        // a cut inside a stream goes on a tile boundary (128 keys; CUDA cores: 32) where the item is long
-        // enough: the item's last tile is then a full one (measured on the serving mix: 0.4 % on the step)
-        if (take < st.n_pages - at && tune.chunk_tokens == 0 && take >= tile_pages + tile_pages / 2)
-          take = std::min<long>((take + tile_pages / 2) / tile_pages * tile_pages, st.n_pages - at);
-        DeviceItem it;
-        it.q_tok0 = st.tok0; it.n_q_tok = st.n_tok; it.kv_head = st.head; it.page0 = st.page0 + at;
-        it.n_pages = (int)take; it.key0 = at * ps; it.part_slot = slot++; it.request = st.request;
-        it.row_block = st.row_block; it.n_parts = 0;
-        p->items.push_back(it);
-        at += (int)take;
-        cost_left -= pc * take;
-        acc += kItemCost + pc * (double)take;
-        if (acc >= share - 0.5 && cta + 1 < n_ctas) next_cta();
+    // (the sum of the waits is not known before the cuts are: made twice where there are any)
+    auto cut = [&](double waits_left) {
+      double cost_left = 0.0, waits = 0.0;
+      for (const Stream& st : streams) cost_left += page_cost(st) * st.n_pages;
+      long streams_left = (long)streams.size();
+      auto share_now = [&](int ctas_left) {
+        return (cost_left + std::max(0.0, waits_left) + kItemCost * ((double)streams_left + ctas_left)) / std::max(1, ctas_left);
+      };
+      double share = share_now(n_ctas);
+      int cta = 0;
+      double acc = 0.0;                              // cost already given to the current CTA
+      int done = 0;                                  // its pages
+      bool waited = false;                           // it has come to a page with new rows
+      p->items.clear();
+      auto next_cta = [&]() { cta_item0[++cta] = (int)p->items.size(); acc = 0.0; done = 0; waited = false; share = share_now(n_ctas - cta); };
+      // what the CTA waits, in pages, when it goes on with `take` pages from entry `from` of `visit`
+      auto wait_for = [&](int from, long take) {
+        if (waited || done >= kWait) return 0.0;
+        const auto e = std::lower_bound(fresh.begin(), fresh.end(), from);
+        return e == fresh.end() || *e >= from + take ? 0.0 : std::max(0.0, kWait - done - (*e - from));
+      };
+      for (const Stream& st : streams) {
+        int at = 0, slot = 0;
+        const size_t first_item = p->items.size();
+        const double pc = page_cost(st);
+        --streams_left;
+        while (at < st.n_pages) {
+          double room = (share - acc - kItemCost) / pc;   // pages that still fit if an item starts here
+          if (room < 1.0 && acc > 0.0 && cta + 1 < n_ctas) { next_cta(); continue; }
+          long take = std::min<long>(st.n_pages - at, chunk_pages);
+          if (cta + 1 < n_ctas) take = std::min<long>(take, std::max<long>(1, (long)(room + 0.5)));
+          // a cut inside a stream goes on a tile boundary (128 keys; CUDA cores: 32) where the item is long
+          // enough: the item's last tile is then a full one (measured on the serving mix: 0.4 % on the step)
+          if (take < st.n_pages - at && tune.chunk_tokens == 0 && take >= tile_pages + tile_pages / 2)
+            take = std::min<long>((take + tile_pages / 2) / tile_pages * tile_pages, st.n_pages - at);
+          double wait = wait_for(st.page0 + at, take);
+          if (wait > 0.0 && cta + 1 < n_ctas) {
+            room -= wait / pc;
+            if (room < 1.0 && acc > 0.0) { next_cta(); continue; }
+            if (tune.chunk_tokens == 0 && room < (double)take) {
+              take = std::max<long>(1, (long)(room + 0.5));
+              if (take >= tile_pages + tile_pages / 2) take = (take + tile_pages / 2) / tile_pages * tile_pages;
+              take = std::min<long>(take, st.n_pages - at);
+              wait = wait_for(st.page0 + at, take);
+            }
+          }
+          DeviceItem it;
+          it.q_tok0 = st.tok0; it.n_q_tok = st.n_tok; it.kv_head = st.head; it.page0 = st.page0 + at;
+          it.n_pages = (int)take; it.key0 = at * ps; it.part_slot = slot++; it.request = st.request;
+          it.row_block = st.row_block; it.n_parts = 0;
+          p->items.push_back(it);
+          at += (int)take;
+          cost_left -= pc * take;
+          acc += kItemCost + pc * (double)take + wait;
+          waits += wait; waits_left -= wait; waited |= wait > 0.0; done += (int)take;
+          if (acc >= share - 0.5 && cta + 1 < n_ctas) next_cta();
+        }
+        for (int i = 0; i < st.n_tok; ++i) n_parts[(size_t)(st.tok0 + i) * Hkv + st.head] = slot;
+        for (size_t i = first_item; i < p->items.size(); ++i) p->items[i].n_parts = slot;
       }
-      for (int i = 0; i < st.n_tok; ++i) n_parts[(size_t)(st.tok0 + i) * Hkv + st.head] = slot;
-      for (size_t i = first_item; i < p->items.size(); ++i) p->items[i].n_parts = slot;
-    }
-    while (cta < n_ctas) cta_item0[++cta] = (int)p->items.size();
+      while (cta < n_ctas) cta_item0[++cta] = (int)p->items.size();
+      return waits;
+    };
+    const double waits = cut(0.0);
+    if (waits > 0.0) cut(waits);
   }
   // Rows that are new this step, per CTA: what a fused step must write before the CTA reads.  The fused step
   // writes them in batches at the start of the kernel; with many new rows per CTA (a branch-open step) the
@@ -700,9 +739,6 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   // 212 with the append kernel; 50 requests cut into parts: 70.2 against 71.5).
   constexpr int kLongCta = 16;
   if (p->fuse_append) {
-    std::vector<int> fresh;                        // entries of `visit` with new rows, ascending
-    for (size_t i = 0; i < visit.size(); ++i)
-      if ((visit[i].y >> 8) & 31) fresh.push_back((int)i);
     for (int c = 0; c < n_ctas && p->fuse_append; ++c) {
       cta_dirty0[c] = (int)dirty.size();
       const int ppt = 128 / ps;                    // pages of a tile
@@ -730,7 +766,6 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   // down, stays as it is); 0: both with M = 128
   p->m64 = (kernel == ASPD_KERNEL_MMA && !deal_streams && !p->dec) ? (tune.mma_m == 64 ? 1 : tune.mma_m == 128 ? 0 : 2) : 0;
   p->stagger_start = (!deal_streams && total_pages <= 6L * 8 * n_ctas) ? 1 : 0;       // at most six 128-key tiles per CTA
-  p->patch_tiles = (!deal_streams && total_pages <= 2L * 8 * n_ctas) ? 1 : 0;
   // Merging inside the attention kernel is an option, not the default.  Measured on every workload of
   // the benchmark, the CTA that stores a pair's last record is a CTA at the very end of its own work,
   // so its fence, count and merge (1.5 us + one memory round trip per 16 rows of the pairs it ended
