@@ -653,13 +653,15 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     // 0.35 % per row), so streams of requests with many branches weigh more
     const double kRowCost = 0.0035;
     auto page_cost = [&](const Stream& st) { return 1.0 + kRowCost * st.n_tok * G; };
-    // A CTA that comes to a page with new rows within its first 256 keys waits for them (its first tiles arrive while
+    // A CTA that comes to a page with new rows within its first 160 keys waits for them (its first tiles arrive while
     // the kernel before this one still runs, the rows are written after it), unless the rows are put into the tiles
-    // (patch_tiles): it gets fewer pages, as many as it could have had by then.  Measured at 0 / 128 / 256 / 384 / 512
-    // keys, us a layer: one request of 16 k tokens and eight branches 16.9 / 16.5 / 16.4 / 16.1 / 16.3, 8 requests
-    // 18.8 / 18.5 / 18.1 / 18.0 / 18.8, 12 requests 22.2 / 22.0 / 21.7 / 22.4 / 23.0; 32 requests, whose CTAs have
-    // two dozen tiles each, 48.3 / 48.3 / 48.2 / 48.3 / 48.2.
-    const double kWait = (kernel == ASPD_KERNEL_MMA && !p->patch_tiles) ? 256.0 / ps : 0.0;
+    // (patch_tiles): it gets fewer pages, as many as it could have had by then.  Cuts lie on tile boundaries, so a
+    // single step can gain or lose a tile: judged over many.  At 0 / 96 / 128 / 160 / 192 / 256 keys, mean us a layer: six
+    // requests of 9 to 16 k tokens with eight branches 16.1 / 15.8 / 15.5 / 15.4 / 15.1 / 15.5 (one of them 16.9 / 16.6 /
+    // 16.4 / 16.0 / 15.8 / 16.4), steps of 3 to 20 requests 18.9 / 18.8 / 18.7 / 18.5 / 18.5 / 18.5 (worst step against 0:
+    // at 160 2.6 % slower, at 192 3.5 %, at 256 the 12 k request 11 %); 32 requests, whose CTAs have two dozen tiles
+    // each, come out the same.
+    const double kWait = (kernel == ASPD_KERNEL_MMA && !p->patch_tiles) ? 160.0 / ps : 0.0;
     // the share is re-derived from what is left whenever a CTA is closed, so rounding does not pile up
     // (the sum of the waits is not known before the cuts are: made twice where there are any)
     auto cut = [&](double waits_left) {

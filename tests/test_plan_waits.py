@@ -26,5 +26,8 @@ def test_cuts(prefix, prior, n_ctas):
         new = {256 + 7 * b for b in range(8)}
         first = [next((i for i, p in enumerate(p for x in it[at[c]:at[c + 1]] for p in range(int(x["page0"]), int(x["page0"] + x["n_pages"])))
                        if p in new), 99) for c in range(len(pages) - 1)]
-        at_once = np.array([f < 8 for f in first])              # (the last CTA takes what is left)
-        assert at_once.any() and pages[:-1][at_once].max() < pages[:-1][~at_once].min() and pages.max() <= 1.4 * pages.mean()
+        # A CTA with a new row in its page f < 10 is charged 10 - f pages; cuts are rounded to tiles of 8, up to 4 pages off
+        # either way, which evens out: less on average, and no CTA (but the last, which takes what is left) above the mean
+        # by more than a tile and the charge of the others.
+        at_once = np.array([f < 8 for f in first])
+        assert at_once.sum() >= 4 and pages[:-1][at_once].mean() < pages[:-1][~at_once].mean() - 1 and pages.max() <= pages.mean() + 8 + 10
