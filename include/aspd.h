@@ -184,7 +184,8 @@ typedef struct {
                                attention and step calls are one launch; 0: a combine launch follows      */
   int32_t mma_m;            /* M of the tensor-core kernel's MMAs in this plan: 128, 64 or 96 (see aspd_tuning_t;
                                0: generic kernel)                                                          */
-  int32_t reserved;
+  int32_t patch_tiles;      /* 1: the fused step puts the new rows into the K/V tiles it has fetched (every CTA has at
+                               most 20 of them then); 0: it fetches their pages after writing them           */
   int64_t workspace_bytes;  /* device memory the plan holds                                 */
   int64_t kv_tokens_read;   /* cached tokens the step must read (each once)                 */
   int64_t algorithmic_bytes;/* K+V of those tokens + q in + out + appended K/V              */

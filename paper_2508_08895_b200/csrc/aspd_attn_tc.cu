@@ -825,7 +825,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
   int2 first_pages = make_int2(0, 0);
   if ((warp == W_KPROD || warp == W_VPROD) && lane < head.w) first_pages = c.pd.visit[head.z + lane];
   // fused step: the CTA's new rows (plan data), an entry per lane of the warps that deal with them
-  const int dirty_rows = c.k_new != nullptr ? head2.y : 0;
+  // (PATCH: the planner lists at most kMostFusedRows of a CTA for such launches; no more than that ever has a place)
+  const int dirty_rows = c.k_new == nullptr ? 0 : PATCH ? min(head2.y, kMostFusedRows) : head2.y;
   const bool patch = PATCH && dirty_rows > 0;
   int4 dirty = make_int4(0, 0, 0, -1);
   if (warp >= W_KPROD && lane < dirty_rows) dirty = c.pd.dirty[head2.x + lane];

@@ -128,7 +128,7 @@ struct aspd_plan {
   int dec = 0;                     // tensor-core plan of a shape that aspd_attn_dec.cu serves (head_dim 64, pages of 8 or 32)
   int max_rows = 0;                // largest number of query rows of an item
   int stagger_start = 0;           // few tiles per CTA: order the requests of a CTA's first tiles (see the producers)
-  int patch_tiles = 0;             // at most two tiles per CTA: a fused step puts the new rows into the tiles (see patch_tile)
+  int patch_tiles = 0;             // at most two tiles per CTA on average: a fused step puts the new rows into the tiles (see patch_tile)
   int single_launch = 0;           // stream-K plan of the tensor-core kernel whose last-arriving CTAs merge the records themselves
   int64_t n_pool_pages = 0;
   int64_t kv_tokens_read = 0;

@@ -738,8 +738,11 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   p->fuse_append = (kernel == ASPD_KERNEL_MMA && !shared_mask && tok_field_fits && p->wide != 2 && !(like && !like->fuse_append)) ? 1 : 0;
   // A CTA with that many tiles has its rows written long before it comes to the pages that hold them, so there any
   // number is written at its start (160 requests, 740 new rows, up to 40 per CTA and head: 205 us a layer against
-  // 212 with the append kernel; 50 requests cut into parts: 70.2 against 71.5).
+  // 212 with the append kernel; 50 requests cut into parts: 70.2 against 71.5).  Not where the tiles are patched:
+  // patch_tiles goes by the mean over the CTAs, so that one of them may be long (a forced cut every chunk_tokens
+  // keys leaves the last CTA with dozens of short tiles), and the rows' place in shared memory is kMostFusedRows long.
   constexpr int kLongCta = 16;
+  const bool patches = like ? like->patch_tiles != 0 : p->patch_tiles != 0;      // an update's launches are the old plan's
   if (p->fuse_append) {
     for (int c = 0; c < n_ctas && p->fuse_append; ++c) {
       cta_dirty0[c] = (int)dirty.size();
@@ -757,7 +760,8 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
       }
       // (32 767 tiles: what the number's field holds)
       const int rows = (int)dirty.size() - cta_dirty0[c];
-      if ((rows > kMostFusedRows && !(tile0 >= kLongCta && !p->dec) && !(like && !like->patch_tiles)) || tile0 > 32767) p->fuse_append = 0;
+      const bool any_number = !patches && (like || (tile0 >= kLongCta && !p->dec));
+      if ((rows > kMostFusedRows && !any_number) || tile0 > 32767) p->fuse_append = 0;
     }
     cta_dirty0[n_ctas] = (int)dirty.size();
     if (!p->fuse_append) { dirty.clear(); std::fill(cta_dirty0.begin(), cta_dirty0.end(), 0); }
@@ -949,7 +953,8 @@ int aspd_plan_info(const aspd_plan_t* p, aspd_plan_info_t* info) {
   info->chunk_tokens = p->chunk_tokens; info->n_ctas = p->n_ctas; info->fused_append = (p->kernel == ASPD_KERNEL_MMA && p->fuse_append) ? 1 : 0;
   info->direct_output = attn_mma_direct(p) ? 1 : 0; info->max_rows_per_item = p->wide ? p->wide * kMaxRowsWide : kMaxRowsPerItem;
   info->dealt = p->dealt; info->single_launch = p->single_launch;
-  info->mma_m = p->kernel == ASPD_KERNEL_MMA ? (p->m64 == 1 ? 64 : p->m64 == 2 ? 96 : 128) : 0; info->reserved = 0;
+  info->mma_m = p->kernel == ASPD_KERNEL_MMA ? (p->m64 == 1 ? 64 : p->m64 == 2 ? 96 : 128) : 0;
+  info->patch_tiles = (info->fused_append && p->patch_tiles && !p->dec && p->m64 != 1 && !p->single_launch) ? 1 : 0;
   info->workspace_bytes = (int64_t)p->device_bytes;
   info->kv_tokens_read = p->kv_tokens_read; info->algorithmic_bytes = p->algorithmic_bytes;
   return ASPD_OK;
