@@ -429,8 +429,10 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   std::vector<int4> tok_vis(n_new);
   int64_t kv_tokens = 0;
   const bool tok_field_fits = n_new < (1 << 18);      // the 18 bits above bit 13 of a page entry hold a token index
+  bool counts_fit = true;                             // the 5 bits before them every page's number of new rows
   auto build_visit = [&](int block_tok) {
     visit.clear(); blocks.clear();
+    counts_fit = true;
     int64_t kv_count = 0;
     int t = 0;
     // new_key0 / new_tok0: the keys [new_key0, len) of the region are this step's new tokens
@@ -450,7 +452,9 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
         const int nv = std::min(ps, len - s0), first_new = std::max(s0, new_key0);
         const int n_newrows = std::max(0, s0 + nv - first_new);
         int y = nv;
-        if (n_newrows > 0) y |= (std::min(n_newrows, 31) << 8);   // 5 bits; a count is only needed where pages have 16 rows
+        // 5 bits: a page of 32 new rows says 31, which is enough to tell that it has some, but not to write them
+        if (n_newrows > 31) counts_fit = false;
+        if (n_newrows > 0) y |= (std::min(n_newrows, 31) << 8);
         if (shared_mask) y |= branch_pages ? (s0 / ps) << 13 : 0;
         else if (n_newrows > 0 && tok_field_fits) y |= (new_tok0 + first_new - new_key0) << 13;
         out[s0 / ps] = make_int2(ids[s0 / ps], y);
@@ -735,7 +739,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   // are found once, not once per KV head and CTA.)
   std::vector<int4> dirty;
   std::vector<int32_t> cta_dirty0(n_ctas + 1, 0);
-  p->fuse_append = (kernel == ASPD_KERNEL_MMA && !shared_mask && tok_field_fits && p->wide != 2 && !(like && !like->fuse_append)) ? 1 : 0;
+  p->fuse_append = (kernel == ASPD_KERNEL_MMA && !shared_mask && tok_field_fits && counts_fit && p->wide != 2 && !(like && !like->fuse_append)) ? 1 : 0;
   // A CTA with that many tiles has its rows written long before it comes to the pages that hold them, so there any
   // number is written at its start (160 requests, 740 new rows, up to 40 per CTA and head: 205 us a layer against
   // 212 with the append kernel; 50 requests cut into parts: 70.2 against 71.5).  Not where the tiles are patched:
