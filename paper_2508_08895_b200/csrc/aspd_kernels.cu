@@ -266,6 +266,7 @@ rerotate_ranges_kernel(const PoolList pools, const int32_t* __restrict__ page_ta
 // crosses warps.  Bound by latency on the steps it serves: 3 branches over 256 tokens (fp32, 4 heads of 64) are
 // 10 CTAs of 32 keys, 7.4 us a step (append, this, combine) in a graph; 5 CTAs of 64 keys 10.2; the kernel before, a
 // block of four warps to 128 keys, each warp walking one row's keys through memory at a time, 153.7.
+// A key of weight 0 for a row is left out of it (its V row may hold Inf or NaN that the row does not see); no measurable time.
 constexpr int kGenThreads = 256, kGenWarps = kGenThreads / 32, kGenKeys = 32;
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool there) {   // 16 zero bytes if not there
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(there ? 16 : 0) : "memory");
@@ -403,10 +404,14 @@ __device__ __forceinline__ void generic_item(const PlanDevice& pd, const DeviceI
         for (int k = 0; k < 4; ++k) lane_elems<T, D>(sm.v[st], j + k, lane, v[k]);
 #pragma unroll
         for (int i = 0; i < RPW; ++i) {
-          const float4 w = *reinterpret_cast<const float4*>(&sm.p[warp][i][j]);
+          const float4 w4 = *reinterpret_cast<const float4*>(&sm.p[warp][i][j]);
+          const float w[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
-          for (int e = 0; e < EPL; ++e)
-            acc[i][e] = fmaf(w.w, v[3][e], fmaf(w.z, v[2][e], fmaf(w.y, v[1][e], fmaf(w.x, v[0][e], acc[i][e]))));
+          for (int k = 0; k < 4; ++k)
+            if (w[k] != 0.f) {                    // a key that the row does not see may hold anything, Inf and NaN too
+#pragma unroll
+              for (int e = 0; e < EPL; ++e) acc[i][e] = fmaf(w[k], v[k][e], acc[i][e]);
+            }
         }
       }
     }
