@@ -404,9 +404,10 @@ __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it,
 
 // --------------------------------------------------------------------------------------- end of an item
 // O^T (tensor memory: lane = element of the head, column = row) and the sums become one record per row for the
-// combine kernel, or the final output (plans that deal whole streams).
+// combine kernel, or the final output (plans that deal whole streams).  Returned: something of this thread's is not
+// finite (see redo_item).
 template <int D, int NR>
-__device__ __forceinline__ void finish_item(const Ctx& c, const DeviceItem& it, DecMisc* misc, uint32_t tmem, int par, bool dead) {
+__device__ __forceinline__ bool finish_item(const Ctx& c, const DeviceItem& it, DecMisc* misc, uint32_t tmem, int par, bool dead) {
   constexpr int HC = NR / 2;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = warp & 3, r0 = (warp >> 2) * HC;
   const int M = it.n_q_tok * (c.n_q_heads / c.n_kv_heads);
@@ -415,9 +416,12 @@ __device__ __forceinline__ void finish_item(const Ctx& c, const DeviceItem& it, 
   const int d = D == 128 ? q * 32 + lane : q * 16 + lane;
   const bool has_d = (D == 128 || lane < 16) && !dead;
   const bool whole = c.out != nullptr;
+  bool bad = false;
+  uint32_t top = 0;                                               // largest magnitude, as bits
   if (tid < NR) {
     const float l = (misc->wm[0][tid] + misc->wm[1][tid]) + (misc->wm[2][tid] + misc->wm[3][tid]);
     misc->al[tid] = l > 0.f ? 1.f / l : 0.f;
+    bad = tid < M && (!(l < INFINITY) || misc->ref[tid] == INFINITY);
     if (!whole && tid < M && !dead) c.pd.ws_ml[misc->row_out[par][tid]] = make_float2(l > 0.f ? misc->ref[tid] : -INFINITY, l);
   }
   if (whole) named_sync(1, kSmThreads);
@@ -427,12 +431,104 @@ __device__ __forceinline__ void finish_item(const Ctx& c, const DeviceItem& it, 
     ASPD_TMEM_LD8(o_addr + c8, o, 0);
     tmem_wait_ld();
 #pragma unroll
+    for (int i = 0; i < 8; ++i) top = max(top, __float_as_uint(o[i]) & 0x7fffffffu);   // (a test per stored element: 1.3 us a layer)
+#pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int r = r0 + c8 + i;
       if (!has_d || r >= M) continue;
       const size_t at = (size_t)misc->row_out[par][r] * D + d;
       if (whole) c.out[at] = __float2bfloat16_rn(o[i] * misc->al[r]);
       else c.pd.ws_o[at] = o[i];
+    }
+  }
+  return bad || (has_d && top >= 0x7f800000u);
+}
+
+// An item whose result is not finite, once more on the CUDA cores and straight from the pools.  The MMAs multiply every
+// V row of a tile by every row's weight, 0 for a key that the row does not see, so that Inf or NaN in one branch's
+// values becomes NaN in its sibling branches; and of an Inf that a row does see the pieces of queries and weights
+// make NaN.  Here a row takes the keys that it sees, as the CUDA-core kernel does.  A warp per query row, 32
+// keys at a time, a key per lane for the scores and D / 32 elements of the head per lane for the sum; nothing is
+// tuned, since finite values never come here (a vote that the item's end takes anyway asks for it) and a function
+// of its own keeps it out of the loop's code.  What the steps pay for asking, us a layer before and now: 8 requests with
+// heads of 64 from the host 14.6 and 14.8, steps with pages of 8 or 32 up to 2 % (inlined: up to 3 %).
+template <int D>
+__device__ __noinline__ void redo_item(const Ctx& c, const DeviceItem it, DecMisc* misc, float* q_sm, int par) {
+  constexpr int EPL = D / 32;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, G = c.n_q_heads / c.n_kv_heads, M = it.n_q_tok * G;
+  const int ps = c.page_size, n_keys = it.n_pages * ps;
+  const uint32_t tb = (uint32_t)ps * D * 2;
+  float* qw = q_sm + warp * D;                                    // the row's query, rotated and scaled
+#pragma unroll 1
+  for (int r = warp; r < M; r += 8) {
+    const int tok = it.q_tok0 + r / G;
+    const __nv_bfloat16* qrow = c.q + ((size_t)tok * c.n_q_heads + it.kv_head * G + r % G) * D;
+    __syncwarp();
+#pragma unroll 1
+    for (int i = lane; i < D / 2; i += 32) {
+      const float2 cs = c.pd.q_cs[(size_t)tok * (D / 2) + i];
+      const float x0 = __bfloat162float(qrow[i]), x1 = __bfloat162float(qrow[i + D / 2]);
+      qw[i] = (x0 * cs.x - x1 * cs.y) * c.scale_log2;
+      qw[i + D / 2] = (x1 * cs.x + x0 * cs.y) * c.scale_log2;
+    }
+    __syncwarp();
+    const int4 vis = misc->vis[par][r / G];
+    float m = -INFINITY, l = 0.f, acc[EPL];
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
+#pragma unroll 1
+    for (int k0 = 0; k0 < n_keys; k0 += 32) {
+      const int j = min(k0 + lane, n_keys - 1), row = j & (ps - 1), kg = it.key0 + j;
+      const int2 pg = c.pd.visit[it.page0 + j / ps];
+      const bool seen = k0 + lane < n_keys && row < (pg.y & 255) && (kg < vis.x || (kg >= vis.y && kg < vis.z) || (pg.y >> 13) * ps + row < vis.w) &&
+                        bounds_ok(c.pd, pg.x, row, ps);
+      if (!__any_sync(0xffffffffu, seen)) continue;
+      float s = -INFINITY;
+      if (seen) {
+        const char* tile = c.k_pool + ((size_t)pg.x * c.n_kv_heads + it.kv_head) * tb;
+        s = 0.f;
+#pragma unroll 2
+        for (int ch = 0; ch < D / 8; ++ch) {
+          const uint4 raw = __ldcg(reinterpret_cast<const uint4*>(tile + tile_offset(row, ch * 16, D * 2)));
+          const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&raw);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 x = __bfloat1622float2(k2[i]), w = *reinterpret_cast<const float2*>(qw + ch * 8 + 2 * i);
+            s = fmaf(w.x, x.x, s); s = fmaf(w.y, x.y, s);
+          }
+        }
+      }
+      float mn = s;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      mn = fmaxf(m, mn);
+      const float w = seen ? exp2f(s - mn) : 0.f, alpha = m == -INFINITY ? 0.f : exp2f(m - mn);
+      float sum = w;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      l = l * alpha + sum;
+      m = mn;
+#pragma unroll
+      for (int e = 0; e < EPL; ++e) acc[e] *= alpha;
+#pragma unroll 2
+      for (int kk = 0; kk < 32; ++kk) {
+        const float wk = __shfl_sync(0xffffffffu, w, kk);
+        const int page = __shfl_sync(0xffffffffu, pg.x, kk), vrow = __shfl_sync(0xffffffffu, row, kk);
+        if (wk == 0.f) continue;
+        const char* vt = c.v_pool + ((size_t)page * c.n_kv_heads + it.kv_head) * tb;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) {
+          const uint32_t bits = __ldcg(reinterpret_cast<const unsigned short*>(vt + tile_offset(vrow, (e * 32 + lane) * 2, D * 2)));
+          acc[e] = fmaf(wk, __uint_as_float(bits << 16), acc[e]);
+        }
+      }
+    }
+    const size_t at = misc->row_out[par][r];
+    if (c.out == nullptr && lane == 0) c.pd.ws_ml[at] = make_float2(m, l);
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) {
+      if (c.out != nullptr) c.out[at * D + e * 32 + lane] = __float2bfloat16_rn(acc[e] * (1.f / l));
+      else c.pd.ws_o[at * D + e * 32 + lane] = acc[e];
     }
   }
 }
@@ -442,7 +538,7 @@ __device__ __forceinline__ void finish_item(const Ctx& c, const DeviceItem& it, 
 // chose per item was 161 KB of code, and a short launch waits for
 // its instructions: 14.5 us a layer on the step above.)
 template <int D, int NR>
-__global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
+__global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const __grid_constant__ Ctx c) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
   DecMisc* misc = reinterpret_cast<DecMisc*>(smem_raw + (base - raw) + c.off_misc);
@@ -513,9 +609,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const Ctx c) {
       dead |= !mbar_wait(bars + 8 * O_FULL, item_no & 1, ab);
       tc_fence_after();
       named_sync(1, kSmThreads);                                  // the row sums of all quadrants
-      finish_item<D, NR>(c, it, misc, tmem, par, dead || *ab);
+      const bool bad = finish_item<D, NR>(c, it, misc, tmem, par, dead || *ab);
       tc_fence_before();
-      if (named_sync_or(1, kSmThreads, dead || *ab)) break;
+      if (named_sync_or(1, kSmThreads, bad || dead || *ab)) {
+        if (c.k_new != nullptr) dead |= !mbar_wait(bars + 8 * A_DONE, 0, ab);     // the step's own rows are in the pools
+        if (named_sync_or(1, kSmThreads, dead || *ab)) break;
+        redo_item<D>(c, it, misc, reinterpret_cast<float*>(smem_raw + (base - raw) + c.off_p), par);
+      }
     }
   } else if (producer) {
     // ================================ bulk-copy producers ================================

@@ -8,7 +8,9 @@ pytestmark = pytest.mark.gpu
 
 # dtype, head_dim, page size, heads, kernel
 SHAPES = [("f32", 64, 16, (4, 1), B.KERNEL_AUTO), ("f32", 128, 8, (28, 4), B.KERNEL_AUTO), ("f32", 64, 32, (64, 2), B.KERNEL_AUTO),
-          ("bf16", 128, 16, (28, 4), B.KERNEL_GENERIC), ("bf16", 64, 16, (14, 2), B.KERNEL_GENERIC)]
+          ("bf16", 128, 16, (28, 4), B.KERNEL_GENERIC), ("bf16", 64, 16, (14, 2), B.KERNEL_GENERIC),
+          ("bf16", 64, 16, (14, 2), B.KERNEL_AUTO), ("bf16", 128, 8, (28, 4), B.KERNEL_AUTO), ("bf16", 64, 32, (64, 1), B.KERNEL_AUTO),
+          ("bf16", 128, 32, (16, 2), B.KERNEL_AUTO), ("bf16", 64, 8, (4, 4), B.KERNEL_AUTO)]
 
 
 def run(dtype, d, page, heads, kernel, poison, fill=0, **kw):
@@ -23,6 +25,17 @@ def run(dtype, d, page, heads, kernel, poison, fill=0, **kw):
     for ph in wl.phases:
         r.step(ph)
     return r.outputs
+
+
+def same(out, exp, shape):
+    """Bit for bit; from the tensor-core kernel, which takes items with such values again on the CUDA cores, up to the rounding
+    to bf16 of results that agree to about 1e-6: one value of some thousands, by one step (2^-8 of the value)."""
+    if shape[0] == "f32" or shape[4] == B.KERNEL_GENERIC:
+        return np.testing.assert_array_equal(out, exp)
+    fin = np.isfinite(exp)
+    np.testing.assert_array_equal(out[~fin], exp[~fin])
+    assert np.isfinite(out[fin]).all() and np.linalg.norm(out[fin] - exp[fin]) <= 1e-3 * np.linalg.norm(exp[fin])
+    assert (out[fin] != exp[fin]).mean() <= 0.02
 
 
 @pytest.mark.parametrize("kw", [dict(), dict(n_ctas=1, fused=True), dict(n_ctas=3, fused=True, stable_cache=True)])
@@ -44,10 +57,10 @@ def test_they_reach_the_rows_that_see_them_and_no_other(shape, kw):
         for t, cells in enumerate(rows):
             for (h, e), v in cells.items():
                 exp[t, h * G:(h + 1) * G, e] = v
-        np.testing.assert_array_equal(out, exp)
+        same(out, exp, shape)
 
 
 @pytest.mark.parametrize("shape", SHAPES)
 def test_rows_that_no_token_was_written_to_do_not_matter(shape):
     for a, b in zip(run(*shape, []), run(*shape, [], fill=255)):            # 0xff bytes: NaN in either type
-        np.testing.assert_array_equal(a, b)
+        same(a, b, shape)
