@@ -389,14 +389,15 @@ int aspd_step_host_async(aspd_plan_t* plan, const void* q /*host*/, const void* 
  *
  * `plan` is a HOST-ONLY plan (aspd_tuning_t.host_only = 1; building it makes no CUDA call).
  * The call copies the plan's tables into a scratch array that is compiled into the library
- * (a file-scope __device__ array of ASPD_STATIC_SCRATCH_BYTES bytes; every GPU that loads the
+ * (a file-scope __device__ array of ASPD_STATIC_SCRATCH_BYTES and 64 KiB; every GPU that loads the
  * library holds that much memory until the process exits), runs the same split-K pass and
  * combine as aspd_branch_attn / aspd_serial_attn (by the plan's mode) with all scratch inside
  * that array, and writes `out`.  It calls no cudaMalloc / cudaFree and no allocating library
  * routine.  q, k_pool, v_pool, out are device buffers as for aspd_branch_attn.
  *
- *  - Plans whose tables plus workspace exceed ASPD_STATIC_SCRATCH_BYTES (less its last 256 bytes,
- *    which hold the status word) are rejected with ASPD_ERR_TOO_LARGE before anything is launched.
+ *  - Plans whose tables plus workspace exceed ASPD_STATIC_SCRATCH_BYTES (less 256 bytes, which hold
+ *    the status word) are rejected with ASPD_ERR_TOO_LARGE before anything is launched.  A host-only
+ *    plan that would be, but fits with fewer and longer work items, is made with those.
  *  - The first call on a device looks the array's device address up (once per device, with
  *    that device current; host threads are serialised on that look-up).  The array's memory is
  *    taken when the CUDA module that holds it is loaded, which with lazy loading may be this first

@@ -197,6 +197,8 @@ int launch_rerotate(const aspd_shape_t* shape, void* k_pool, const int32_t* page
                     int n, cudaStream_t s);
 int launch_rerotate_ranges(const aspd_shape_t* shape, void* const* k_pools, int n_layers, const int32_t* page_table,
                            const int32_t* ranges, int n_ranges, cudaStream_t s);
+// the plan's tables and records fit into the array that aspd_attn_static has for them
+bool fits_static_scratch(const aspd_plan* p);
 int set_profile_buffer(long long* device_buf, int cta);
 int launch_wait_probe(long long limit_cycles, int32_t* status_dev, cudaStream_t s);
 int launch_read_token(const aspd_shape_t* shape, const void* pool, int64_t page, int row, int kv_head,

@@ -353,9 +353,10 @@ static int plan_to_device(aspd_plan* p, cudaStream_t s);
 
 // like: the plan that this one is to take the place of (aspd_plan_update re-plans on the host for the device that
 // plan lives on): the grid of its device, its way of splitting the streams and, as far as possible, of writing new rows
+// coarse: fewer and longer items, for host-only plans whose records would not fit into the static scratch otherwise
 static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req, const aspd_branch_t* br,
                             const int32_t* page_ids, int n_req, int64_t n_pool_pages, int mode, const int32_t* q_pos,
-                            const aspd_tuning_t* tuning, void* stream, const aspd_plan* like, aspd_plan_t** plan_out) {
+                            const aspd_tuning_t* tuning, void* stream, const aspd_plan* like, bool coarse, aspd_plan_t** plan_out) {
   if (!plan_out) return ASPD_ERR_INVALID_ARG;
   *plan_out = nullptr;
   int rc = check_shape(shape);
@@ -559,13 +560,14 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   };
   build_streams(max_tok);
   const bool cores = kernel == ASPD_KERNEL_GENERIC;
-  const int tile_pages = std::max(1, (cores ? 32 : 128) / ps);
+  // pages that a CTA gets at least, and the grain of cuts inside a stream
+  const int cta_pages = coarse ? 8 : std::max(1, (cores ? 32 : 128) / ps), tile_pages = !coarse ? cta_pages : ps == 16 ? 8 : 1;
   auto ctas_for = [&](long pages) {
     // do not cut finer than one 128-key tile per CTA (measured on a 2.5 k-token step: 80 CTAs with a
     // full tile each take 10.6 us per layer, 148 CTAs with half a tile 11.9: fewer records to combine);
     // the CUDA-core kernel takes 32 keys at a time and two of its CTAs fit an SM
-    const int want = tune.n_ctas > 0 ? tune.n_ctas : p->sm_count * (cores ? 2 : 1);
-    return (int)std::max(1L, std::min((long)want, (pages + tile_pages - 1) / tile_pages));
+    const int want = tune.n_ctas > 0 ? tune.n_ctas : p->sm_count * (cores && !coarse ? 2 : 1);
+    return (int)std::max(1L, std::min((long)want, (pages + cta_pages - 1) / cta_pages));
   };
   // Dealing the streams out whole, largest first, each to the CTA with the least so far.  A stream costs its pages and
   // kDealItem more.  Returned: the largest share over the mean one.  (Rounds back and forth over the CTAs, as they were
@@ -605,7 +607,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   constexpr double kDealSkew = 1.2;
   bool deal_streams = mode == ASPD_MODE_BRANCH && !shared_mask && tune.chunk_tokens == 0 &&
                       (long)streams.size() >= 2L * ctas_for(total_pages) && (tune.n_ctas > 0 || ctas_for(total_pages) >= p->sm_count);
-  if (deal_streams && (long)streams.size() < 4L * ctas_for(total_pages)) deal_streams = deal_out(ctas_for(total_pages)) <= kDealSkew;
+  if (deal_streams && (long)streams.size() < 4L * ctas_for(total_pages)) deal_streams = !coarse && deal_out(ctas_for(total_pages)) <= kDealSkew;
   if (like) deal_streams = like->dealt != 0;
   p->wide = 0;
   if (deal_streams) {
@@ -652,7 +654,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     // Every CTA gets the same cost, cost = pages + kItemCost per item it starts: an item boundary
     // (new query tile, ragged last tile, epilogue) costs about as much as streaming a dozen pages,
     // so CTAs that end up with several short items get fewer pages.
-    const double kItemCost = (cores ? 64.0 : 192.0) / ps;
+    const double kItemCost = coarse ? 12.0 : (cores ? 64.0 : 192.0) / ps;
     // a page costs a little more the more query rows are scored against it (best measured balance:
     // 0.35 % per row), so streams of requests with many branches weigh more
     const double kRowCost = 0.0035;
@@ -665,7 +667,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     // 16.4 / 16.0 / 15.8 / 16.4), steps of 3 to 20 requests 18.9 / 18.8 / 18.7 / 18.5 / 18.5 / 18.5 (worst step against 0:
     // at 160 2.6 % slower, at 192 3.5 %, at 256 the 12 k request 11 %); 32 requests, whose CTAs have two dozen tiles
     // each, come out the same.
-    const double kWait = (kernel == ASPD_KERNEL_MMA && !p->patch_tiles) ? 160.0 / ps : 0.0;
+    const double kWait = (kernel == ASPD_KERNEL_MMA && !p->patch_tiles && !coarse) ? 160.0 / ps : 0.0;
     // the share is re-derived from what is left whenever a CTA is closed, so rounding does not pile up
     // (the sum of the waits is not known before the cuts are: made twice where there are any)
     auto cut = [&](double waits_left) {
@@ -800,7 +802,16 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
 int aspd_plan_create(const aspd_shape_t* shape, const aspd_request_t* req, const aspd_branch_t* br,
                      const int32_t* page_ids, int n_req, int64_t n_pool_pages, int mode, const int32_t* q_pos,
                      const aspd_tuning_t* tuning, void* stream, aspd_plan_t** plan_out) {
-  return plan_create_impl(shape, req, br, page_ids, n_req, n_pool_pages, mode, q_pos, tuning, stream, nullptr, plan_out);
+  const int rc = plan_create_impl(shape, req, br, page_ids, n_req, n_pool_pages, mode, q_pos, tuning, stream, nullptr, false, plan_out);
+  if (rc || !tuning || !tuning->host_only || fits_static_scratch(*plan_out)) return rc;
+  // Cut for speed, the CUDA-core kernel's steps have up to two items per SM and so twice the records of steps that
+  // give every SM one share: 28/4 heads of 128 in fp32, 16 tokens over 3 k, 9.9 MB instead of 5.0.  A host-only plan
+  // that aspd_attn_static could not take is made again with those.
+  aspd_plan_t* longer = nullptr;
+  if (plan_create_impl(shape, req, br, page_ids, n_req, n_pool_pages, mode, q_pos, tuning, stream, nullptr, true, &longer) != ASPD_OK) return rc;
+  if (fits_static_scratch(longer)) std::swap(longer, *plan_out);
+  delete longer;
+  return rc;
 }
 
 // ---- one device allocation, one staging blob ----------------------------------------------
@@ -915,7 +926,7 @@ int aspd_plan_update(aspd_plan_t* p, const aspd_request_t* req, const aspd_branc
   aspd_tuning_t tune = p->tune;
   tune.host_only = 1;
   aspd_plan* t = nullptr;
-  int rc = plan_create_impl(&p->shape, req, br, page_ids, n_req, p->n_pool_pages, p->mode, q_pos, &tune, nullptr, p, &t);
+  int rc = plan_create_impl(&p->shape, req, br, page_ids, n_req, p->n_pool_pages, p->mode, q_pos, &tune, nullptr, p, false, &t);
   if (rc) return rc;
   const aspd::PlanLayout& L = p->layout;
   if (t->n_new != p->n_new || t->n_ctas != p->n_ctas || t->kernel != p->kernel || t->wide != p->wide || t->dealt != p->dealt ||

@@ -12,9 +12,13 @@ using namespace aspd;
 
 namespace {
 
+// A CTA's entry in the table of CTAs grew from 16 to 32 bytes; what the entries take more has room of its own, so that
+// a plan of ASPD_STATIC_SCRATCH_BYTES still fits.
+constexpr size_t kHeadRoom = 64u << 10, kScratchBytes = ASPD_STATIC_SCRATCH_BYTES + kHeadRoom;
+
 // The scratch.  In host code `g_scratch` is only a handle for the symbol, not a device address;
 // the address a kernel may use comes from cudaGetSymbolAddress (below).
-static __device__ __align__(256) unsigned char g_scratch[ASPD_STATIC_SCRATCH_BYTES];
+static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
 constexpr int kMaxDevices = 64;
 unsigned char* g_scratch_addr[kMaxDevices] = {};
@@ -38,9 +42,37 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // The status word sits at a fixed place, the array's last 256 bytes, so that aspd_static_status
 // finds it whatever the last call's tables looked like.
-constexpr size_t kStatusOffset = ASPD_STATIC_SCRATCH_BYTES - 256;
+constexpr size_t kStatusOffset = kScratchBytes - 256;
+
+// Where the tables and the split-K workspace lie inside the scratch array.
+struct StaticLayout {
+  size_t items, cta, visit, tvis, rb, qcs, pbase, upload_bytes, wso, wsml, end;
+};
+StaticLayout static_layout(const aspd_plan* p) {
+  const int d = p->shape.head_dim, G = p->shape.n_q_heads / p->shape.n_kv_heads;
+  size_t off = 0;
+  auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
+  StaticLayout L;
+  L.items = take(sizeof(DeviceItem) * p->items.size());
+  L.cta = take(2 * sizeof(int4) * (size_t)(p->n_ctas > 0 ? p->n_ctas : 1));
+  L.visit = take(sizeof(int2) * p->visit.size());
+  L.tvis = take(sizeof(int4) * p->tok_vis.size());
+  L.rb = take(sizeof(int2) * p->row_blocks.size());
+  L.qcs = take(sizeof(float2) * (size_t)p->n_new * (d / 2));
+  L.pbase = take(sizeof(int32_t) * p->part_base.size());
+  L.upload_bytes = off;
+  L.wso = take(sizeof(float) * (size_t)p->n_partials * G * d);
+  L.wsml = take(sizeof(float2) * (size_t)p->n_partials * G);
+  L.end = off;
+  return L;
+}
 
 }  // namespace
+
+bool aspd::fits_static_scratch(const aspd_plan* p) {
+  const size_t heads = sizeof(int4) * (size_t)p->n_ctas;
+  return static_layout(p).end <= ASPD_STATIC_SCRATCH_BYTES - 256 + (heads < kHeadRoom ? heads : kHeadRoom);
+}
 
 extern "C" int aspd_attn_static(const aspd_plan_t* plan, const void* q, const void* k_pool, const void* v_pool, void* out,
                                 void* stream) {
@@ -54,22 +86,10 @@ extern "C" int aspd_attn_static(const aspd_plan_t* plan, const void* q, const vo
   if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess) return ASPD_ERR_CUDA;
   if (capturing != cudaStreamCaptureStatusNone) return ASPD_ERR_UNSUPPORTED;
   const aspd_shape_t& sh = plan->shape;
-  const int d = sh.head_dim, G = sh.n_q_heads / sh.n_kv_heads, n_new = plan->n_new;
+  const int d = sh.head_dim, n_new = plan->n_new;
 
-  // layout of the tables and of the split-K workspace inside the scratch array
-  size_t off = 0;
-  auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
-  const size_t o_items = take(sizeof(DeviceItem) * plan->items.size());
-  const size_t o_cta = take(2 * sizeof(int4) * (size_t)(plan->n_ctas > 0 ? plan->n_ctas : 1));
-  const size_t o_visit = take(sizeof(int2) * plan->visit.size());
-  const size_t o_tvis = take(sizeof(int4) * plan->tok_vis.size());
-  const size_t o_rb = take(sizeof(int2) * plan->row_blocks.size());
-  const size_t o_qcs = take(sizeof(float2) * (size_t)n_new * (d / 2));
-  const size_t o_pbase = take(sizeof(int32_t) * plan->part_base.size());
-  const size_t upload_bytes = off;
-  const size_t o_wso = take(sizeof(float) * (size_t)plan->n_partials * G * d);
-  const size_t o_wsml = take(sizeof(float2) * (size_t)plan->n_partials * G);
-  if (off > kStatusOffset) return ASPD_ERR_TOO_LARGE;
+  if (!aspd::fits_static_scratch(plan)) return ASPD_ERR_TOO_LARGE;
+  const StaticLayout L = static_layout(plan);
 
   unsigned char* base = nullptr;
   int rc = scratch_address(&base);
@@ -77,14 +97,14 @@ extern "C" int aspd_attn_static(const aspd_plan_t* plan, const void* q, const vo
 
   // tables: everything that must start from a known value is rewritten here (the status word
   // and the work counter start at zero; the workspace is fully written before it is read)
-  std::vector<uint8_t> blob(upload_bytes, 0);
-  memcpy(blob.data() + o_items, plan->items.data(), sizeof(DeviceItem) * plan->items.size());
-  aspd::fill_cta_head(plan, reinterpret_cast<int4*>(blob.data() + o_cta));
-  memcpy(blob.data() + o_visit, plan->visit.data(), sizeof(int2) * plan->visit.size());
-  memcpy(blob.data() + o_tvis, plan->tok_vis.data(), sizeof(int4) * plan->tok_vis.size());
-  memcpy(blob.data() + o_rb, plan->row_blocks.data(), sizeof(int2) * plan->row_blocks.size());
-  memcpy(blob.data() + o_pbase, plan->part_base.data(), sizeof(int32_t) * plan->part_base.size());
-  float2* qcs = reinterpret_cast<float2*>(blob.data() + o_qcs);
+  std::vector<uint8_t> blob(L.upload_bytes, 0);
+  memcpy(blob.data() + L.items, plan->items.data(), sizeof(DeviceItem) * plan->items.size());
+  aspd::fill_cta_head(plan, reinterpret_cast<int4*>(blob.data() + L.cta));
+  memcpy(blob.data() + L.visit, plan->visit.data(), sizeof(int2) * plan->visit.size());
+  memcpy(blob.data() + L.tvis, plan->tok_vis.data(), sizeof(int4) * plan->tok_vis.size());
+  memcpy(blob.data() + L.rb, plan->row_blocks.data(), sizeof(int2) * plan->row_blocks.size());
+  memcpy(blob.data() + L.pbase, plan->part_base.data(), sizeof(int32_t) * plan->part_base.size());
+  float2* qcs = reinterpret_cast<float2*>(blob.data() + L.qcs);
   double inv_freq[64];
   for (int i = 0; i < d / 2; ++i) inv_freq[i] = pow((double)sh.rope_theta, -2.0 * i / d);
   for (int t = 0; t < n_new; ++t)
@@ -94,7 +114,7 @@ extern "C" int aspd_attn_static(const aspd_plan_t* plan, const void* q, const vo
     }
   // the source is pageable host memory: the copy is staged before the call returns (the host may
   // wait for earlier work on the stream); the status word and the work counter start at zero
-  if (cudaMemcpyAsync(base, blob.data(), upload_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+  if (cudaMemcpyAsync(base, blob.data(), L.upload_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaMemsetAsync(base + kStatusOffset, 0, 2 * sizeof(int32_t), s) != cudaSuccess)
     return ASPD_ERR_CUDA;
 
@@ -108,17 +128,17 @@ extern "C" int aspd_attn_static(const aspd_plan_t* plan, const void* q, const vo
   shell.dealt = plan->dealt; shell.wide = plan->wide; shell.shared_mask = plan->shared_mask; shell.m64 = plan->m64; shell.dec = plan->dec; shell.max_rows = plan->max_rows;   // which kernel variant the items were made for
   shell.device_bytes = 0; shell.device_base = nullptr;
   memset(&shell.dev, 0, sizeof(shell.dev));
-  shell.dev.items = (const DeviceItem*)(base + o_items);
-  shell.dev.cta_head = (const int4*)(base + o_cta);
-  shell.dev.visit = (const int2*)(base + o_visit);
-  shell.dev.tok_vis = (const int4*)(base + o_tvis);
-  shell.dev.row_blocks = (const int2*)(base + o_rb);
-  shell.dev.q_cs = (const float2*)(base + o_qcs);
-  shell.dev.part_base = (const int32_t*)(base + o_pbase);
+  shell.dev.items = (const DeviceItem*)(base + L.items);
+  shell.dev.cta_head = (const int4*)(base + L.cta);
+  shell.dev.visit = (const int2*)(base + L.visit);
+  shell.dev.tok_vis = (const int4*)(base + L.tvis);
+  shell.dev.row_blocks = (const int2*)(base + L.rb);
+  shell.dev.q_cs = (const float2*)(base + L.qcs);
+  shell.dev.part_base = (const int32_t*)(base + L.pbase);
   shell.dev.status = (int32_t*)(base + kStatusOffset);
   shell.dev.work_counter = shell.dev.status + 1;
-  shell.dev.ws_o = (float*)(base + o_wso);
-  shell.dev.ws_ml = (float2*)(base + o_wsml);
+  shell.dev.ws_o = (float*)(base + L.wso);
+  shell.dev.ws_ml = (float2*)(base + L.wsml);
   shell.dev.pool_limit = (int32_t)plan->n_pool_pages;
 
   // plans that deal whole streams have one item per (token, KV head): their kernel writes the output
