@@ -742,12 +742,19 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   std::vector<int4> dirty;
   std::vector<int32_t> cta_dirty0(n_ctas + 1, 0);
   p->fuse_append = (kernel == ASPD_KERNEL_MMA && !shared_mask && tok_field_fits && counts_fit && p->wide != 2 && !(like && !like->fuse_append)) ? 1 : 0;
-  // A CTA with that many tiles has its rows written long before it comes to the pages that hold them, so there any
-  // number is written at its start (160 requests, 740 new rows, up to 40 per CTA and head: 205 us a layer against
-  // 212 with the append kernel; 50 requests cut into parts: 70.2 against 71.5).  Not where the tiles are patched:
-  // patch_tiles goes by the mean over the CTAs, so that one of them may be long (a forced cut every chunk_tokens
-  // keys leaves the last CTA with dozens of short tiles), and the rows' place in shared memory is kMostFusedRows long.
+  // A CTA with that many tiles has its rows written long before it comes to the pages that hold them, so there more are
+  // written at its start, as long as that does not take longer than the tiles: up to 2.5 to a tile over the step where
+  // the streams are dealt, which begin with a prefix, and one to a tile in any CTA where they are cut, since a CTA may
+  // then begin with the new rows.  8 layers from the host, us with the rows written here and by the append kernel:
+  // dealt, 0.25 to 1 a tile 1540 and 1594, 858 and 896; 1.7 to 1.8 382 and 414, 772 and 788; 2.4 585 and 569; 4.3 1250
+  // and 1103; 6 and 8 795 and 665, 765 and 630.  Cut, 0.6 to 0.7 a tile 638 and 648, 606 and 613, 608 and 614; 1.3 478
+  // and 456; 1.6 569 and 563; 5 to 8 523 and 419, 968 and 645, 1333 and 809 (branches of up to 100 tokens, 640 rows to a CTA).
+  // Not where the tiles are patched: patch_tiles goes by the mean over the CTAs, so that one of them may be long (a
+  // forced cut every chunk_tokens keys leaves the last CTA with dozens of short tiles), and the rows' place in shared
+  // memory is kMostFusedRows long.
   constexpr int kLongCta = 16;
+  long all_tiles = 0;
+  bool many = false;                               // a CTA has more than kMostFusedRows
   const bool patches = like ? like->patch_tiles != 0 : p->patch_tiles != 0;      // an update's launches are the old plan's
   if (p->fuse_append) {
     for (int c = 0; c < n_ctas && p->fuse_append; ++c) {
@@ -766,10 +773,12 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
       }
       // (32 767 tiles: what the number's field holds)
       const int rows = (int)dirty.size() - cta_dirty0[c];
-      const bool any_number = !patches && (like || (tile0 >= kLongCta && !p->dec));
-      if ((rows > kMostFusedRows && !any_number) || tile0 > 32767) p->fuse_append = 0;
+      const bool more = !patches && (like || (tile0 >= kLongCta && !p->dec && (deal_streams || rows <= tile0)));
+      if ((rows > kMostFusedRows && !more) || tile0 > 32767) p->fuse_append = 0;
+      many |= rows > kMostFusedRows; all_tiles += tile0;
     }
     cta_dirty0[n_ctas] = (int)dirty.size();
+    if (many && deal_streams && !like && dirty.size() > 2.5 * all_tiles) p->fuse_append = 0;
     if (!p->fuse_append) { dirty.clear(); std::fill(cta_dirty0.begin(), cta_dirty0.end(), 0); }
   }
   // the merge of a token's records inside the attention kernel: stream-K plans of the tensor-core kernel

