@@ -54,49 +54,78 @@ size_t rounded_size(size_t bytes, size_t least) {
   return align_up(std::max(bytes, least), std::max(least, p2 / 4));
 }
 
+// Into the park, as the latest block or as the one parked longest ago.  It keeps the blocks of the latest plans: the ones
+// parked longest ago make room.  (A park that kept the earliest ones -- a batch whose size has changed since never
+// fits them -- turned every later plan into cudaMalloc + cudaFree, i.e. a device synchronisation per step: a
+// serving mix step of 28 layers took 2.2 ms instead of 1.5 once eight other sizes had been planned.)
+void block_park(const PlanBlock& b, bool latest) {
+  std::vector<PlanBlock> evicted;
+  {
+    std::lock_guard<std::mutex> lock(g_blocks_mu);
+    g_blocks.insert(latest ? g_blocks.end() : g_blocks.begin(), b);
+    size_t parked = 0;
+    for (const PlanBlock& x : g_blocks) parked += x.bytes;
+    while (g_blocks.size() > kParkedMax || parked > kParkedMaxBytes) {
+      parked -= g_blocks.front().bytes;
+      evicted.push_back(g_blocks.front());
+      g_blocks.erase(g_blocks.begin());
+    }
+  }
+  for (PlanBlock& x : evicted) block_free(x);
+}
+
+// (The lock is held for the list alone: what waits for the GPU, allocates or frees does so with the block taken out of
+// it, so that plans of other threads, streams and devices go on.)
 int block_acquire(size_t bytes, size_t host_need, cudaStream_t s, PlanBlock* out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return ASPD_ERR_CUDA;
   bytes = rounded_size(bytes, 4u << 20); host_need = rounded_size(host_need, 64u << 10);
+  PlanBlock b;
+  int fitting = 0;
+  bool ready = false;                              // b's copy is through
   {
     std::lock_guard<std::mutex> lock(g_blocks_mu);
-    int best = -1, oldest = -1, fitting = 0;
+    int best = -1, oldest = -1;
     for (int i = 0; i < (int)g_blocks.size(); ++i) {
       if (g_blocks[i].device != dev || g_blocks[i].bytes < bytes || g_blocks[i].bytes > 4 * bytes) continue;
       ++fitting;
       if (oldest < 0) oldest = i;
       if ((best < 0 || g_blocks[i].bytes < g_blocks[best].bytes) && cudaEventQuery(g_blocks[i].upload_done) == cudaSuccess) best = i;
     }
-    // Every fitting block still has its copy queued.  A new block (device and page-locked memory) takes the host the
-    // better part of a millisecond, so a copy that is about to finish is waited for first; and with a couple of
-    // blocks parked the host is simply ahead of the GPU and waits for the oldest one instead of allocating more.
-    if (best < 0 && fitting == 1) {
-      const auto until = std::chrono::steady_clock::now() + std::chrono::microseconds(300);
-      do {
-        if (cudaEventQuery(g_blocks[oldest].upload_done) == cudaSuccess) best = oldest;
-      } while (best < 0 && std::chrono::steady_clock::now() < until);
-    }
-    if (best < 0 && fitting >= 2 && cudaEventSynchronize(g_blocks[oldest].upload_done) == cudaSuccess) best = oldest;
+    ready = best >= 0;
+    if (best < 0) best = oldest;
     if (best >= 0) {
-      PlanBlock b;
       std::swap(b, g_blocks[best]);
       g_blocks.erase(g_blocks.begin() + best);
-      int rc = ASPD_OK;
-      for (int i = 0; i < b.n_wait; ++i)
-        if (cudaStreamWaitEvent(s, b.events[i], 0) != cudaSuccess) rc = ASPD_ERR_CUDA;
-      b.n_wait = 0;
-      if (rc == ASPD_OK && b.host_bytes < host_need) {           // too small for the new tables (its last copy has completed)
-        cudaFreeHost(b.host);
-        b.host = nullptr; b.host_bytes = 0;
-        if (cudaMallocHost(&b.host, host_need) != cudaSuccess) rc = ASPD_ERR_NOMEM;
-        else b.host_bytes = host_need;
-      }
-      if (rc) { block_free(b); return rc; }
-      *out = b;
-      return ASPD_OK;
     }
   }
-  PlanBlock b;
+  // Every fitting block still has its copy queued.  A new block (device and page-locked memory) takes the host the
+  // better part of a millisecond, so a copy that is about to finish is waited for first; and with a couple of
+  // blocks parked the host is simply ahead of the GPU and waits for the oldest one instead of allocating more.
+  if (!ready && fitting == 1) {
+    const auto until = std::chrono::steady_clock::now() + std::chrono::microseconds(300);
+    do {
+      ready = cudaEventQuery(b.upload_done) == cudaSuccess;
+    } while (!ready && std::chrono::steady_clock::now() < until);
+  }
+  if (!ready && fitting >= 2) ready = cudaEventSynchronize(b.upload_done) == cudaSuccess;
+  if (ready) {
+    int rc = ASPD_OK;
+    for (int i = 0; i < b.n_wait; ++i)
+      if (cudaStreamWaitEvent(s, b.events[i], 0) != cudaSuccess) rc = ASPD_ERR_CUDA;
+    b.n_wait = 0;
+    if (rc == ASPD_OK && b.host_bytes < host_need) {             // too small for the new tables (its last copy has completed)
+      cudaFreeHost(b.host);
+      b.host = nullptr; b.host_bytes = 0;
+      if (cudaMallocHost(&b.host, host_need) != cudaSuccess) { b.host = nullptr; rc = ASPD_ERR_NOMEM; }
+      else b.host_bytes = host_need;
+    }
+    if (rc) { block_free(b); return rc; }
+    *out = b;
+    return ASPD_OK;
+  }
+  if (fitting > 0) block_park(b, false);
+  b = PlanBlock();
   b.device = dev; b.bytes = bytes; b.host_bytes = host_need;
   if (cudaMalloc(&b.ptr, bytes) != cudaSuccess) { b.ptr = nullptr; return ASPD_ERR_NOMEM; }
   if (cudaMallocHost(&b.host, host_need) != cudaSuccess) { b.host = nullptr; block_free(b); return ASPD_ERR_NOMEM; }
@@ -119,23 +148,7 @@ int block_release(PlanBlock& b, const std::vector<cudaStream_t>& streams) {
     else b.n_wait = (int)i + 1;
   }
   if (!park) return block_free(b) ? ASPD_OK : ASPD_ERR_CUDA;
-  // The park keeps the blocks of the latest plans: the ones parked longest ago make room.  (A park
-  // that kept the earliest ones -- a batch whose size has changed since never fits them -- turned
-  // every later plan into cudaMalloc + cudaFree, i.e. a device synchronisation per step: a serving
-  // mix step of 28 layers took 2.46 ms instead of 1.48 once eight other sizes had been planned.)
-  std::vector<PlanBlock> evicted;
-  {
-    std::lock_guard<std::mutex> lock(g_blocks_mu);
-    size_t parked = b.bytes;
-    for (const PlanBlock& x : g_blocks) parked += x.bytes;
-    while (!g_blocks.empty() && (g_blocks.size() >= kParkedMax || parked > kParkedMaxBytes)) {
-      parked -= g_blocks.front().bytes;
-      evicted.push_back(g_blocks.front());
-      g_blocks.erase(g_blocks.begin());
-    }
-    g_blocks.push_back(b);
-  }
-  for (PlanBlock& x : evicted) block_free(x);
+  block_park(b, true);
   return ASPD_OK;
 }
 
