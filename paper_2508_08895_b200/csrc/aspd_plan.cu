@@ -79,7 +79,9 @@ void block_park(const PlanBlock& b, bool latest) {
 int block_acquire(size_t bytes, size_t host_need, cudaStream_t s, PlanBlock* out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return ASPD_ERR_CUDA;
+  const size_t least = bytes;
   bytes = rounded_size(bytes, 4u << 20); host_need = rounded_size(host_need, 64u << 10);
+  if (bytes > kParkedMaxBytes) bytes = least;      // never parked, so there is nobody to share a size with
   PlanBlock b;
   int fitting = 0;
   bool ready = false;                              // b's copy is through
@@ -127,7 +129,12 @@ int block_acquire(size_t bytes, size_t host_need, cudaStream_t s, PlanBlock* out
   if (fitting > 0) block_park(b, false);
   b = PlanBlock();
   b.device = dev; b.bytes = bytes; b.host_bytes = host_need;
-  if (cudaMalloc(&b.ptr, bytes) != cudaSuccess) { b.ptr = nullptr; return ASPD_ERR_NOMEM; }
+  if (cudaMalloc(&b.ptr, bytes) != cudaSuccess) {
+    b.ptr = nullptr;
+    cudaGetLastError();                            // (the next launch's check would find it)
+    b.bytes = least;                               // what was added for the sake of other plans may be what does not fit
+    if (cudaMalloc(&b.ptr, least) != cudaSuccess) { b.ptr = nullptr; return ASPD_ERR_NOMEM; }
+  }
   if (cudaMallocHost(&b.host, host_need) != cudaSuccess) { b.host = nullptr; block_free(b); return ASPD_ERR_NOMEM; }
   if (cudaEventCreateWithFlags(&b.upload_done, cudaEventDisableTiming) != cudaSuccess) { b.upload_done = nullptr; block_free(b); return ASPD_ERR_CUDA; }
   *out = b;

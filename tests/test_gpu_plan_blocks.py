@@ -63,3 +63,27 @@ def test_blocks_that_change_streams_keep_the_plans_apart(n_streams):
     torch.cuda.synchronize()
     for i, out in enumerate(outs):
         assert (E.to_host_f32(out) == want[i % 3]).all(), i
+
+
+@pytest.mark.parametrize("tokens,least", [(80, 1 << 30), (160, 2 << 30)])
+def test_a_plan_that_just_fits_is_made(tokens, least):
+    """Blocks are rounded up to sizes that plans share; with less than that free, the plan's own size will do."""
+    import torch
+    wl = W.build_segment_workload("near", 3, 28, 4, 128, "bf16", 1e6, [15000], [[0] * 8], [[tokens // 8] * 8])
+    ph = wl.phases[-1]
+    make = lambda: B.Plan(_shape(wl), ph.desc, wl.n_pool_pages, B.MODE_BRANCH, chunk_tokens=16)   # noqa: E731
+    plan = make()
+    need = plan.info.workspace_bytes
+    assert least < need < least + (least >> 4)                  # a 16th above a power of two: rounded up by up to a quarter of it
+    plan.destroy()
+    torch.cuda.synchronize()
+    B.release_cached_memory()
+    torch.cuda.empty_cache()
+    spare = torch.cuda.mem_get_info()[0] - need - (96 << 20)
+    held = torch.empty(spare, dtype=torch.uint8, device="cuda")
+    plan = make()
+    assert plan.status() == 0
+    plan.destroy()
+    del held
+    torch.cuda.empty_cache()
+    B.release_cached_memory()
