@@ -24,6 +24,9 @@
  *     the library -- read tokens back with aspd_debug_read_token.  Pools must be zero-filled
  *     (or at least hold no NaN/Inf bit patterns) before their first use: the rows of a partly
  *     filled page that no token has been written to yet are multiplied by a weight of exactly 0.
+ *     The same holds for keys that a query does not see (another branch's) in bf16 with heads of
+ *     128 and pages of 16: Inf or NaN in such a key's V row reaches the query as NaN.  In fp32 and
+ *     in the other bf16 shapes it does not: those kernels leave keys of weight 0 out.
  *     Device buffers (q, out, k_new, v_new, the pools) must start on a 16-byte boundary (the
  *     kernels move them in 16-byte pieces); a call given one that does not returns
  *     ASPD_ERR_INVALID_ARG and launches nothing.
