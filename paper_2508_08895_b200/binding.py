@@ -158,8 +158,8 @@ def _stream(stream) -> Optional[int]:
 
 
 def _current_stream() -> Optional[int]:
-    """Handle of torch's current stream.  (``torch.cuda.current_stream()`` makes a Stream object first: 4.4 us
-    a call, a quarter of a step's host time; the raw handle of the current device takes 0.1 us.)"""
+    """Handle of torch's current stream.  (``torch.cuda.current_stream()`` makes a Stream object first: 4.0
+    to 4.4 us a call, a quarter of a step's host time; the raw handle of the current device takes 0.15 us.)"""
     global _raw_stream, _get_device
     if _raw_stream is None:
         import torch

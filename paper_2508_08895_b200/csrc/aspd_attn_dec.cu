@@ -18,7 +18,7 @@
 // accumulator); K and V are bf16 as stored.
 //
 // Bound by latency on the steps these shapes have so far: measured on 8 requests of 0.5-4 k tokens (14/2 heads of
-// 64, 9.4 MB a layer) 14.1 us a layer, launches included, against 1060 us with the CUDA-core kernel, whose warps walked a row's
+// 64, 9.4 MB a layer) 14.8 us a layer from the host, against 1060 us with the CUDA-core kernel, whose warps walked a row's
 // keys alone.  One CTA per SM, as many K and V tiles in flight as fit (up to four of either).
 //
 // Warp roles: 0-7 softmax, query preparation and epilogue (TMEM lane quadrant = warp % 4; warps w and w + 4
@@ -535,8 +535,8 @@ __device__ __noinline__ void redo_item(const Ctx& c, const DeviceItem it, DecMis
 
 // -------------------------------------------------------------------------------------------- the kernel
 // NR: rows that the plan's largest row block is padded to; its smaller blocks are padded as far.  (One instance that
-// chose per item was 161 KB of code, and a short launch waits for
-// its instructions: 14.5 us a layer on the step above.)
+// chose per item was 161 KB of code, these are 65 to 99, and a short launch waits for its instructions: 14.5 against
+// 14.1 us a layer in a graph on the step above.)
 template <int D, int NR>
 __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const __grid_constant__ Ctx c) {
   extern __shared__ uint8_t smem_raw[];

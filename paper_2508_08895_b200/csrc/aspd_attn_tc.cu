@@ -762,7 +762,8 @@ __device__ __forceinline__ void append_new_rows(const Ctx& c, uint32_t base, int
 // The step's new rows inside tile g of the CTA (K tile for kv = 0, V tile for 1), by the producer warp that has
 // copied the tile's pages as they were: the rows are put over what was copied, and the MMA issuer waits for the
 // slot's patch barrier before it uses such a tile.  So a page with new rows is fetched beside the append and not
-// behind it.  For plans of at most two tiles per CTA, whose time is that chain (one request of 2 k tokens, four
+// behind it.  For plans of at most two tiles per CTA on average and
+// kMostFusedRows rows in any CTA, whose time is that chain (one request of 2 k tokens, four
 // branches: 9.4 against 10.5 us a layer); with more tiles a producer that has a tile to patch gets late with its
 // next requests (32 requests, 10 tiles per CTA and more: 53.3 against 48.4 us).
 // `mine`: lane l holds dirty entry l of the CTA, which carries above its row the page's index in its tile and the
@@ -795,8 +796,8 @@ __device__ __forceinline__ bool patch_tile(uint32_t base, uint32_t bars, volatil
 // WIDE: row blocks of up to 128 query rows (plans that deal whole streams to the CTAs); one
 // query tile instead of two, Misc in the place of the second.
 // MODE: instances, not run-time switches, because a short launch is bound by fetching its instructions (a fifth of
-// all warp time on one request of 2 k tokens), and the code of a path that is not taken still separates the lines
-// of the one that is (145 KB with everything in one instance, 81 without the options: one request 9.6 -> 9.3 us a
+// all warp time on one request of 2 k tokens, 15 % with the instances), and the code of a path that is not taken still separates the lines
+// of the one that is (145 KB with everything in one instance, 74 and 80 now: one request 9.6 -> 9.3 us a
 // layer, branch-open step 16.0 -> 14.7, serial step of 32 requests 45.3 -> 43.8).
 //   kPlain
 //   kOptions   what few callers ask for: scores with M = 64, records merged inside the kernel, whole streams dealt in
