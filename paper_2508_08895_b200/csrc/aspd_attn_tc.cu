@@ -645,11 +645,10 @@ template <int U>
 struct QUnits {
   uint32_t lo[U][4], hi[U][4];   // per unit: the rotated chunk of the first and of the second span, bf16 pairs
 };
-// tile128: the rows always form a 128-row tile of their own (no replication), however few they are
 template <int NT = 128, int U = 4>
-__device__ __forceinline__ void prep_q_compute(const Ctx& c, const DeviceItem& it, int rank, int e0, QUnits<U>& qu, bool tile128 = false) {
+__device__ __forceinline__ void prep_q_compute(const Ctx& c, const DeviceItem& it, int rank, int e0, QUnits<U>& qu) {
   const int G = c.G;
-  const int M = it.n_q_tok * G, R = tile128 ? 128 : (M <= 32 ? 32 : (M <= 64 ? 64 : 128));
+  const int M = it.n_q_tok * G, R = M <= 32 ? 32 : (M <= 64 ? 64 : 128);
   uint4 a[U], b[U];
   float4 w[U][4];
 #pragma unroll
@@ -681,10 +680,9 @@ __device__ __forceinline__ void prep_q_compute(const Ctx& c, const DeviceItem& i
   }
 }
 template <int NT = 128, int U = 4>
-__device__ __forceinline__ void prep_q_store(const Ctx& c, const DeviceItem& it, uint32_t qbuf, int rank, int e0, const QUnits<U>& qu,
-                                             bool tile128 = false) {
+__device__ __forceinline__ void prep_q_store(const Ctx& c, const DeviceItem& it, uint32_t qbuf, int rank, int e0, const QUnits<U>& qu) {
   const int G = c.G;
-  const int M = it.n_q_tok * G, R = tile128 ? 128 : (M <= 32 ? 32 : (M <= 64 ? 64 : 128)), KS = (c.m64 && !tile128 ? 64 : 128) / R;
+  const int M = it.n_q_tok * G, R = M <= 32 ? 32 : (M <= 64 ? 64 : 128), KS = (c.m64 ? 64 : 128) / R;
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int e = e0 + rank + u * NT, r = e >> 3, ch = e & 7;
@@ -1270,7 +1268,7 @@ static int launch_tc(const aspd_plan* p, const void* q, const void* k_new, const
   if (p->wide == 2) {                       // row blocks of two query tiles: final outputs only
     if (c.out == nullptr) return ASPD_ERR_UNSUPPORTED;
     c.k_new = nullptr; c.v_new = nullptr;
-    return launch_pdl(attn_tc_w2_kernel, dim3(p->n_ctas), dim3(kThreads), kSmemBytesW2, s, c) == cudaSuccess ? ASPD_OK : ASPD_ERR_CUDA;
+    return launch_pdl(attn_tc_w2_kernel, dim3(p->n_ctas), dim3(kThreadsW2), kSmemBytesW2, s, c) == cudaSuccess ? ASPD_OK : ASPD_ERR_CUDA;
   }
   auto* kernel = p->wide ? attn_tc_kernel<true, kPlain>
                  : c.m64 || c.merge_out != nullptr || c.out != nullptr ? attn_tc_kernel<false, kOptions>

@@ -33,16 +33,6 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-// The same question without any waiting (try_wait may suspend the thread for a while before it answers).
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
 // Bounded wait: false means "give up" (time limit hit here or in another role).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           long long limit = kWaitCycles) {
@@ -71,7 +61,7 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
 }
-// The same two, executed by a whole warp with warp-uniform operands; lane 0 alone issues.  With
+// The commit, executed by a whole warp with warp-uniform operands; lane 0 alone issues.  With
 // uniform control flow around them the descriptors stay in the uniform datapath.
 __device__ __forceinline__ void tc_commit_lane0(uint32_t bar) {
   asm volatile(
@@ -79,25 +69,6 @@ __device__ __forceinline__ void tc_commit_lane0(uint32_t bar) {
       "mov.u32 l, %%laneid;\n\t"
       "setp.eq.u32 e, l, 0;\n\t"
       "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_mma_lane0(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p, e;\n\t.reg .u32 l;\n\t"
-      "mov.u32 l, %%laneid;\n\t"
-      "setp.eq.u32 e, l, 0;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
-}
-// A operand in tensor memory (M = 128: lane = row, 16-bit elements packed two to a column).
-__device__ __forceinline__ void tc_mma_ts_lane0(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p, e;\n\t.reg .u32 l;\n\t"
-      "mov.u32 l, %%laneid;\n\t"
-      "setp.eq.u32 e, l, 0;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
 }
 // Whole operations in one statement each, so that the issuing warp spends a handful of instructions
 // per MMA (it shares its scheduler with softmax warps; descriptor arithmetic per MMA made an
@@ -257,6 +228,12 @@ __device__ __forceinline__ bool named_sync_or(int id, int n, bool pred) {
                ::"f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), \
                  "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]), "r"(taddr) : "memory")
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// The same, with the 32 loaded values as its operands: nothing that uses them can be placed before it, while loads
+// issued after it may still be on their way.
+#define ASPD_RW8(v, o) "+f"(v[o + 0]), "+f"(v[o + 1]), "+f"(v[o + 2]), "+f"(v[o + 3]), "+f"(v[o + 4]), "+f"(v[o + 5]), "+f"(v[o + 6]), "+f"(v[o + 7])
+__device__ __forceinline__ void tmem_wait_ld32(float (&v)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : ASPD_RW8(v, 0), ASPD_RW8(v, 8), ASPD_RW8(v, 16), ASPD_RW8(v, 24)::"memory");
+}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Shared-memory matrix descriptor, 128-byte swizzle, descriptor version 1.
@@ -273,25 +250,6 @@ __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-// 2^x for two values on the FMA and integer pipes instead of the special-function unit (which takes
-// a warp's instruction only every 8 cycles): x = n + f with n the nearest integer (the magic-number
-// addition leaves n in the low bits), 2^f by a cubic (largest relative error 8e-5 on [-1/2, 1/2],
-// a twenty-fifth of what rounding the result to bf16 costs), n added to the exponent bits.  The
-// argument is clamped to the exponent range, so that a huge value still ends far above 2^40 and a
-// tiny one near 2^-126.
-__device__ __forceinline__ float2 ex2_fma2(float2 x) {
-  x.x = fminf(fmaxf(x.x, -126.f), 127.f);
-  x.y = fminf(fmaxf(x.y, -126.f), 127.f);
-  const float2 magic = make_float2(12582912.f, 12582912.f);
-  const float2 t = __fadd2_rn(x, magic);
-  const float2 n = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
-  const float2 f = __ffma2_rn(n, make_float2(-1.f, -1.f), x);
-  float2 p = __ffma2_rn(f, make_float2(0.05519810691f, 0.05519810691f), make_float2(0.24267712235f, 0.24267712235f));
-  p = __ffma2_rn(p, f, make_float2(0.69326180220f, 0.69326180220f));
-  p = __ffma2_rn(p, f, make_float2(0.99992275238f, 0.99992275238f));
-  return make_float2(__int_as_float(__float_as_int(p.x) + (__float_as_int(t.x) << 23)),
-                     __int_as_float(__float_as_int(p.y) + (__float_as_int(t.y) << 23)));
 }
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
