@@ -43,6 +43,7 @@ constexpr int W_KPROD = 8, W_MMA = 9, W_VPROD = 11, W_EPI = 12;   // warp roles 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRaise = 8.0f;                 // raise the reference maximum only beyond 2^8
 constexpr float kLazyLimit = 1099511627776.0f;  // 2^40: a tile's sum of exponentials beyond which the reference is raised
+constexpr float kLazyLow = 8.673617e-19f;      // 2^-60: a sum of a row's first exponentials below which the reference is lowered
 constexpr float kLower = 32.0f;                // wide variant: lower the initial reference (0) when a row's first keys are below 2^-32
 
 constexpr uint32_t kTileBytes = 32768;         // one K, V, Q or P tile: 128 rows x 256 B
@@ -167,7 +168,8 @@ __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it,
   const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
   const bool o_owner = half == 0 && (warp & 3) < R / 32;   // threads whose TMEM lane holds a row of O
   const int ob = item_no & 1;
-  float m_ref = -INFINITY, l = 0.f;
+  float m_ref = 0.f, l = 0.f;
+  bool seen = false;   // this thread has had a key that its row sees
   bool dead = false;   // a wait gave up: keep walking the same control flow, report at the end
   for (int t = 0; t < n_tiles; ++t, ++g) {
     const int sb = g & 1;
@@ -180,16 +182,16 @@ __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it,
     else ASPD_TMEM_LD16(s_addr, s, 0);
     tmem_wait_ld();
     if (tid == 0) ASPD_STAMP(c, g, 1);
-    // After an item's first tile the rows have a reference maximum, and a tile's exponentials are
-    // taken against it right away: one pass (mask, packed fp32 pairs, the exponentials), no maximum,
-    // no exchange between the threads of a row.  The reference then stays where it is unless an
-    // exponent passes 2^40, which shows in the sum; the barrier below ORs that over the CTA and the
+    // A tile's exponentials are taken against the row's reference as it is, 0 at the item's start: one pass (mask,
+    // packed fp32 pairs, the exponentials), no maximum, no exchange between the threads of a row.  The reference
+    // stays where it is unless an exponent passes 2^40, or the first keys of a row are so far below it that their
+    // exponentials could vanish, which shows in the sum; the barrier below ORs that over the CTA and the
     // tile is redone the long way (scores read again from TMEM, row maximum exchanged, reference
-    // raised, O rescaled).  Everything is floating point, so a reference up to 2^40 below a row's
-    // true maximum costs no precision.
-    bool lazy = t > 0;
-    if (lazy) {
-      if (m_ref == -INFINITY) m_ref = 0.f;        // the row has seen nothing so far (l and O are 0): any reference will do
+    // moved, O rescaled).  Everything is floating point, so a reference up to 2^40 below or 2^60 above a row's
+    // true maximum costs no precision.  (The first tile went the long way always: 28 layers of one request of
+    // 2 k keys 284 -> 275 us, of a serial step over 1.1 k 219 -> 209.)
+    bool lazy, any = false;                        // any: a key of this tile that the row sees
+    {
       float2 lsum = make_float2(0.f, 0.f);
       const float2 sc2 = make_float2(c.scale_log2, c.scale_log2), nm2 = make_float2(-m_ref, -m_ref);
 #pragma unroll
@@ -198,6 +200,7 @@ __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it,
         const int kb = it.key0 + t * kTile + col0 + pg * 16;
         const uint32_t mask = bits_between(0, min(nv, vis.x - kb)) | bits_between(vis.y - kb, min(nv, vis.z - kb)) |
                               bits_between(0, min(nv, vis.w - (ye >> 13) * 16));
+        any |= mask != 0;
 #pragma unroll
         for (int i = 0; i < 16; i += 2) {
           float2 x = __ffma2_rn(make_float2(s[pg * 16 + i], s[pg * 16 + i + 1]), sc2, nm2);
@@ -211,7 +214,7 @@ __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it,
         }
       }
       const float tsum = lsum.x + lsum.y;
-      lazy = !named_sync_or(1, kSoftmaxThreads, !(tsum <= kLazyLimit));
+      lazy = !named_sync_or(1, kSoftmaxThreads, !(tsum <= kLazyLimit) || (any && !seen && tsum < kLazyLow));
       if (lazy) {
         l += tsum;
       } else {                                     // rare: the scores again, then the long way
@@ -245,15 +248,20 @@ __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it,
     }
     mx *= c.scale_log2;                           // the scale is positive: max commutes with it
     misc->smax[sb][tid] = mx;
+    misc->smax[sb ^ 1][tid] = seen ? 1.f : 0.f;
     named_sync(1, kSoftmaxThreads);
-    float m_tile = mx;
+    float m_tile = mx, row_seen = 0.f;            // row_seen: one of the row's threads had a key before
 #pragma unroll
-    for (int jj = 0; jj < KS; ++jj)
+    for (int jj = 0; jj < KS; ++jj) {
       m_tile = fmaxf(m_tile, fmaxf(misc->smax[sb][jj * R + r], misc->smax[sb][128 + jj * R + r]));
-    const bool upd = m_tile > m_ref + kRaise;     // also true for the first finite maximum (m_ref = -inf)
+      row_seen = fmaxf(row_seen, fmaxf(misc->smax[sb ^ 1][jj * R + r], misc->smax[sb ^ 1][128 + jj * R + r]));
+    }
+    const float old = row_seen > 0.f ? m_ref : -INFINITY;      // a row that has seen nothing (l and O are 0) takes any
+    const bool upd = m_tile > old + kRaise;       // also true for the first finite maximum (old = -inf)
     float alpha = 1.f;
-    if (upd) { alpha = ex2(m_ref - m_tile); m_ref = m_tile; }
+    if (upd) { alpha = ex2(old - m_tile); m_ref = m_tile; }
     l *= alpha;
+    named_sync(1, kSoftmaxThreads);               // both arrays are read
     if (t > 0 && c.pv64) {
       // O comes from an M = 64 MMA: row 16 q + i sits in lane i of quadrant q, which is not the lane of
       // the thread that knows the row's factor.  The factors go through shared memory (the other score
@@ -299,9 +307,8 @@ __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it,
         tc_fence_before();
       }
     }
-    const float nmsafe = m_ref == -INFINITY ? 0.f : -m_ref;
     float2 lsum = make_float2(0.f, 0.f);
-    const float2 sc2 = make_float2(c.scale_log2, c.scale_log2), nm2 = make_float2(nmsafe, nmsafe);
+    const float2 sc2 = make_float2(c.scale_log2, c.scale_log2), nm2 = make_float2(-m_ref, -m_ref);
 #pragma unroll
     for (int i = 0; i < HC; i += 2) {             // p = 2^(s * scale - m): packed fp32 pairs (one FFMA, one FADD per two scores), two MUFU
       float2 x = __ffma2_rn(make_float2(s[i], s[i + 1]), sc2, nm2);
@@ -311,6 +318,7 @@ __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it,
     }
     l += lsum.x + lsum.y;
     }
+    seen |= any;
     tc_fence_before();
     mbar_arrive(bars + 8 * (S_EMPTY + sb));       // the scores are not needed again
     if (tid == 0) ASPD_STAMP(c, g, 3);
