@@ -131,7 +131,7 @@ __device__ __forceinline__ void drain_merge_queue(const Ctx& c, const Misc* misc
   for (int u = warp_rank; u < n; u += n_warps) {
     const int idx = misc->mq[u / G][0], g = u % G, tok = idx / c.n_kv_heads, h = idx % c.n_kv_heads;
     const int p0 = misc->mq[u / G][1], np = misc->mq[u / G][2];
-    combine_row<__nv_bfloat16, 128>(c.pd.ws_o, c.pd.ws_ml, p0, np, G, g, lane, c.merge_out + ((size_t)tok * c.n_q_heads + h * G + g) * 128);
+    combine_row<__nv_bfloat16, 128, 1>(c.pd.ws_o, c.pd.ws_ml, p0, np, G, g, lane, c.merge_out + ((size_t)tok * c.n_q_heads + h * G + g) * 128);
   }
 }
 

@@ -127,6 +127,7 @@ struct aspd_plan {
   int m64 = 0;                     // stream-K plan of the tensor-core kernel whose MMAs take M = 64 (row blocks are at most 64 rows)
   int dec = 0;                     // tensor-core plan of a shape that aspd_attn_dec.cu serves (head_dim 64, pages of 8 or 32)
   int max_rows = 0;                // largest number of query rows of an item
+  int max_parts = 0;               // largest number of records of a (token, KV head)
   int stagger_start = 0;           // few tiles per CTA: order the requests of a CTA's first tiles (see the producers)
   int patch_tiles = 0;             // at most two tiles per CTA on average: a fused step puts the new rows into the tiles (see patch_tile)
   int single_launch = 0;           // stream-K plan of the tensor-core kernel whose last-arriving CTAs merge the records themselves
@@ -159,6 +160,10 @@ namespace aspd {
 // launch latency and set-up of a kernel overlap the tail of the one before it.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// A value that is the same in all lanes of a (converged) warp, known to the compiler as such: loops and branches on it
+// need no divergence handling and what it feeds stays in uniform registers.
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,

@@ -452,19 +452,16 @@ __global__ void __launch_bounds__(kGenThreads, 2) attn_generic_kernel(PlanDevice
 // ------------------------------------------------------------------------------ combine
 // One warp per (new token, query head): merge the partial records of (token, KV head) by
 // log-sum-exp in one pass with a running maximum.  Where the records lie is plan data and is
-// read before the dependency wait; then each round loads the (max, sum) pairs of eight records
-// and their O rows together, so a row with up to eight records costs one memory round trip.
-template <typename T, int D>
-__global__ void combine_kernel(PlanDevice pd, T* __restrict__ out, int n_new, int n_q_heads, int n_kv_heads) {
+// read before the dependency wait.
+template <typename T, int D, int NB>
+__global__ void __launch_bounds__(128) combine_kernel(PlanDevice pd, T* __restrict__ out, int n_q_heads, int n_kv_heads, int G) {
   pdl_launch_dependents();
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  const bool active = w < n_new * n_q_heads;
-  const int tok = active ? w / n_q_heads : 0, hq = active ? w % n_q_heads : 0;
-  const int G = n_q_heads / n_kv_heads, h = hq / G, g = hq % G;
-  const int p0 = pd.part_base[tok * n_kv_heads + h], n = pd.part_base[tok * n_kv_heads + h + 1] - p0;
+  // (what all lanes agree on is taken from lane 0, which lets the compiler know: 9 instead of 15 KB of code)
+  const int tok = blockIdx.x, hq = blockIdx.y * 4 + uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int h = min(hq, n_q_heads - 1) / G, g = hq - h * G;
+  const int p0 = uniform(pd.part_base[tok * n_kv_heads + h]), n = uniform(pd.part_base[tok * n_kv_heads + h + 1]) - p0;
   pdl_wait();
-  if (!active) return;
-  combine_row<T, D, true>(pd.ws_o, pd.ws_ml, p0, n, G, g, lane, out + ((size_t)tok * n_q_heads + hq) * D);
+  if (hq < n_q_heads) combine_row<T, D, NB>(pd.ws_o, pd.ws_ml, p0, n, G, g, lane, out + ((size_t)tok * n_q_heads + hq) * D);
 }
 
 template <typename T>
@@ -530,8 +527,8 @@ int launch_qcs(const aspd_plan* p, cudaStream_t s) {
   return check_launch();
 }
 
-template <typename T, int D>
-static int launch_combine_of(const aspd_plan* p, void* out, cudaStream_t s) {
+template <typename T, int D, int NB>
+static int launch_combine_rows(const aspd_plan* p, void* out, cudaStream_t s) {
   const aspd_shape_t& sh = p->shape;
   static int sms[64] = {};                         // per device: SMs, known once the kernel has been configured there
   int dev = 0;
@@ -539,7 +536,7 @@ static int launch_combine_of(const aspd_plan* p, void* out, cudaStream_t s) {
   int n_sms = dev >= 0 && dev < 64 ? sms[dev] : 0;
   if (n_sms == 0) {
     if (cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(combine_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombineClaim) != cudaSuccess)
+        cudaFuncSetAttribute(combine_kernel<T, D, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombineClaim) != cudaSuccess)
       return ASPD_ERR_CUDA;
     if (dev >= 0 && dev < 64) sms[dev] = n_sms;
   }
@@ -551,9 +548,19 @@ static int launch_combine_of(const aspd_plan* p, void* out, cudaStream_t s) {
   // 330 / 306, one token after another over 1 k 255 / 213 / 213, eight branches over 16 k 517 / 627 / 495, eight
   // requests with heads of 64 410 / 402 / 364.  A grid larger than the chip spreads anyway, and would run in waves
   // (six branches opened with twelve tokens each, 504 blocks: 480 / 438 / 524).
-  const int blocks = (p->n_new * sh.n_q_heads + 3) / 4;
+  const dim3 grid((unsigned)p->n_new, (unsigned)(sh.n_q_heads + 3) / 4);
+  const long blocks = (long)grid.x * grid.y;
   const size_t claim = blocks <= n_sms ? kCombineClaim : 0;
-  return status_of(launch_pdl(combine_kernel<T, D>, dim3(blocks), dim3(128), claim, s, p->dev, (T*)out, p->n_new, sh.n_q_heads, sh.n_kv_heads));
+  return status_of(launch_pdl(combine_kernel<T, D, NB>, grid, dim3(128), claim, s, p->dev, (T*)out, sh.n_q_heads, sh.n_kv_heads, sh.n_q_heads / sh.n_kv_heads));
+}
+
+template <typename T, int D>
+static int launch_combine_of(const aspd_plan* p, void* out, cudaStream_t s) {
+  // as many records in flight as the plan's rows have, up to 32: more take registers, and with them blocks from an SM
+  // (504 blocks of rows with six records at three: 418 us a pass of 28 layers, at one 395)
+  const int nb = (p->max_parts + 7) / 8;
+  return nb <= 1 ? launch_combine_rows<T, D, 1>(p, out, s) : nb == 2 ? launch_combine_rows<T, D, 2>(p, out, s)
+       : nb == 3 ? launch_combine_rows<T, D, 3>(p, out, s) : launch_combine_rows<T, D, 4>(p, out, s);
 }
 
 int launch_combine(const aspd_plan* p, void* out, cudaStream_t s) {

@@ -814,6 +814,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   // more than the combine launch costs, whose blocks are resident and waiting when the pass ends.
   p->single_launch = (kernel == ASPD_KERNEL_MMA && !deal_streams && !p->dec && tune.combine == ASPD_COMBINE_FUSED && max_tok <= 16) ? 1 : 0;   // 16: an item's tokens in the merge queue
   for (size_t i = 0; i < n_parts.size(); ++i) part_base[i + 1] = part_base[i] + n_parts[i];
+  for (int n : n_parts) p->max_parts = std::max(p->max_parts, n);
   p->n_items = (int)p->items.size();
   p->n_partials = part_base[n_parts.size()];
   p->kv_tokens_read = kv_tokens;
@@ -971,7 +972,7 @@ int aspd_plan_update(aspd_plan_t* p, const aspd_request_t* req, const aspd_branc
   }
   // the page-locked buffer is written again: its previous copy must be through
   if (cudaEventSynchronize(p->block.upload_done) != cudaSuccess) { delete t; return ASPD_ERR_CUDA; }
-  p->n_req = t->n_req; p->n_items = t->n_items; p->n_partials = t->n_partials; p->n_row_blocks = t->n_row_blocks;
+  p->n_req = t->n_req; p->n_items = t->n_items; p->n_partials = t->n_partials; p->n_row_blocks = t->n_row_blocks; p->max_parts = t->max_parts;
   p->kv_tokens_read = t->kv_tokens_read; p->algorithmic_bytes = t->algorithmic_bytes;
   p->items.swap(t->items); p->visit.swap(t->visit); p->tok_vis.swap(t->tok_vis); p->cta_item0.swap(t->cta_item0);
   p->part_base.swap(t->part_base); p->q_pos.swap(t->q_pos); p->row_blocks.swap(t->row_blocks);
