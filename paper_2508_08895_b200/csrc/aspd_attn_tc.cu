@@ -39,7 +39,7 @@ namespace {
 constexpr int kTile = 128;                     // keys per tile
 constexpr int kThreads = 512;
 constexpr int kSoftmaxThreads = 256;           // two warps per TMEM lane quadrant, each taking half of the columns
-constexpr int W_KPROD = 8, W_MMA = 9, W_VPROD = 11, W_EPI = 12;   // warp roles (0-7 softmax, 10 idle, 12-15 epilogue)
+constexpr int W_KPROD = 8, W_MMA = 9, W_IDLE = 10, W_VPROD = 11, W_EPI = 12;   // warp roles (0-7 softmax, 10 only set-up, 12-15 epilogue)
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRaise = 8.0f;                 // raise the reference maximum only beyond 2^8
 constexpr float kLazyLimit = 1099511627776.0f;  // 2^40: a tile's sum of exponentials beyond which the reference is raised
@@ -138,10 +138,10 @@ __device__ __forceinline__ void drain_merge_queue(const Ctx& c, const Misc* misc
 // r / G of a row index below 256 (G is at most 64): a division by a run-time number is some forty instructions
 __device__ __forceinline__ int token_of(const Ctx& c, int r) { return (r * c.inv_g) >> 16; }
 
-// Item idx of this CTA (rel = idx - item_begin): from the shared-memory cache when it is there.
+// Item idx of this CTA (rel = idx - item_begin): from the shared-memory cache when it is there.  Called by whole warps.
 __device__ __forceinline__ DeviceItem get_item(const Ctx& c, const Misc* misc, int idx, int item_begin) {
   const int rel = idx - item_begin;
-  return rel < kItemCache ? misc->items[rel] : c.pd.items[idx];
+  return uniform_item(rel < kItemCache ? misc->items[rel] : c.pd.items[idx]);
 }
 
 // ------------------------------------------------------------------------------- softmax role
@@ -155,7 +155,7 @@ template <int NC>   // NC = padded row count R = columns of a row replica; a thr
 __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it, Misc* misc, uint32_t bars, uint32_t smem_p,
                                              uint32_t tmem, int item_no, int& g) {   // item_no = index among this CTA's items
   constexpr int R = NC, KS = 128 / NC, HC = NC / 2;
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5);
   const int tmem_lane = tid & 127, half = tid >> 7;     // of the thread; which half of the replica's columns
   const int r = tmem_lane % R, j = tmem_lane / R;
   const int col0 = j * NC + half * HC;           // first tile column (key) of this thread
@@ -524,7 +524,7 @@ __device__ __forceinline__ bool softmax_item_m64(const Ctx& c, const DeviceItem&
 // visible key) the reference is raised and the warp repeats the pass from TMEM.
 __device__ __forceinline__ bool softmax_item_wide(const Ctx& c, const DeviceItem& it, Misc* misc, uint32_t bars, uint32_t smem_p,
                                                   uint32_t tmem, int item_no, int& g) {
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5);
   const int r = tid & 127, half = tid >> 7;
   const int col0 = half * 64;
   const int G = c.G, M = it.n_q_tok * G;
@@ -820,12 +820,26 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
   constexpr uint32_t off_misc = WIDE ? OFF_MISC_WIDE : OFF_MISC;
   Misc* misc = reinterpret_cast<Misc*>(smem + off_misc);
   const uint32_t bars = base + off_misc;          // bars[] is the first member of Misc
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   volatile int* ab = &misc->abort_flag;
   if (tid == 0) ASPD_CTA_STAMP(c, 0);
   if (tid == 0) pdl_launch_dependents();
   const int4 head = c.pd.cta_head[2 * blockIdx.x], head2 = c.pd.cta_head[2 * blockIdx.x + 1];
-  const int item_begin = head.x, item_end = head.y;
+  // barriers and tensor memory by two warps that have no part in the tables, while those are on their way
+  if (warp == W_MMA) {
+    auto of = [](int first, int n) { return ((1u << n) - 1u) << first; };
+    const uint32_t by256 = of(S_EMPTY, 2) | of(P_FULL, 1) | of(Q_FULL, 2) | of(E_FULL, 2), by128 = of(O_EMPTY, 2) | of(A_DONE, 1);
+    static_assert(NUM_BARS <= 32, "a lane initialises one of them");
+    if (lane < NUM_BARS) mbar_init(bars + 8 * lane, (by256 >> lane) & 1u ? 256 : (by128 >> lane) & 1u ? 128 : 1);
+    if (lane == 0) { misc->abort_flag = 0; misc->mq_n = 0; }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == W_IDLE) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&misc->tmem_base)), "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  const int item_begin = uniform(head.x), item_end = uniform(head.y);
   // Plan tables do not depend on earlier kernels of the stream: the CTA's items and, for the
   // producers, the first batch of page entries (whose place comes with the head entry, so that it
   // is the second load of the kernel, not the fourth) are fetched while the CTA is still setting up.
@@ -833,7 +847,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
   if ((warp == W_KPROD || warp == W_VPROD) && lane < head.w) first_pages = c.pd.visit[head.z + lane];
   // fused step: the CTA's new rows (plan data), an entry per lane of the warps that deal with them
   // (PATCH: the planner lists at most kMostFusedRows of a CTA for such launches; no more than that ever has a place)
-  const int dirty_rows = c.k_new == nullptr ? 0 : PATCH ? min(head2.y, kMostFusedRows) : head2.y;
+  const int dirty_rows = c.k_new == nullptr ? 0 : uniform(PATCH ? min(head2.y, kMostFusedRows) : head2.y);
   const bool patch = PATCH && dirty_rows > 0;
   int4 dirty = make_int4(0, 0, 0, -1);
   if (warp >= W_KPROD && lane < dirty_rows) dirty = c.pd.dirty[head2.x + lane];
@@ -841,25 +855,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
     const int n_cached = min(item_end - item_begin, kItemCache);
     for (int e = tid; e < n_cached * (int)(sizeof(DeviceItem) / 4); e += kThreads)
       reinterpret_cast<int*>(misc->items)[e] = reinterpret_cast<const int*>(c.pd.items + item_begin)[e];
-    for (int e = tid; e < n_cached * kMaxTokPerItem; e += kThreads) {
-      const DeviceItem& ci = c.pd.items[item_begin + e / kMaxTokPerItem];
-      const int tl = e % kMaxTokPerItem;
-      if (tl < ci.n_q_tok) misc->vis[e / kMaxTokPerItem][tl] = c.pd.tok_vis[ci.q_tok0 + tl];
-    }
   }
 
-  if (tid == 0) {
-    const int counts[NUM_BARS] = {1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 256, 256, 256, 1, 1, 1, 128, 128, 256, 256, 1, 1, 256, 256, 1, 1, 1, 1, 128};
-    for (int i = 0; i < NUM_BARS; ++i) mbar_init(bars + 8 * i, counts[i]);
-    misc->abort_flag = 0;
-    misc->mq_n = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&misc->tmem_base)), "r"(512u)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -869,6 +866,17 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
   // With the plan's stable-cache promise the two producer warps go ahead and fetch pages that
   // hold no new rows; they wait themselves before the first page that does.
   const bool producer_runs_ahead = c.early_fetch && (warp == W_KPROD || warp == W_VPROD);
+  // (The ranges of the items' tokens are the third of a chain of loads.  Only the softmax warps use them, so the other
+  // roles do not wait for them at the barrier above.  With that, and barriers and tensor memory set up beside the loads
+  // of the tables: 28 layers of 17 k keys 406 -> 385 us, of 32 requests 1 346 -> 1 320.)
+  if (warp < 8) {
+    const int n_cached = min(item_end - item_begin, kItemCache);
+    for (int e = tid; e < n_cached * kMaxTokPerItem; e += kSoftmaxThreads) {
+      const DeviceItem& ci = misc->items[e / kMaxTokPerItem];
+      const int tl = e % kMaxTokPerItem;
+      if (tl < ci.n_q_tok) misc->vis[e / kMaxTokPerItem][tl] = c.pd.tok_vis[ci.q_tok0 + tl];
+    }
+  }
   if (!producer_runs_ahead) pdl_wait();
   if (tid == 0) ASPD_CTA_STAMP(c, 1);
 
@@ -876,9 +884,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
     // =============================== softmax ===============================
     // The first query tile, while the first K/V tiles are in flight and the epilogue threads write the new rows.
     if (item_begin < item_end) {
-      prep_q<kSoftmaxThreads, WIDE ? 4 : 2>(c, misc->items[0], base + OFF_Q, tid);
+      prep_q<kSoftmaxThreads, WIDE ? 4 : 2>(c, get_item(c, misc, item_begin, item_begin), base + OFF_Q, tid);
       fence_async_smem();
       mbar_arrive(bars + 8 * Q_FULL);
+      named_sync(1, kSoftmaxThreads);              // the items' ranges are there
     }
     int g = 0, item_no = 0;
     for (int idx = item_begin; idx < item_end; ++idx, ++item_no) {
@@ -1035,9 +1044,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
       int g = 0, item_no = 0;
       bool ok = true, have_prev = false;
       TileRef prev = {0, 0, 0, 0, 0, 0, 0};
-      const int ib = __shfl_sync(full_mask, item_begin, 0), ie = __shfl_sync(full_mask, item_end, 0);
+      const int ib = item_begin, ie = item_end;
       for (int idx = ib; idx < ie && ok; ++idx, ++item_no) {
-        const int n_pages = __shfl_sync(full_mask, get_item(c, misc, idx, ib).n_pages, 0), n_tiles = (n_pages + 7) >> 3;
+        const int n_pages = get_item(c, misc, idx, ib).n_pages, n_tiles = (n_pages + 7) >> 3;
         for (int t = 0; t < n_tiles && ok; ++t, ++g) {
           TileRef cur = {min(8, n_pages - t * 8), t == 0, t == n_tiles - 1, WIDE ? 0 : item_no & 1, item_no & 1, item_no, 0};
           ok = issue_s(cur, g);
@@ -1217,7 +1226,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(Ctx c) {
   tc_fence_before();
   __syncthreads();
   if (tid == 0) ASPD_CTA_STAMP(c, 3);
-  if (warp == 0) {
+  if (warp == W_IDLE) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
   }

@@ -60,7 +60,7 @@ static_assert(sizeof(MiscW2) <= 2048, "MiscW2 must fit behind the tiles");
 
 __device__ __forceinline__ DeviceItem get_item_w2(const Ctx& c, const MiscW2* misc, int idx, int item_begin) {
   const int rel = idx - item_begin;
-  return rel < kItemCacheW2 ? misc->items[rel] : c.pd.items[idx];
+  return uniform_item(rel < kItemCacheW2 ? misc->items[rel] : c.pd.items[idx]);
 }
 
 // One arrival per warp: what its lanes did before is ordered by the warp barrier.
@@ -111,7 +111,7 @@ __device__ __forceinline__ void prep_tile_w2(const Ctx& c, int q_tok0, int n_tok
 // One softmax group over all items of the CTA.  grp = 0 / 1, r = the thread's row in its tile.
 __device__ __forceinline__ void softmax_group_w2(const Ctx& c, MiscW2* misc, uint32_t bars, uint32_t base, uint32_t tmem, int item_begin,
                                                  int item_end, int grp, int tpt) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r = tid & 127;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31, r = tid & 127;
   const int G = c.G;
   volatile int* ab = &misc->abort_flag;
   const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
@@ -322,12 +322,12 @@ __global__ void __launch_bounds__(kThreadsW2, 1) attn_tc_w2_kernel(Ctx c) {
   uint8_t* smem = smem_raw + (base - raw);
   MiscW2* misc = reinterpret_cast<MiscW2*>(smem + W2_OFF_MISC);
   const uint32_t bars = base + W2_OFF_MISC;       // bars[] is the first member
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   volatile int* ab = &misc->abort_flag;
   if (tid == 0) ASPD_CTA_STAMP(c, 0);
   if (tid == 0) pdl_launch_dependents();
   const int4 head = c.pd.cta_head[2 * blockIdx.x];
-  const int item_begin = head.x, item_end = head.y;
+  const int item_begin = uniform(head.x), item_end = uniform(head.y);
   int2 first_pages = make_int2(0, 0);
   if ((warp == W2_KPROD || warp == W2_VPROD) && lane < head.w) first_pages = c.pd.visit[head.z + lane];
   {
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(kThreadsW2, 1) attn_tc_w2_kernel(Ctx c) {
     const int grp = warp - W2_ISSUE;
     const uint32_t fm = 0xffffffffu;
     const uint32_t tmem_u = __shfl_sync(fm, tmem, 0), base_u = __shfl_sync(fm, base, 0), bars_u = base_u + W2_OFF_MISC;
-    const int ib = __shfl_sync(fm, item_begin, 0), ie = __shfl_sync(fm, item_end, 0);
+    const int ib = item_begin, ie = item_end;
     auto wait_all = [&](uint32_t bar, uint32_t parity) { return __all_sync(fm, mbar_wait(bar, parity, ab)) != 0; };
     // A parity only tells the two latest phases of a barrier apart.  Group 1 is absent from items with
     // a single query tile, so its cursor may come to an item that group 0 has not reached yet and
@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(kThreadsW2, 1) attn_tc_w2_kernel(Ctx c) {
     bool ok = true;
     for (int idx = ib; idx < ie && ok; ++idx) {
       const DeviceItem it = get_item_w2(c, misc, idx, ib);
-      const int n_pages = __shfl_sync(fm, it.n_pages, 0), n_q_tok = __shfl_sync(fm, it.n_q_tok, 0), n_tiles = (n_pages + 7) >> 3;
+      const int n_pages = it.n_pages, n_q_tok = it.n_q_tok, n_tiles = (n_pages + 7) >> 3;
       if (n_q_tok > grp * tpt) {
         const bool both = n_q_tok > tpt;
         // a K or V tile is free when both groups are through with it; a group that is absent has its share done here

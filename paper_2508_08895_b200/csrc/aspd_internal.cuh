@@ -164,6 +164,10 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // A value that is the same in all lanes of a (converged) warp, known to the compiler as such: loops and branches on it
 // need no divergence handling and what it feeds stays in uniform registers.
 __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+__device__ __forceinline__ DeviceItem uniform_item(const DeviceItem& it) {       // (fields that nobody reads cost nothing)
+  return {uniform(it.q_tok0), uniform(it.n_q_tok), uniform(it.kv_head), uniform(it.page0), uniform(it.n_pages), uniform(it.key0),
+          uniform(it.part_slot), uniform(it.request), uniform(it.row_block), uniform(it.n_parts)};
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
