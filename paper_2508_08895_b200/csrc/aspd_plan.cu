@@ -646,16 +646,17 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   }
   p->max_rows = 0;
   for (const int2& rb : row_blocks) p->max_rows = std::max(p->max_rows, rb.y * G);
-  const int n_ctas = ctas_for(total_pages);
+  const int base_ctas = ctas_for(total_pages);
+  int n_ctas = like && like->tile_cut ? like->n_ctas : base_ctas;
   const int chunk_pages = tune.chunk_tokens > 0 ? tune.chunk_tokens / ps : (1 << 28);
-  p->chunk_tokens = tune.chunk_tokens; p->n_ctas = n_ctas;
+  p->chunk_tokens = tune.chunk_tokens; p->base_ctas = base_ctas;
   std::vector<int32_t> n_parts((size_t)n_new * Hkv, 0), part_base((size_t)n_new * Hkv + 1, 0), cta_item0(n_ctas + 1, 0);
   p->dealt = deal_streams ? 1 : 0;
   std::vector<int> fresh;                          // entries of `visit` with new rows, ascending
   if (kernel == ASPD_KERNEL_MMA)
     for (size_t i = 0; i < visit.size(); ++i)
       if ((visit[i].y >> 8) & 31) fresh.push_back((int)i);
-  p->patch_tiles = (!deal_streams && total_pages <= 2L * 8 * n_ctas) ? 1 : 0;
+  p->patch_tiles = (!deal_streams && total_pages <= 2L * 8 * base_ctas) ? 1 : 0;
   if (deal_streams) {
     deal_out(n_ctas);
     for (int c = 0; c < n_ctas; ++c) {
@@ -752,9 +753,78 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
       while (cta < n_ctas) cta_item0[++cta] = (int)p->items.size();
       return waits;
     };
-    const double waits = cut(0.0);
-    if (waits > 0.0) cut(waits);
+    if (!(like && like->tile_cut)) {
+      const double waits = cut(0.0);
+      if (waits > 0.0) cut(waits);
+    }
+    // A step of a few tiles per CTA takes as long as its slowest CTA, and that is a chain of tiles, whatever they hold, and
+    // of items.  The cut above counts pages: one request of 2.5 k keys became 71 CTAs of one tile and 11 of nine pages,
+    // which are two.  So such a step is also cut by tiles: every CTA one item of at most T tiles, the least T for which
+    // the SMs suffice, fewer where it would wait for new rows within its first kWaitKeys keys; and that cut is taken if its
+    // longest CTA has fewer tiles, or (up to four) as many where the other has CTAs of several items and there are hardly fewer of them.  us a pass, cut by pages and by tiles: 2 tiles and 1: one request of 2.5 k keys 244 and 235, a serial
+    // step over 1.1 k 196 and 185; 4 and 3: two requests opened with up to 26 tokens a branch 393 and 381; 4 with two items and 4:
+    // 17 k keys 418 and 406.  Not where the tiles come out the same (four requests of 2.2 k: 461 and 498 by tiles) and
+    // not with several items to a CTA (six branches opened with twelve tokens, 3 and 2 tiles: 395 and 408).
+    constexpr int kWaitKeys = 480, kTileCost = 320;          // a tile is 128 keys and a chain as long as 192 more
+    const int tp = 128 / ps;                                 // pages of a tile
+    if (kernel == ASPD_KERNEL_MMA && !coarse && tune.chunk_tokens == 0 && tune.n_ctas == 0 && !streams.empty() && !(like && !like->tile_cut) &&
+        (like || total_pages <= 6L * tp * base_ctas)) {
+      const int most = like ? n_ctas : p->sm_count;
+      std::vector<DeviceItem> cut_items;
+      // an item of at most T tiles to every CTA, fewer for one that comes to new rows within its first `wait_keys` keys; false: too few SMs
+      auto pack = [&](int T, int wait_keys) {
+        cut_items.clear();
+        for (const Stream& st : streams) {
+          const size_t first_item = cut_items.size();
+          for (int at = 0, slot = 0; at < st.n_pages; ++slot) {
+            if ((int)cut_items.size() >= most) return false;
+            int take = std::min(T * tp, st.n_pages - at);
+            if (wait_keys > 0) {
+              const auto e = std::lower_bound(fresh.begin(), fresh.end(), st.page0 + at);
+              const int before = e == fresh.end() ? take : *e - st.page0 - at;         // pages before the first with new rows
+              const int wait = wait_keys - kTileCost * (before / tp);
+              if (before < take && wait > 0) take = std::min(take, std::max(1, (T * kTileCost - wait) / kTileCost) * tp);
+            }
+            DeviceItem it;
+            it.q_tok0 = st.tok0; it.n_q_tok = st.n_tok; it.kv_head = st.head; it.page0 = st.page0 + at; it.n_pages = take; it.key0 = at * ps;
+            it.part_slot = slot; it.request = st.request; it.row_block = st.row_block; it.n_parts = 0;
+            cut_items.push_back(it);
+            at += take;
+          }
+          for (size_t i = first_item; i < cut_items.size(); ++i) cut_items[i].n_parts = (int)(cut_items.size() - first_item);
+        }
+        return true;
+      };
+      long tiles = 0;
+      for (const Stream& st : streams) tiles += (st.n_pages + tp - 1) / tp;
+      int longest = 0;                               // of the cut by pages
+      for (int c = 0; !like && c < n_ctas; ++c) {
+        int n = 0;
+        for (int i = cta_item0[c]; i < cta_item0[c + 1]; ++i) n += (p->items[i].n_pages + tp - 1) / tp;
+        longest = std::max(longest, n);
+      }
+      const int several = (int)p->items.size() > n_ctas && longest <= 4 ? 1 : 0;
+      bool done = false;
+      for (int T = (int)std::max(1L, (tiles + most - 1) / most); !done && (like || T < longest + several); ++T)
+        for (int w = p->patch_tiles ? 0 : kWaitKeys; !done && w >= 0; w -= kTileCost / 2) done = pack(T, w);
+      if (done && !like) {
+        int now = 0;
+        for (const DeviceItem& it : cut_items) now = std::max(now, (it.n_pages + tp - 1) / tp);
+        done = now < longest || 10 * cut_items.size() >= 9 * (size_t)n_ctas;
+      }
+      if (done) {
+        p->tile_cut = 1;
+        p->items.swap(cut_items);
+        // (a plan to be updated in place has a CTA to spare for every stream, whose number of tiles may grow)
+        if (!like) n_ctas = tune.updatable ? (int)std::min<long>(p->sm_count, std::max<long>((long)p->items.size(), base_ctas + (long)streams.size())) : (int)p->items.size();
+        cta_item0.assign(n_ctas + 1, (int)p->items.size());
+        for (int c = 0; c < (int)p->items.size(); ++c) cta_item0[c] = c;
+        for (const DeviceItem& it : p->items)
+          for (int i = 0; i < it.n_q_tok; ++i) n_parts[(size_t)(it.q_tok0 + i) * Hkv + it.kv_head] = it.n_parts;
+      }
+    }
   }
+  p->n_ctas = n_ctas;
   // Rows that are new this step, per CTA: what a fused step must write before the CTA reads.  The fused step
   // writes them in batches at the start of the kernel; with many new rows per CTA (a branch-open step) the
   // separate append kernel is the faster way, and such plans carry no list.  (The few pages that hold new rows
@@ -959,7 +1029,7 @@ int aspd_plan_update(aspd_plan_t* p, const aspd_request_t* req, const aspd_branc
   int rc = plan_create_impl(&p->shape, req, br, page_ids, n_req, p->n_pool_pages, p->mode, q_pos, &tune, nullptr, p, false, &t);
   if (rc) return rc;
   const aspd::PlanLayout& L = p->layout;
-  if (t->n_new != p->n_new || t->n_ctas != p->n_ctas || t->kernel != p->kernel || t->wide != p->wide || t->dealt != p->dealt ||
+  if (t->n_new != p->n_new || t->n_ctas != p->n_ctas || t->base_ctas != p->base_ctas || t->kernel != p->kernel || t->wide != p->wide || t->dealt != p->dealt ||
       t->fuse_append != p->fuse_append || t->shared_mask != p->shared_mask || t->single_launch != p->single_launch || t->m64 != p->m64 || (p->dec && padded_rows(t->max_rows) != padded_rows(p->max_rows)) || t->kernel != ASPD_KERNEL_MMA ||
       t->row_blocks.size() != L.n_row_blocks || t->part_base.size() != L.n_part_base) {
     delete t;
