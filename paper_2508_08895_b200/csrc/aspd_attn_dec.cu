@@ -269,7 +269,7 @@ template <int D, int NR>
 __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it, DecMisc* misc, uint32_t bars, uint32_t smem_p, uint32_t tmem,
                                              int par, int& g) {
   constexpr int HC = NR / 2;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = warp & 3, r0 = (warp >> 2) * HC;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31, q = warp & 3, r0 = (warp >> 2) * HC;
   const int kl = q * 32 + lane;                                  // this thread's key inside a tile
   const int ps = c.page_size, ps_shift = 31 - __clz(ps), ppt = kTile >> ps_shift;
   const int G = c.n_q_heads / c.n_kv_heads, M = it.n_q_tok * G;
@@ -409,7 +409,7 @@ __device__ __forceinline__ bool softmax_item(const Ctx& c, const DeviceItem& it,
 template <int D, int NR>
 __device__ __forceinline__ bool finish_item(const Ctx& c, const DeviceItem& it, DecMisc* misc, uint32_t tmem, int par, bool dead) {
   constexpr int HC = NR / 2;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = warp & 3, r0 = (warp >> 2) * HC;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31, q = warp & 3, r0 = (warp >> 2) * HC;
   const int M = it.n_q_tok * (c.n_q_heads / c.n_kv_heads);
   const uint32_t o_addr = tmem + ((uint32_t)(q * 32) << 16) + COL_O + r0;
   // head element of this thread's lane: M = 64 MMAs (D = 64) keep 16 rows in lanes 0..15 of each quadrant
@@ -543,12 +543,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const __grid_cons
   const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
   DecMisc* misc = reinterpret_cast<DecMisc*>(smem_raw + (base - raw) + c.off_misc);
   const uint32_t bars = base + c.off_misc;          // bars[] is the first member
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   volatile int* ab = &misc->abort_flag;
   constexpr uint32_t kTileBytes = kTile * D * 2;
   if (tid == 0) pdl_launch_dependents();
   const int4 head = c.pd.cta_head[2 * blockIdx.x], head2 = c.pd.cta_head[2 * blockIdx.x + 1];
-  const int item_begin = head.x, item_end = head.y;
+  const int item_begin = uniform(head.x), item_end = uniform(head.y);
   const int ps = c.page_size, ps_shift = 31 - __clz(ps), ppt = kTile >> ps_shift;
   int2 first_pages = make_int2(0, 0);
   if ((warp == W_K || warp == W_V) && lane < head.w) first_pages = c.pd.visit[head.z + lane];
@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const __grid_cons
   const uint32_t tmem = misc->tmem_base;
   // plan data of the first item
   DeviceItem first = {};
-  if (warp < 8 && item_begin < item_end) first = c.pd.items[item_begin];
+  if (warp < 8 && item_begin < item_end) first = uniform_item(c.pd.items[item_begin]);
   // everything above touches only the plan's own tables; inputs written by earlier kernels of the stream are
   // used from here on.  With the plan's stable-cache promise the producers go ahead with pages that hold no
   // new rows; they wait themselves before the first page that does.
@@ -598,13 +598,13 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const __grid_cons
     };
     if (item_begin < item_end) start_item(first, 0);
     for (int idx = item_begin; idx < item_end; ++idx, ++item_no) {
-      const DeviceItem it = idx == item_begin ? first : c.pd.items[idx];
+      const DeviceItem it = idx == item_begin ? first : uniform_item(c.pd.items[idx]);
       const int par = item_no & 1;
       named_sync(1, kSmThreads);                                  // the item's ranges are there
       dead |= !softmax_item<D, NR>(c, it, misc, bars, base + c.off_p, tmem, par, g);
       if (idx + 1 < item_end) {                                   // the next query tile as soon as this item's last scores are issued
         dead |= !mbar_wait(bars + 8 * Q_EMPTY, item_no & 1, ab);
-        start_item(c.pd.items[idx + 1], par ^ 1);
+        start_item(uniform_item(c.pd.items[idx + 1]), par ^ 1);
       }
       dead |= !mbar_wait(bars + 8 * O_FULL, item_no & 1, ab);
       tc_fence_after();
@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_dec_kernel(const __grid_cons
     bool ok = true, appended = false, waited = false;
     int2 nxt = first_pages;
     for (int idx = item_begin; idx < item_end && ok; ++idx) {
-      const DeviceItem it = c.pd.items[idx];
+      const DeviceItem it = uniform_item(c.pd.items[idx]);
       const int n_tiles = (it.n_pages + ppt - 1) / ppt;
       int2 cur = make_int2(0, 0);
       for (int t = 0; t < n_tiles && ok; ++t, ++g) {
