@@ -805,7 +805,9 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
       }
       const int several = (int)p->items.size() > n_ctas && longest <= 4 ? 1 : 0;
       bool done = false;
-      for (int T = (int)std::max(1L, (tiles + most - 1) / most); !done && (like || T < longest + several); ++T)
+      int T = (int)std::max(1L, (tiles + most - 1) / most);
+      if (like) T = std::max(T, like->tile_cut);     // an update's records have the room of the plan that it updates
+      for (; !done && (like || T < longest + several); ++T)
         for (int w = p->patch_tiles ? 0 : kWaitKeys; !done && w >= 0; w -= kTileCost / 2) done = pack(T, w);
       if (done && !like) {
         int now = 0;
@@ -813,7 +815,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
         done = now < longest || 10 * cut_items.size() >= 9 * (size_t)n_ctas;
       }
       if (done) {
-        p->tile_cut = 1;
+        p->tile_cut = T - 1;
         p->items.swap(cut_items);
         // (a plan to be updated in place has a CTA to spare for every stream, whose number of tiles may grow)
         if (!like) n_ctas = tune.updatable ? (int)std::min<long>(p->sm_count, std::max<long>((long)p->items.size(), base_ctas + (long)streams.size())) : (int)p->items.size();
