@@ -186,7 +186,8 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 // launchers (each returns an aspd_status_t)
 int launch_append(const aspd_plan* p, const void* k_new, const void* v_new, const int32_t* pos,
                   void* k_pool, void* v_pool, cudaStream_t s);
-int launch_attn_generic(const aspd_plan* p, const void* q, const void* k_pool, const void* v_pool,
+// k_new / v_new non-null: the step's new rows are written first
+int launch_attn_generic(const aspd_plan* p, const void* q, const void* k_new, const void* v_new, const void* k_pool, const void* v_pool,
                         cudaStream_t s);
 // out: null = (m, l, O) records for the combine kernel; non-null = final output, written by the
 // kernel itself when the plan has one item per (token, KV head) (ignored otherwise)

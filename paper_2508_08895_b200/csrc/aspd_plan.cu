@@ -653,9 +653,8 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   std::vector<int32_t> n_parts((size_t)n_new * Hkv, 0), part_base((size_t)n_new * Hkv + 1, 0), cta_item0(n_ctas + 1, 0);
   p->dealt = deal_streams ? 1 : 0;
   std::vector<int> fresh;                          // entries of `visit` with new rows, ascending
-  if (kernel == ASPD_KERNEL_MMA)
-    for (size_t i = 0; i < visit.size(); ++i)
-      if ((visit[i].y >> 8) & 31) fresh.push_back((int)i);
+  for (size_t i = 0; i < visit.size(); ++i)
+    if ((visit[i].y >> 8) & 31) fresh.push_back((int)i);
   p->patch_tiles = (!deal_streams && total_pages <= 2L * 8 * base_ctas) ? 1 : 0;
   if (deal_streams) {
     deal_out(n_ctas);
@@ -833,7 +832,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   // are found once, not once per KV head and CTA.)
   std::vector<int4> dirty;
   std::vector<int32_t> cta_dirty0(n_ctas + 1, 0);
-  p->fuse_append = (kernel == ASPD_KERNEL_MMA && !shared_mask && tok_field_fits && counts_fit && p->wide != 2 && !(like && !like->fuse_append)) ? 1 : 0;
+  p->fuse_append = (!shared_mask && tok_field_fits && counts_fit && p->wide != 2 && !(like && !like->fuse_append)) ? 1 : 0;
   // A CTA with that many tiles has its rows written long before it comes to the pages that hold them, so there more are
   // written at its start, as long as that does not take longer than the tiles: up to 2.5 to a tile over the step where
   // the streams are dealt, which begin with a prefix, and one to a tile in any CTA where they are cut, since a CTA may
@@ -865,7 +864,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
       }
       // (32 767 tiles: what the number's field holds)
       const int rows = (int)dirty.size() - cta_dirty0[c];
-      const bool more = !patches && (like || (tile0 >= kLongCta && !p->dec && (deal_streams || rows <= tile0)));
+      const bool more = !patches && !cores && (like || (tile0 >= kLongCta && !p->dec && (deal_streams || rows <= tile0)));
       if ((rows > kMostFusedRows && !more) || tile0 > 32767) p->fuse_append = 0;
       many |= rows > kMostFusedRows; all_tiles += tile0;
     }
@@ -1139,7 +1138,7 @@ int aspd_attn_partials(aspd_plan_t* p, const void* q, const void* k_pool, const 
   cudaStream_t s = (cudaStream_t)stream;
   note_stream(p, stream);
   return p->kernel == ASPD_KERNEL_MMA ? launch_attn_mma(p, q, k_pool, v_pool, nullptr, s)
-                                      : launch_attn_generic(p, q, k_pool, v_pool, s);
+                                      : launch_attn_generic(p, q, nullptr, nullptr, k_pool, v_pool, s);
 }
 
 int aspd_step_partials(aspd_plan_t* p, const void* q, const void* k_new, const void* v_new, void* k_pool, void* v_pool,
@@ -1195,9 +1194,11 @@ static int run_step(aspd_plan_t* p, int mode, const void* q, const void* k_new, 
   } else if (p->kernel == ASPD_KERNEL_MMA) {
     rc = launch_append(p, k_new, v_new, p->dev.tok_pos, k_pool, v_pool, s);
     if (rc == ASPD_OK) rc = launch_attn_mma(p, q, k_pool, v_pool, out, s);
+  } else if (p->fuse_append) {
+    rc = launch_attn_generic(p, q, k_new, v_new, k_pool, v_pool, s);
   } else {
     rc = launch_append(p, k_new, v_new, p->dev.tok_pos, k_pool, v_pool, s);
-    if (rc == ASPD_OK) rc = launch_attn_generic(p, q, k_pool, v_pool, s);
+    if (rc == ASPD_OK) rc = launch_attn_generic(p, q, nullptr, nullptr, k_pool, v_pool, s);
   }
   if (rc || attn_mma_writes_output(p)) return rc;
   return launch_combine(p, out, s);

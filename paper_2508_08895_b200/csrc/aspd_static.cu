@@ -144,7 +144,7 @@ extern "C" int aspd_attn_static(const aspd_plan_t* plan, const void* q, const vo
   // plans that deal whole streams have one item per (token, KV head): their kernel writes the output
   if (attn_mma_direct(&shell)) return launch_attn_mma(&shell, q, k_pool, v_pool, out, s);
   rc = shell.kernel == ASPD_KERNEL_MMA ? launch_attn_mma(&shell, q, k_pool, v_pool, nullptr, s)
-                                       : launch_attn_generic(&shell, q, k_pool, v_pool, s);
+                                       : launch_attn_generic(&shell, q, nullptr, nullptr, k_pool, v_pool, s);
   if (rc) return rc;
   return launch_combine(&shell, out, s);
 }
