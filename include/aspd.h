@@ -177,7 +177,8 @@ typedef struct {
   int32_t chunk_tokens;     /* forced maximum keys per item (0: none)                       */
   int32_t n_ctas;           /* CTAs of the persistent grid = shares the streams are cut into */
   int32_t fused_append;     /* 1: aspd_branch_step / aspd_serial_step write the new rows inside the
-                               attention pass; 0: they run the append kernel first               */
+                               attention pass; 0: they run the append kernel first (or, with the
+                               CUDA-core kernel, write few new rows inside its pass)              */
   int32_t direct_output;    /* 1: one item per (token, KV head) and the attention kernel writes the
                                output itself (no records, no combine launch)                     */
   int32_t max_rows_per_item;/* query rows (tokens x group heads) an item may carry: 64, 128 or 256  */

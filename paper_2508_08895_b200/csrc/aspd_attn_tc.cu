@@ -14,17 +14,15 @@
 // The 128 accumulator lanes are used as R x KS: the query rows (padded to R = 32 or 64) are
 // replicated KS = 128 / R times in the A operand, and softmax thread (j, r) handles row r over
 // the j-th key sub-range of the tile only, so all 128 threads share the exponentials.  The KS
-// threads of a row agree on one reference maximum per tile (exchanged through shared memory)
-// and write their P values into the SAME row r of the P tile, so the second MMA sums over all
-// keys by itself and rows >= R of its output are simply ignored.  The reference maximum is only
-// raised when the tile maximum exceeds it by more than 2^8, which keeps P exactly consistent
-// with the (m, l, O) record while making the rescale of O in TMEM rare.
+// threads of a row take their exponentials against one reference (0 at an item's start, moved only when a sum leaves
+// 2^-60 .. 2^40, see softmax_item) and write their P values into the SAME row r of the P tile, so the second MMA sums over all
+// keys by itself and rows >= R of its output are simply ignored.
 //
 // Warp roles: 0-7 softmax (TMEM lane quadrant = warp % 4; warps w and w + 4 share the rows of a
 // quadrant and take half of the columns each), 8 and 11 bulk-copy producers (K and V), 9 MMA
 // issuer (one elected lane), 12-15 fused append of the step's new rows (aspd_branch_step /
 // aspd_serial_step), query preparation (RoPE, bf16, swizzled store, one item ahead) and epilogue
-// (TMEM lane quadrant = warp - 12); warp 10 is idle.  All cross-role hand-offs are mbarriers; every
+// (TMEM lane quadrant = warp - 12); warp 10 allocates the tensor memory and is idle then.  All cross-role hand-offs are mbarriers; every
 // wait is bounded and on expiry sets the plan's status word to ASPD_ERR_TIMEOUT and makes all
 // roles drain and exit.
 #include <type_traits>
