@@ -47,7 +47,8 @@ __device__ __forceinline__ void add_row(float (&acc)[EPL], const float (&x)[EPL]
 // other CTAs of the same launch.
 // Up to 64 records share a maximum: their (max, sum) pairs, two to a lane, and the first 8 * NB of their O rows are
 // asked for together, the maximum and the weights are made once, and then every row is a broadcast and D / 32
-// multiply-adds a lane, so that a row cut into up to 8 * NB parts costs one round trip to L2.  NB changes no bit of the result.
+// multiply-adds a lane, so that a row cut into up to 8 * NB parts costs one round trip to L2.  Every NB takes any number of
+// records and gives the same bits: a captured launch keeps its instance while updates of its plan change the cuts.
 template <typename T, int D, int NB>
 __device__ __forceinline__ void combine_row(const float* __restrict__ ws_o, const float2* __restrict__ ws_ml, int p0, int n, int G,
                                             int g, int lane, T* __restrict__ dst) {
@@ -67,9 +68,10 @@ __device__ __forceinline__ void combine_row(const float* __restrict__ ws_o, cons
     if (lane + 32 < cnt) ml1 = __ldcg(pair + 32 * G);
     float w0 = 0.f, w1 = 0.f;
 #pragma unroll 1
-    for (int b0 = 0; b0 < cnt; b0 += kRows, row += kRows * stride) {
+    for (int b0 = 0; b0 < cnt; b0 += kRows) {
       float v[kRows][EPL];
       fetch_rows<kRows, EPL>(v, row, stride, cnt - b0);
+      row += (kGroup % kRows ? min(kRows, cnt - b0) : kRows) * stride;
       asm volatile("" : "+r"(b0));                 // (one copy of the loop's body, not one for its first turn)
       if (b0 == 0) {
         // records of chunks with no visible key have sum 0
@@ -88,7 +90,8 @@ __device__ __forceinline__ void combine_row(const float* __restrict__ ws_o, cons
 #pragma unroll
         for (int e = 0; e < EPL; ++e) acc[e] *= alpha;
       }
-      const float wb = __shfl_sync(0xffffffffu, lane >= b0 ? w0 : w1, b0 + lane);     // of record b0 + lane (the source lane is taken modulo 32)
+      float wb = __shfl_sync(0xffffffffu, lane >= b0 ? w0 : w1, b0 + lane);           // of record b0 + lane (the source lane is taken modulo 32)
+      if (kGroup % kRows && b0 + lane >= cnt) wb = 0.f;                               // 24 rows: the group's last turn has 16 of them
 #pragma unroll
       for (int k = 0; k < kRows; ++k) add_row<EPL>(acc, v[k], __shfl_sync(0xffffffffu, wb, k));
     }

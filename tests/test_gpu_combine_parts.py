@@ -1,4 +1,5 @@
-"""The merge of rows cut into one part up to more than the 64 that share a maximum, in every kernel instance."""
+"""The merge of rows cut into one part up to more than the 64 that share a maximum (a new plan each, so in the instance made
+for that many; test_gpu_graph_parts.py has each instance take more)."""
 import numpy as np
 import pytest
 
