@@ -1,5 +1,5 @@
-"""An item's first tile against a reference of 0, as the tensor-core kernels take it: logits so low or so high that the
-tile has to be done again with the rows' own maxima, and rows that see their first key tiles later."""
+"""Logits so low or so high that a tile cannot be taken against the reference that its rows have: an item's first tile, and
+rows that see their first key tiles later."""
 import numpy as np
 import pytest
 
@@ -31,3 +31,16 @@ def test_equal_logits_far_from_zero(d, heads, n_ctas, logit):
         for g, r in zip(run.outputs, ref.outputs):
             assert np.isfinite(g).all()
             check(g, r, wl.dtype, f"{d} {heads} {n_ctas} {logit} {fused}")
+
+
+@pytest.mark.parametrize("d,heads,page", [(128, (28, 4), 16), (128, (4, 4), 16), (128, (64, 1), 16), (64, (14, 2), 16), (128, (28, 4), 8)])
+def test_the_largest_weight_is_one(d, heads, page):
+    """Branches that begin a sequence: every token sees itself alone, and its output is its V to the bit.  The weights that
+    meet V are bf16 and their sum is not, so that a weight of 2^x that bf16 does not hold would show."""
+    from paper_2508_08895_b200 import engine as E
+    prior = [[0], [0, 0, 0], [0] * 8]
+    wl = W.build_segment_workload("lone", 76, *heads, d, "bf16", 1e6, [0, 0, 0], prior, [[1] * len(p) for p in prior], serial_steps=0, page_size=page)
+    for fused in (False, True):
+        run = E.run_workload(wl, fused=fused, stable_cache=fused)
+        v = wl.phases[-1].v_new
+        assert np.array_equal(run.outputs[-1], np.repeat(v, heads[0] // heads[1], axis=1))
