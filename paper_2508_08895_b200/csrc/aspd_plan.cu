@@ -769,6 +769,7 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     if (kernel == ASPD_KERNEL_MMA && !coarse && tune.chunk_tokens == 0 && tune.n_ctas == 0 && !streams.empty() && !(like && !like->tile_cut) &&
         (like || total_pages <= 6L * tp * base_ctas)) {
       const int most = like ? n_ctas : p->sm_count;
+      if ((long)streams.size() > most && like) { delete p; return ASPD_ERR_UNSUPPORTED; }      // an item each at least
       std::vector<DeviceItem> cut_items;
       // an item of at most T tiles to every CTA, fewer for one that comes to new rows within its first `wait_keys` keys; false: too few SMs
       auto pack = [&](int T, int wait_keys) {
@@ -781,8 +782,8 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
             if (wait_keys > 0) {
               const auto e = std::lower_bound(fresh.begin(), fresh.end(), st.page0 + at);
               const int before = e == fresh.end() ? take : *e - st.page0 - at;         // pages before the first with new rows
-              const int wait = wait_keys - kTileCost * (before / tp);
-              if (before < take && wait > 0) take = std::min(take, std::max(1, (T * kTileCost - wait) / kTileCost) * tp);
+              const long wait = wait_keys - (long)kTileCost * (before / tp);
+              if (before < take && wait > 0) take = (int)std::min<long>(take, std::max(1L, ((long)T * kTileCost - wait) / kTileCost) * tp);
             }
             DeviceItem it;
             it.q_tok0 = st.tok0; it.n_q_tok = st.n_tok; it.kv_head = st.head; it.page0 = st.page0 + at; it.n_pages = take; it.key0 = at * ps;
@@ -795,7 +796,11 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
         return true;
       };
       long tiles = 0;
-      for (const Stream& st : streams) tiles += (st.n_pages + tp - 1) / tp;
+      int longest_stream = 0;
+      for (const Stream& st : streams) {
+        tiles += (st.n_pages + tp - 1) / tp;
+        longest_stream = std::max(longest_stream, (st.n_pages + tp - 1) / tp);
+      }
       int longest = 0;                               // of the cut by pages
       for (int c = 0; !like && c < n_ctas; ++c) {
         int n = 0;
@@ -806,7 +811,9 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
       bool done = false;
       int T = (int)std::max(1L, (tiles + most - 1) / most);
       if (like) T = std::max(T, like->tile_cut);     // an update's records have the room of the plan that it updates
-      for (; !done && (like || T < longest + several); ++T)
+      // (an update's streams have an item each at the latest with as many tiles as the longest has)
+      const int last = like ? std::max(T, longest_stream) : longest + several - 1;
+      for (; !done && T <= last; ++T)
         for (int w = p->patch_tiles ? 0 : kWaitKeys; !done && w >= 0; w -= kTileCost / 2) done = pack(T, w);
       if (done && !like) {
         int now = 0;
