@@ -480,12 +480,15 @@ __global__ void __launch_bounds__(kThreadsW2, 1) attn_tc_w2_kernel(Ctx c) {
             if (lane == 0 && grp == 0) ASPD_STAMP(c, g, 10 + h);
             // 16 keys = one page per k-step
             tc_mma_ts_pv_lane0(o_tmem, s_tmem + h * 64, smem_desc(vbuf + 4 * h * 4096, 1024, 2048), idesc_pv, (t > 0 || h > 0) ? 1u : 0u, min(4, npg - 4 * h));
+            // (Asked for only when a row's reference moves.  Before the word of the scores behind it, which send the group
+            // two halves on, and before O's: a group that waits for half hc - 1 then knows that half hc - 2 is through,
+            // and the parity tells the two apart.)
+            tc_commit_lane0(bar_pvdone);
             if (npg1 > 4 * h) issue_s(t + 1, h);
             if (h == halves - 1) {
               if (t == n_tiles - 1) tc_commit_lane0(bars_u + 8 * (WO_FULL + grp));
               release(bars_u + 8 * (WV_EMPTY + (g & 1)));
             }
-            tc_commit_lane0(bar_pvdone);       // (asked for only when a row's reference moves)
           }
         }
         if (grp == 0 && lane == 0) *lead = idx + 1;
