@@ -494,15 +494,30 @@ __global__ void __launch_bounds__(kGenThreads, 2) attn_generic_kernel(PlanDevice
 // One warp per (new token, query head): merge the partial records of (token, KV head) by
 // log-sum-exp in one pass with a running maximum.  Where the records lie is plan data and is
 // read before the dependency wait.
-template <typename T, int D, int NB>
-__global__ void __launch_bounds__(128) combine_kernel(PlanDevice pd, T* __restrict__ out, int n_q_heads, int n_kv_heads, int G) {
+// FLAT: the rows of all tokens are numbered through, four to a block; otherwise a token's heads have blocks of their own, a
+// grid of (tokens, heads / 4).  FLAT where four does not divide the heads: every fourth block of 14 heads had two idle
+// warps, and eight requests' 152 blocks did not fit the chip at a time, which 133 do (24 layers 356 and 344 us).  Not
+// where it does: its 64 registers instead of 72 let eight instead of seven waiting blocks onto an SM, so that a large grid
+// lies on fewer of them (504 blocks, 28 layers 398 and 407 us).
+// inv_g: floor((2^32 - 1) / G), so that the upper word of a row times it is row / G or one less.
+template <typename T, int D, int NB, bool FLAT>
+__global__ void __launch_bounds__(128) combine_kernel(PlanDevice pd, T* __restrict__ out, int n_rows, int n_q_heads, int G, uint32_t inv_g) {
   pdl_launch_dependents();
   // (what all lanes agree on is taken from lane 0, which lets the compiler know: 9 instead of 15 KB of code)
-  const int tok = blockIdx.x, hq = blockIdx.y * 4 + uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int h = min(hq, n_q_heads - 1) / G, g = hq - h * G;
-  const int p0 = uniform(pd.part_base[tok * n_kv_heads + h]), n = uniform(pd.part_base[tok * n_kv_heads + h + 1]) - p0;
+  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  int row, pair, g;                                // of all rows; of all (token, KV head) pairs; in the pair's group
+  if constexpr (FLAT) {
+    row = blockIdx.x * 4 + warp;
+    const int r = min(row, n_rows - 1);
+    pair = (int)__umulhi((uint32_t)r, inv_g); g = r - pair * G;
+    if (g >= G) { ++pair; g -= G; }
+  } else {
+    const int tok = blockIdx.x, hq = blockIdx.y * 4 + warp, h = hq / G;
+    row = tok * n_q_heads + hq; pair = tok * (n_q_heads / G) + h; g = hq - h * G;
+  }
+  const int p0 = uniform(pd.part_base[pair]), n = uniform(pd.part_base[pair + 1]) - p0;
   pdl_wait();
-  if (hq < n_q_heads) combine_row<T, D, NB>(pd.ws_o, pd.ws_ml, p0, n, G, g, lane, out + ((size_t)tok * n_q_heads + hq) * D);
+  if (!FLAT || row < n_rows) combine_row<T, D, NB>(pd.ws_o, pd.ws_ml, p0, n, G, g, lane, out + (size_t)row * D);
 }
 
 template <typename T>
@@ -570,7 +585,7 @@ int launch_qcs(const aspd_plan* p, cudaStream_t s) {
   return check_launch();
 }
 
-template <typename T, int D, int NB>
+template <typename T, int D, int NB, bool FLAT>
 static int launch_combine_rows(const aspd_plan* p, void* out, cudaStream_t s) {
   const aspd_shape_t& sh = p->shape;
   static int sms[64] = {};                         // per device: SMs, known once the kernel has been configured there
@@ -579,7 +594,7 @@ static int launch_combine_rows(const aspd_plan* p, void* out, cudaStream_t s) {
   int n_sms = dev >= 0 && dev < 64 ? sms[dev] : 0;
   if (n_sms == 0) {
     if (cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(combine_kernel<T, D, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombineClaim) != cudaSuccess)
+        cudaFuncSetAttribute(combine_kernel<T, D, NB, FLAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombineClaim) != cudaSuccess)
       return ASPD_ERR_CUDA;
     if (dev >= 0 && dev < 64) sms[dev] = n_sms;
   }
@@ -591,25 +606,30 @@ static int launch_combine_rows(const aspd_plan* p, void* out, cudaStream_t s) {
   // 330 / 306, one token after another over 1 k 255 / 213 / 213, eight branches over 16 k 517 / 627 / 495, eight
   // requests with heads of 64 410 / 402 / 364.  A grid larger than the chip spreads anyway, and would run in waves
   // (six branches opened with twelve tokens each, 504 blocks: 480 / 438 / 524).
-  const dim3 grid((unsigned)p->n_new, (unsigned)(sh.n_q_heads + 3) / 4);
-  const long blocks = (long)grid.x * grid.y;
+  const int rows = p->n_new * sh.n_q_heads, blocks = (rows + 3) / 4, G = sh.n_q_heads / sh.n_kv_heads;
   const size_t claim = blocks <= n_sms ? kCombineClaim : 0;
-  return status_of(launch_pdl(combine_kernel<T, D, NB>, grid, dim3(128), claim, s, p->dev, (T*)out, sh.n_q_heads, sh.n_kv_heads, sh.n_q_heads / sh.n_kv_heads));
+  const dim3 grid = FLAT ? dim3(blocks) : dim3(p->n_new, sh.n_q_heads / 4);
+  return status_of(launch_pdl(combine_kernel<T, D, NB, FLAT>, grid, dim3(128), claim, s, p->dev, (T*)out, rows, sh.n_q_heads, G, 0xFFFFFFFFu / (uint32_t)G));
 }
 
-template <typename T, int D>
+template <typename T, int D, bool FLAT>
 static int launch_combine_of(const aspd_plan* p, void* out, cudaStream_t s) {
   // as many records in flight as the plan's rows have, up to 32: more take registers, and with them blocks from an SM
   // (504 blocks of rows with six records at three: 418 us a pass of 28 layers, at one 395)
   const int nb = (p->max_parts + 7) / 8;
-  return nb <= 1 ? launch_combine_rows<T, D, 1>(p, out, s) : nb == 2 ? launch_combine_rows<T, D, 2>(p, out, s)
-       : nb == 3 ? launch_combine_rows<T, D, 3>(p, out, s) : launch_combine_rows<T, D, 4>(p, out, s);
+  return nb <= 1 ? launch_combine_rows<T, D, 1, FLAT>(p, out, s) : nb == 2 ? launch_combine_rows<T, D, 2, FLAT>(p, out, s)
+       : nb == 3 ? launch_combine_rows<T, D, 3, FLAT>(p, out, s) : launch_combine_rows<T, D, 4, FLAT>(p, out, s);
+}
+
+template <typename T, int D>
+static int launch_combine_heads(const aspd_plan* p, void* out, cudaStream_t s) {
+  return p->shape.n_q_heads % 4 == 0 ? launch_combine_of<T, D, false>(p, out, s) : launch_combine_of<T, D, true>(p, out, s);
 }
 
 int launch_combine(const aspd_plan* p, void* out, cudaStream_t s) {
   const aspd_shape_t& sh = p->shape;
-  if (sh.dtype == ASPD_DTYPE_BF16) return sh.head_dim == 128 ? launch_combine_of<__nv_bfloat16, 128>(p, out, s) : launch_combine_of<__nv_bfloat16, 64>(p, out, s);
-  return sh.head_dim == 128 ? launch_combine_of<float, 128>(p, out, s) : launch_combine_of<float, 64>(p, out, s);
+  if (sh.dtype == ASPD_DTYPE_BF16) return sh.head_dim == 128 ? launch_combine_heads<__nv_bfloat16, 128>(p, out, s) : launch_combine_heads<__nv_bfloat16, 64>(p, out, s);
+  return sh.head_dim == 128 ? launch_combine_heads<float, 128>(p, out, s) : launch_combine_heads<float, 64>(p, out, s);
 }
 
 int launch_rerotate(const aspd_shape_t* sh, void* k_pool, const int32_t* pages, const int32_t* rows, const int32_t* delta,
