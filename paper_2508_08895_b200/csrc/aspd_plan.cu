@@ -820,6 +820,22 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
         for (const DeviceItem& it : cut_items) now = std::max(now, (it.n_pages + tp - 1) / tp);
         done = now < longest || 10 * cut_items.size() >= 9 * (size_t)n_ctas;
       }
+      // (not where a CTA gets more new rows than it writes itself and none has them by pages: such a step would take a launch more)
+      if (done && !like) {
+        auto rows_of = [&](const DeviceItem& it) {
+          int n = 0;
+          for (auto e = std::lower_bound(fresh.begin(), fresh.end(), it.page0); e != fresh.end() && *e < it.page0 + it.n_pages; ++e) n += (visit[*e].y >> 8) & 31;
+          return n;
+        };
+        if (std::any_of(cut_items.begin(), cut_items.end(), [&](const DeviceItem& it) { return rows_of(it) > kMostFusedRows; })) {
+          done = false;
+          for (int c = 0; c < n_ctas && !done; ++c) {
+            int n = 0;
+            for (int i = cta_item0[c]; i < cta_item0[c + 1]; ++i) n += rows_of(p->items[i]);
+            done = n > kMostFusedRows;
+          }
+        }
+      }
       if (done) {
         p->tile_cut = T - 1;
         p->items.swap(cut_items);

@@ -36,3 +36,17 @@ def test_tiles_of_short_steps(d, page, seed):
         if sum(-(-n // ppt) for n, _ in streams.values()) <= SMS:
             assert max(int(tiles[first[c]:first[c + 1]].sum()) for c in range(len(first) - 1)) == 1
         plan.destroy()
+
+
+@pytest.mark.parametrize("heads,d,page,n_req,prefix,seed", [((16, 2), 128, 16, 10, (500, 1600), 20), ((4, 1), 64, 8, 26, (470, 1420), 0),
+                                                            ((4, 1), 64, 8, 26, (470, 1420), 30)])
+def test_cuts_keep_the_pass_that_writes_the_new_rows(heads, d, page, n_req, prefix, seed):
+    """Up to 24 branches of one token: by tiles a CTA would get more new rows than it writes itself, by pages none does."""
+    rng = np.random.default_rng(seed)
+    lens = [int(x) for x in rng.integers(*prefix, size=n_req)]
+    prior = [[0] * int(rng.integers(1, 25)) for _ in range(n_req)]
+    wl = W.build_segment_workload("rows", 73, *heads, d, "bf16", 1e6, lens, prior, [[1] * len(p) for p in prior], page_size=page)
+    ph = wl.phases[-1]
+    plan = B.Plan(B.make_shape(*heads, d, page, "bf16", 1e6, d ** -0.5), ph.desc, wl.n_pool_pages, ph.mode, host_only=True)
+    assert plan.info.fused_append == 1
+    plan.destroy()
