@@ -118,6 +118,7 @@ struct aspd_plan {
   int n_ctas = 0;
   int base_ctas = 0;               // CTAs by pages alone: an update of the plan has to come to the same number
   int tile_cut = 0;                // the streams are cut by tiles, an item of at most that many to a CTA (steps of a few tiles per CTA)
+  size_t room_items = 0, room_partials = 0;   // updatable plan cut by tiles: items and records by pages, for which it has room too
   int host_only = 0;
   int sm_count = 0;
   int n_row_blocks = 0;

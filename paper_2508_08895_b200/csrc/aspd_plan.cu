@@ -808,33 +808,49 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
         longest = std::max(longest, n);
       }
       const int several = (int)p->items.size() > n_ctas && longest <= 4 ? 1 : 0;
+      // new rows that come to a CTA, and whether some CTA would have more than it writes itself
+      auto rows_of = [&](const DeviceItem& it) {
+        int n = 0;
+        for (auto e = std::lower_bound(fresh.begin(), fresh.end(), it.page0); e != fresh.end() && *e < it.page0 + it.n_pages; ++e) n += (visit[*e].y >> 8) & 31;
+        return n;
+      };
+      auto many_rows = [&]() { return std::any_of(cut_items.begin(), cut_items.end(), [&](const DeviceItem& it) { return rows_of(it) > kMostFusedRows; }); };
+      auto many_rows_by_pages = [&]() {
+        for (int c = 0; c < n_ctas; ++c) {
+          int n = 0;
+          for (int i = cta_item0[c]; i < cta_item0[c + 1]; ++i) n += rows_of(p->items[i]);
+          if (n > kMostFusedRows) return true;
+        }
+        return false;
+      };
+      auto records_of = [](const std::vector<DeviceItem>& items) { long n = 0; for (const DeviceItem& it : items) n += it.n_q_tok; return n; };
+      // an update has the room of the plan that it updates, and its launches
+      auto fits_plan = [&]() {
+        return cut_items.size() <= like->layout.cap_items && records_of(cut_items) <= (long)like->layout.cap_partials &&
+               !(like->fuse_append && like->patch_tiles && many_rows());
+      };
       bool done = false;
       int T = (int)std::max(1L, (tiles + most - 1) / most);
-      if (like) T = std::max(T, like->tile_cut);     // an update's records have the room of the plan that it updates
+      if (like) T = std::max(T, like->tile_cut);
       // (an update's streams have an item each at the latest with as many tiles as the longest has)
       const int last = like ? std::max(T, longest_stream) : longest + several - 1;
       for (; !done && T <= last; ++T)
-        for (int w = p->patch_tiles ? 0 : kWaitKeys; !done && w >= 0; w -= kTileCost / 2) done = pack(T, w);
+        for (int w = p->patch_tiles ? 0 : kWaitKeys; !done && w >= 0; w -= kTileCost / 2) done = pack(T, w) && (!like || fits_plan());
       if (done && !like) {
         int now = 0;
         for (const DeviceItem& it : cut_items) now = std::max(now, (it.n_pages + tp - 1) / tp);
         done = now < longest || 10 * cut_items.size() >= 9 * (size_t)n_ctas;
       }
-      // (not where a CTA gets more new rows than it writes itself and none has them by pages: such a step would take a launch more)
+      // not where a CTA gets more new rows than it writes itself and none has them by pages: such a step would take a
+      // launch more.  Nor, if the plan is to be updated, the other way round: updates have to keep the plan's launches.
       if (done && !like) {
-        auto rows_of = [&](const DeviceItem& it) {
-          int n = 0;
-          for (auto e = std::lower_bound(fresh.begin(), fresh.end(), it.page0); e != fresh.end() && *e < it.page0 + it.n_pages; ++e) n += (visit[*e].y >> 8) & 31;
-          return n;
-        };
-        if (std::any_of(cut_items.begin(), cut_items.end(), [&](const DeviceItem& it) { return rows_of(it) > kMostFusedRows; })) {
-          done = false;
-          for (int c = 0; c < n_ctas && !done; ++c) {
-            int n = 0;
-            for (int i = cta_item0[c]; i < cta_item0[c + 1]; ++i) n += rows_of(p->items[i]);
-            done = n > kMostFusedRows;
-          }
-        }
+        const bool by_tiles = many_rows();
+        if (by_tiles || tune.updatable) done = by_tiles == many_rows_by_pages();
+      }
+      if (done && tune.updatable && !like) { p->room_items = p->items.size(); p->room_partials = records_of(p->items); }
+      if (!done && like) {                             // an update that no cut by tiles fits is cut by pages
+        const double waits = cut(0.0);
+        if (waits > 0.0) cut(waits);
       }
       if (done) {
         p->tile_cut = T - 1;
@@ -946,8 +962,8 @@ static void plan_layout(const aspd_plan* p, double slack, aspd::PlanLayout* L) {
   const aspd_shape_t& sh = p->shape;
   const int d = sh.head_dim, Hq = sh.n_q_heads, Hkv = sh.n_kv_heads, G = Hq / Hkv, es = esize_of(sh.dtype), n_new = p->n_new;
   auto cap = [&](size_t n) { return std::max<size_t>(1, (size_t)((double)n * slack) + (slack > 1.0 ? 64 : 0)); };
-  L->cap_items = cap(p->items.size()); L->cap_visit = cap(p->visit.size()); L->cap_dirty = cap(p->dirty.size());
-  L->cap_partials = p->wide == 2 ? 1 : cap((size_t)p->n_partials);      // (the two-tile kernel never writes records)
+  L->cap_items = cap(std::max(p->items.size(), p->room_items)); L->cap_visit = cap(p->visit.size()); L->cap_dirty = cap(p->dirty.size());
+  L->cap_partials = p->wide == 2 ? 1 : cap(std::max((size_t)p->n_partials, p->room_partials));      // (the two-tile kernel never writes records)
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   L->o_items = take(sizeof(DeviceItem) * L->cap_items);
