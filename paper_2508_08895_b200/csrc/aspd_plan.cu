@@ -759,25 +759,27 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
     // A step of a few tiles per CTA takes as long as its slowest CTA, and that is a chain of tiles, whatever they hold, and
     // of items.  The cut above counts pages: one request of 2.5 k keys became 71 CTAs of one tile and 11 of nine pages,
     // which are two.  So such a step is also cut by tiles: every CTA one item of at most T tiles, the least T for which
-    // the SMs suffice, fewer where it would wait for new rows within its first kWaitKeys keys; and that cut is taken if its
-    // longest CTA has fewer tiles, or (up to four) as many where the other has CTAs of several items and there are hardly fewer of them.  us a pass, cut by pages and by tiles: 2 tiles and 1: one request of 2.5 k keys 244 and 235, a serial
-    // step over 1.1 k 196 and 185; 4 and 3: two requests opened with up to 26 tokens a branch 393 and 381; 4 with two items and 4:
-    // 17 k keys 418 and 406.  Not where the tiles come out the same (four requests of 2.2 k: 461 and 498 by tiles) and
-    // not with several items to a CTA (six branches opened with twelve tokens, 3 and 2 tiles: 395 and 408).
+    // the SMs suffice, fewer where it would wait for new rows within its first kWaitKeys keys; and that cut is taken if
+    // its longest CTA has fewer tiles, or (up to four) as many where the other has CTAs of several items and there are
+    // hardly fewer of them.  us a pass, cut by pages and by tiles: 2 tiles and 1: one request of 2.5 k keys 244 and 235,
+    // a serial step over 1.1 k 196 and 185; 4 and 3: two requests opened with up to 26 tokens a branch 393 and 381; 4
+    // with two items and 4: 17 k keys 418 and 406.  Not where the tiles come out the same (four requests of 2.2 k: 461
+    // and 498 by tiles) and not with several items to a CTA (six branches opened with twelve tokens, 3 and 2 tiles: 395
+    // and 408).
     constexpr int kWaitKeys = 480, kTileCost = 320;          // a tile is 128 keys and a chain as long as 192 more
     const int tp = 128 / ps;                                 // pages of a tile
     if (kernel == ASPD_KERNEL_MMA && !coarse && tune.chunk_tokens == 0 && tune.n_ctas == 0 && !streams.empty() && !(like && !like->tile_cut) &&
         (like || total_pages <= 6L * tp * base_ctas)) {
       const int most = like ? n_ctas : p->sm_count;
       if ((long)streams.size() > most && like) { delete p; return ASPD_ERR_UNSUPPORTED; }      // an item each at least
-      std::vector<DeviceItem> cut_items;
-      // an item of at most T tiles to every CTA, fewer for one that comes to new rows within its first `wait_keys` keys; false: too few SMs
+      // Pages of the items, an item of at most T tiles to every CTA, fewer for one that comes to new rows within its first
+      // `wait_keys` keys; false: too few SMs.  Row block by row block: its streams, one to a KV head, are cut alike.
+      std::vector<int> takes;
       auto pack = [&](int T, int wait_keys) {
-        cut_items.clear();
-        for (const Stream& st : streams) {
-          const size_t first_item = cut_items.size();
-          for (int at = 0, slot = 0; at < st.n_pages; ++slot) {
-            if ((int)cut_items.size() >= most) return false;
+        takes.clear();
+        for (size_t s = 0; s < streams.size(); s += Hkv) {
+          const Stream& st = streams[s];
+          for (int at = 0; at < st.n_pages; at += takes.back()) {
             int take = std::min(T * tp, st.n_pages - at);
             if (wait_keys > 0) {
               const auto e = std::lower_bound(fresh.begin(), fresh.end(), st.page0 + at);
@@ -785,15 +787,17 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
               const long wait = wait_keys - (long)kTileCost * (before / tp);
               if (before < take && wait > 0) take = (int)std::min<long>(take, std::max(1L, ((long)T * kTileCost - wait) / kTileCost) * tp);
             }
-            DeviceItem it;
-            it.q_tok0 = st.tok0; it.n_q_tok = st.n_tok; it.kv_head = st.head; it.page0 = st.page0 + at; it.n_pages = take; it.key0 = at * ps;
-            it.part_slot = slot; it.request = st.request; it.row_block = st.row_block; it.n_parts = 0;
-            cut_items.push_back(it);
-            at += take;
+            takes.push_back(take);
           }
-          for (size_t i = first_item; i < cut_items.size(); ++i) cut_items[i].n_parts = (int)(cut_items.size() - first_item);
+          if ((long)takes.size() * Hkv > most) return false;
         }
         return true;
+      };
+      // of those: f(pages, first page in `visit`, stream) for every row block's items
+      auto each_take = [&](auto f) {
+        size_t i = 0;
+        for (size_t s = 0; s < streams.size(); s += Hkv)
+          for (int at = 0; at < streams[s].n_pages; at += takes[i++]) f(takes[i], streams[s].page0 + at, streams[s]);
       };
       long tiles = 0;
       int longest_stream = 0;
@@ -801,6 +805,12 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
         tiles += (st.n_pages + tp - 1) / tp;
         longest_stream = std::max(longest_stream, (st.n_pages + tp - 1) / tp);
       }
+      // items of T tiles, which no wait makes fewer
+      auto least_items = [&](int T) {
+        long n = 0;
+        for (size_t s = 0; s < streams.size(); s += Hkv) n += (streams[s].n_pages + T * tp - 1) / (T * tp);
+        return n * Hkv;
+      };
       int longest = 0;                               // of the cut by pages
       for (int c = 0; !like && c < n_ctas; ++c) {
         int n = 0;
@@ -809,24 +819,29 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
       }
       const int several = (int)p->items.size() > n_ctas && longest <= 4 ? 1 : 0;
       // new rows that come to a CTA, and whether some CTA would have more than it writes itself
-      auto rows_of = [&](const DeviceItem& it) {
+      auto rows_of = [&](int from, int n_pages) {
         int n = 0;
-        for (auto e = std::lower_bound(fresh.begin(), fresh.end(), it.page0); e != fresh.end() && *e < it.page0 + it.n_pages; ++e) n += (visit[*e].y >> 8) & 31;
+        for (auto e = std::lower_bound(fresh.begin(), fresh.end(), from); e != fresh.end() && *e < from + n_pages; ++e) n += (visit[*e].y >> 8) & 31;
         return n;
       };
-      auto many_rows = [&]() { return std::any_of(cut_items.begin(), cut_items.end(), [&](const DeviceItem& it) { return rows_of(it) > kMostFusedRows; }); };
+      auto many_rows = [&]() {
+        bool many = false;
+        each_take([&](int take, int from, const Stream&) { many |= rows_of(from, take) > kMostFusedRows; });
+        return many;
+      };
       auto many_rows_by_pages = [&]() {
         for (int c = 0; c < n_ctas; ++c) {
           int n = 0;
-          for (int i = cta_item0[c]; i < cta_item0[c + 1]; ++i) n += rows_of(p->items[i]);
+          for (int i = cta_item0[c]; i < cta_item0[c + 1]; ++i) n += rows_of(p->items[i].page0, p->items[i].n_pages);
           if (n > kMostFusedRows) return true;
         }
         return false;
       };
-      auto records_of = [](const std::vector<DeviceItem>& items) { long n = 0; for (const DeviceItem& it : items) n += it.n_q_tok; return n; };
       // an update has the room of the plan that it updates, and its launches
       auto fits_plan = [&]() {
-        return cut_items.size() <= like->layout.cap_items && records_of(cut_items) <= (long)like->layout.cap_partials &&
+        long records = 0;
+        each_take([&](int, int, const Stream& st) { records += (long)st.n_tok * Hkv; });
+        return takes.size() * Hkv <= like->layout.cap_items && records <= (long)like->layout.cap_partials &&
                !(like->fuse_append && like->patch_tiles && many_rows());
       };
       bool done = false;
@@ -835,11 +850,11 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
       // (an update's streams have an item each at the latest with as many tiles as the longest has)
       const int last = like ? std::max(T, longest_stream) : longest + several - 1;
       for (; !done && T <= last; ++T)
-        for (int w = p->patch_tiles ? 0 : kWaitKeys; !done && w >= 0; w -= kTileCost / 2) done = pack(T, w) && (!like || fits_plan());
+        for (int w = least_items(T) > most ? -1 : p->patch_tiles ? 0 : kWaitKeys; !done && w >= 0; w -= kTileCost / 2) done = pack(T, w) && (!like || fits_plan());
       if (done && !like) {
         int now = 0;
-        for (const DeviceItem& it : cut_items) now = std::max(now, (it.n_pages + tp - 1) / tp);
-        done = now < longest || 10 * cut_items.size() >= 9 * (size_t)n_ctas;
+        for (int take : takes) now = std::max(now, (take + tp - 1) / tp);
+        done = now < longest || 10 * takes.size() * Hkv >= 9 * (size_t)n_ctas;
       }
       // not where a CTA gets more new rows than it writes itself and none has them by pages: such a step would take a
       // launch more.  Nor, if the plan is to be updated, the other way round: updates have to keep the plan's launches.
@@ -847,20 +862,39 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
         const bool by_tiles = many_rows();
         if (by_tiles || tune.updatable) done = by_tiles == many_rows_by_pages();
       }
-      if (done && tune.updatable && !like) { p->room_items = p->items.size(); p->room_partials = records_of(p->items); }
+      if (done && tune.updatable && !like) {
+        p->room_items = p->items.size();
+        for (const DeviceItem& it : p->items) p->room_partials += it.n_q_tok;
+      }
       if (!done && like) {                             // an update that no cut by tiles fits is cut by pages
         const double waits = cut(0.0);
         if (waits > 0.0) cut(waits);
       }
       if (done) {
         p->tile_cut = T - 1;
-        p->items.swap(cut_items);
+        p->items.clear();
+        size_t i0 = 0;
+        for (size_t s = 0; s < streams.size(); s += Hkv) {
+          size_t i1 = i0;
+          for (int h = 0; h < Hkv; ++h) {
+            const Stream& st = streams[s + h];
+            int at = 0;
+            for (i1 = i0; at < st.n_pages; at += takes[i1++]) {
+              DeviceItem it;
+              it.q_tok0 = st.tok0; it.n_q_tok = st.n_tok; it.kv_head = st.head; it.page0 = st.page0 + at; it.n_pages = takes[i1]; it.key0 = at * ps;
+              it.part_slot = (int)(i1 - i0); it.request = st.request; it.row_block = st.row_block; it.n_parts = 0;
+              p->items.push_back(it);
+            }
+            const int parts = (int)(i1 - i0);
+            for (size_t i = p->items.size() - parts; i < p->items.size(); ++i) p->items[i].n_parts = parts;
+            for (int i = 0; i < st.n_tok; ++i) n_parts[(size_t)(st.tok0 + i) * Hkv + st.head] = parts;
+          }
+          i0 = i1;
+        }
         // (a plan to be updated in place has a CTA to spare for every stream, whose number of tiles may grow)
         if (!like) n_ctas = tune.updatable ? (int)std::min<long>(p->sm_count, std::max<long>((long)p->items.size(), base_ctas + (long)streams.size())) : (int)p->items.size();
         cta_item0.assign(n_ctas + 1, (int)p->items.size());
         for (int c = 0; c < (int)p->items.size(); ++c) cta_item0[c] = c;
-        for (const DeviceItem& it : p->items)
-          for (int i = 0; i < it.n_q_tok; ++i) n_parts[(size_t)(it.q_tok0 + i) * Hkv + it.kv_head] = it.n_parts;
       }
     }
   }
