@@ -958,7 +958,9 @@ static int plan_create_impl(const aspd_shape_t* shape, const aspd_request_t* req
   // more than the combine launch costs, whose blocks are resident and waiting when the pass ends.
   p->single_launch = (kernel == ASPD_KERNEL_MMA && !deal_streams && !p->dec && tune.combine == ASPD_COMBINE_FUSED && max_tok <= 16) ? 1 : 0;   // 16: an item's tokens in the merge queue
   for (size_t i = 0; i < n_parts.size(); ++i) part_base[i + 1] = part_base[i] + n_parts[i];
-  for (int n : n_parts) p->max_parts = std::max(p->max_parts, n);
+  int max_parts = 0;                               // (not the plan's own in the loop, where it would be stored and read again every time)
+  for (int n : n_parts) max_parts = std::max(max_parts, n);
+  p->max_parts = max_parts;
   p->n_items = (int)p->items.size();
   p->n_partials = part_base[n_parts.size()];
   p->kv_tokens_read = kv_tokens;
