@@ -14,9 +14,9 @@
 // The 128 accumulator lanes are used as R x KS: the query rows (padded to R = 32 or 64) are
 // replicated KS = 128 / R times in the A operand, and softmax thread (j, r) handles row r over
 // the j-th key sub-range of the tile only, so all 128 threads share the exponentials.  The KS
-// threads of a row take their exponentials against one reference (0 at an item's start, moved only when a sum leaves
-// 2^-60 .. 2^40, see softmax_item) and write their P values into the SAME row r of the P tile, so the second MMA sums over all
-// keys by itself and rows >= R of its output are simply ignored.
+// threads of a row take their exponentials against one reference (the maximum of the item's first tile, moved only when
+// a sum leaves 2^-60 .. 2^40, see softmax_item) and write their P values into the SAME row r of the P tile, so the second
+// MMA sums over all keys by itself and rows >= R of its output are simply ignored.
 //
 // Warp roles: 0-7 softmax (TMEM lane quadrant = warp % 4; warps w and w + 4 share the rows of a
 // quadrant and take half of the columns each), 8 and 11 bulk-copy producers (K and V), 9 MMA

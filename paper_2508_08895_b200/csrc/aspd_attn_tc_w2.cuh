@@ -20,11 +20,12 @@
 //
 // Bound by the softmax groups' passes (about 1 000-1 200 cycles for 64 scores a row beside the other group's, 512 of
 // them the special-function unit's) and, in long runs, by the power cap.  Whole branches of 32 requests, 28 layers:
-// 25.2 -> 22.6 ms a pass (at 1 720 and 1 655 MHz under the cap); of four requests, below the cap, 1 605 -> 1 197 us.
+// 25.2 -> 22.2 ms a pass under the cap (24.9 -> 23.8 on a box that held less clock); of four requests, below the cap,
+// 1 605 -> 1 197 us.
 // What made the difference to four issuer warps and 512 threads of 128 registers: a group rotates its next query
 // tile itself right after its last P of an item, all loads at once (four warps that issued MMAs as well took 16 000
 // cycles from an item's last P to the next item's first scores, thirteen times a CTA), and scores run right behind the
-// P.V before them without a word in between.  Measured and not taken, same workload: scores of a whole tile in one
+// P.V before them without a word in between (see the issuers).  Measured and not taken, same workload: scores of a whole tile in one
 // MMA (26.2 ms: nothing for the tensor pipe to do while a group is in its passes), a quarter of the exponentials as a
 // polynomial on the FMA pipe (22.9; it takes power, and is less precise), the next half's scores asked for before P
 // is stored (24.1).
@@ -32,7 +33,7 @@
 
 namespace {      // included inside namespace aspd
 
-constexpr int kThreadsW2 = 384;               // 168 registers a thread: the exponent pass and the query preparation fit without spills
+constexpr int kThreadsW2 = 384;               // 168 registers a thread; 44 bytes are spilled
 constexpr int W2_KPROD = 8, W2_VPROD = 9, W2_ISSUE = 10;
 constexpr uint32_t W2_OFF_K = 0, W2_OFF_V = 2 * kTileBytes, W2_OFF_Q = 4 * kTileBytes, W2_OFF_OUT = 6 * kTileBytes,
                    W2_OFF_MISC = 7 * kTileBytes;
@@ -413,8 +414,10 @@ __global__ void __launch_bounds__(kThreadsW2, 1) attn_tc_w2_kernel(Ctx c) {
   } else {
     // ================================ MMA issuers (warp 10: group 0, warp 11: group 1) ================================
     // One warp per group, one cursor, operations in the order the operands come: the P.V of a half as soon as its P
-    // is there, the next scores right behind the P.V that frees their columns.  MMAs of one issuer run in the order
-    // they are issued, so scores that overwrite P need no word that the P.V has read it.  All lanes wait
+    // is there, the next scores right behind the P.V that frees their columns.  Scores that overwrite P have no word that
+    // the P.V has read it: they rest on the tensor pipe's taking the MMAs of one thread in the order that it issues them.
+    // PTX names that order for MMAs of one shape into one accumulator; for these two, which differ in both, it is how the
+    // pipe works, and what attention kernels with P over its scores commonly rest on.  All lanes wait
     // (suspending), lane 0 issues: a warp that diverges around a wait, or polls, spends more cycles on asking
     // than the operations take.
     const int grp = warp - W2_ISSUE;

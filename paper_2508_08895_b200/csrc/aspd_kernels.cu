@@ -432,7 +432,7 @@ __device__ __forceinline__ void generic_item(const PlanDevice& pd, const DeviceI
 
 // The step's new rows in pages that THIS CTA reads (fused step), K rotated with the plan's sines and cosines, V as is.
 // CTAs that read the same page write identical bytes.  A thread takes a chunk pair of K and of V, as the append kernel's do.
-// One launch less a step: three branches over 256 tokens (one layer, 4 heads of 64, a plan per step) 29.5 -> 26.4 us, two requests of
+// One launch less a step: three branches over 256 tokens (one layer, 4 heads of 64, a plan per step) 29.7 -> 27.5 us, two requests of
 // 0.4 k tokens (four layers, 8 heads of 128) 57 -> 49.5.
 template <typename T, int D>
 __device__ __forceinline__ void generic_append(const PlanDevice& pd, const T* __restrict__ k_new, const T* __restrict__ v_new, char* k_pool, char* v_pool,
@@ -492,8 +492,8 @@ __global__ void __launch_bounds__(kGenThreads, 2) attn_generic_kernel(PlanDevice
 
 // ------------------------------------------------------------------------------ combine
 // One warp per (new token, query head): merge the partial records of (token, KV head) by
-// log-sum-exp in one pass with a running maximum.  Where the records lie is plan data and is
-// read before the dependency wait.
+// log-sum-exp, up to 64 of them against one maximum (combine_row).  Where the records lie is plan
+// data and is read before the dependency wait.
 // FLAT: the rows of all tokens are numbered through, four to a block; otherwise a token's heads have blocks of their own, a
 // grid of (tokens, heads / 4).  FLAT where four does not divide the heads: every fourth block of 14 heads had two idle
 // warps, and eight requests' 152 blocks did not fit the chip at a time, which 133 do (24 layers 356 and 344 us).  Not
