@@ -417,7 +417,8 @@ __global__ void __launch_bounds__(kThreadsW2, 1) attn_tc_w2_kernel(Ctx c) {
     // is there, the next scores right behind the P.V that frees their columns.  Scores that overwrite P have no word that
     // the P.V has read it: they rest on the tensor pipe's taking the MMAs of one thread in the order that it issues them.
     // PTX names that order for MMAs of one shape into one accumulator; for these two, which differ in both, it is how the
-    // pipe works, and what attention kernels with P over its scores commonly rest on.  All lanes wait
+    // pipe works, and what attention kernels with P over its scores commonly rest on.  (A wait for the P.V there: 24.6
+    // instead of 22.4 ms a pass.)  All lanes wait
     // (suspending), lane 0 issues: a warp that diverges around a wait, or polls, spends more cycles on asking
     // than the operations take.
     const int grp = warp - W2_ISSUE;
